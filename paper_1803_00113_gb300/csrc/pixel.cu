@@ -35,14 +35,19 @@ constexpr float kHalfLog2e = 0.72134752044448170368f;   // log2(e) / 2
 //                                   | per PSF component k: galaxy pairs, then singles
 //   derivs layout: header | origins | star {A, lw | P, 0}
 //                                   | per PSF component k: galaxy pairs, then singles
-// A galaxy component has 16 values {A, lw | -P11, -P12, -P22, tau |
-// -2 P12, -2 P11^2, -2 P22^2, -2 P12^2 | -4 P12, -2 P12 P11, -2 P12 P22, 0}:
-// the signs are chosen so that no formula below negates an operand.  The components of PSF
+// (with the pairs' skip radii between origins and stars, see stage_skip).
+// A galaxy component has 20 values {A, lw | -P11, -P12, -P22, tau |
+// -2 P12, -2 P11^2, -2 P22^2, -2 P12^2 | -4 P12, -2 P12 P11, -2 P12 P22,
+// -2 P11 | -2 P22, -4 P11, -4 P22, 0}: the signs are chosen so that no
+// formula below negates an operand.  An FP32 instruction with three distinct
+// register operands issues every 3 cycles per 64 lanes here (1.55 per 32),
+// with two every 2, so sums with a constant multiple of P take it staged, as
+// an addition, rather than as an FMA with 2 or 4.  The components of PSF
 // component k come in pairs (exponential j, de Vaucouleurs j) for
 // j < min(n_exp, n_dev), their values interleaved (exponential in the even
 // slots), so that one packed two-wide FP32 instruction (ffma2, which rounds
 // each half as fmaf does) evaluates both; the components without a partner
-// follow with their 16 values in a row.
+// follow with their 20 values in a row.
 // A = -log2(e)/2 (P11, 2 P12, P22) are the coefficients of the exponent's
 // quadratic form: log2 phi = lw + A11 dx^2 + A12 dx dy + A22 dy^2.  Every
 // component convolved with PSF component k has that component's mean (the
@@ -53,8 +58,9 @@ constexpr float kHalfLog2e = 0.72134752044448170368f;   // log2(e) / 2
 constexpr int kOrgF = 8;                                   // (mx, my) per k, padded
 constexpr int kValF = 4;
 constexpr int kStarF = 8;
-constexpr int kGalF = 16;
-constexpr int kCompBase = kHdr + kOrgF;
+constexpr int kGalF = 20;
+constexpr int kSkipBase = kHdr + kOrgF;                    // skip radii, kMaxProf per k
+constexpr int kCompBase = kSkipBase + kPsf * kMaxProf;
 constexpr int kValRecF = kCompBase + kMaxComp * kValF;
 constexpr int kDerivRecF = kCompBase + kPsf * kStarF + kPsf * 2 * kMaxProf * kGalF;
 static_assert(2 * kPsf <= kOrgF && kValRecF % 4 == 0 && kDerivRecF % 4 == 0, "staged layout");
@@ -117,7 +123,8 @@ __device__ __forceinline__ void stage_record(float* __restrict__ dst, const floa
       const int j = dev ? jj - ne : jj;
       const float vals[kGalF] = {q.x, q.y, q.z, q.w, -p11, -p12, -p22, b.z,
                                  -2.f * p12, -2.f * p11 * p11, -2.f * p22 * p22, -2.f * p12 * p12,
-                                 -4.f * p12, (-2.f * p12) * p11, (-2.f * p12) * p22, 0.f};
+                                 -4.f * p12, (-2.f * p12) * p11, (-2.f * p12) * p22, -2.f * p11,
+                                 -2.f * p22, -4.f * p11, -4.f * p22, 0.f};
       float* base = dst + kCompBase + kPsf * kStarF + k * per * kGalF;
       if (j < nb) {
         float* o = base + j * 2 * kGalF + (dev ? 1 : 0);
@@ -132,6 +139,50 @@ __device__ __forceinline__ void stage_record(float* __restrict__ dst, const floa
       }
     }
   }
+}
+
+// Skip radii of the staged galaxy pairs, after stage_record and a warp
+// barrier (kPairF floats a pair, its first eight {A11, A12, A22, lw} in both
+// layouts): for d^2 beyond rec[kSkipBase + k kMaxProf + j] both halves of pair
+// j have log2 phi <= lw - lambda_min(-A) d^2 < -128, where exp2 (which
+// flushes denormals here) returns zero, so the pair would add exact zeros.
+// 0.1 % on the radius and two powers of two of slack cover the rounding of
+// the bound and of the exponent; an ill-conditioned or non-finite form is
+// never skipped.
+template <int kPairF>
+__device__ __forceinline__ void stage_skip(float* __restrict__ rec, int base, int ne, int nd,
+                                           int lane) {
+  const int nb = ne < nd ? ne : nd;
+  if (lane < kPsf * nb) {
+    const int k = lane / nb, j = lane - k * nb;
+    const float* c = rec + base + k * (ne + nd) * (kPairF / 2) + j * kPairF;
+    float r = 0.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float a = -c[h], b = -0.5f * c[2 + h], d = -c[4 + h], lw = c[6 + h];
+      const float det = fmaf(a, d, -b * b);
+      const float lmax = 0.5f * (a + d + sqrtf(fmaf(a - d, a - d, 4.f * b * b)));
+      const bool ok = a > 0.f && d > 0.f && det > 1e-3f * a * d && lw < INFINITY;
+      r = fmaxf(r, ok ? 1.001f * fmaxf(lw + 128.f, 0.f) * (lmax / det) : INFINITY);
+    }
+    rec[kSkipBase + k * kMaxProf + j] = r;
+  }
+  __syncwarp();
+}
+
+// First pair of PSF component k that a pass over pixels with smallest squared
+// offset d2 (of the whole warp) has to evaluate.
+__device__ __forceinline__ int first_pair(const float* __restrict__ rec, int k, int nb, float d2,
+                                          int lane) {
+  const float r = rec[kSkipBase + k * kMaxProf + (lane & (kMaxProf - 1))];
+  const unsigned m = __ballot_sync(0xffffffffu, lane < nb && !(d2 > r));
+  return m ? __ffs(m) - 1 : nb;
+}
+
+// Smallest of the warp's squared offsets (not negative, so their bits order
+// as they do; NaN orders last).
+__device__ __forceinline__ float warp_min_d2(float d2) {
+  return __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(d2)));
 }
 
 // A pixel's offset from PSF component k's mean, and its products.
@@ -218,7 +269,7 @@ struct GalSums {
   float t4a, t4b, t4c, t4d, t4e;       // 1111, 1112, 1122, 1222, 2222
 };
 
-// One galaxy component of the derivs layout (16 staged values).
+// One galaxy component of the derivs layout (its first 16 values).
 __device__ __forceinline__ void gal_accumulate(const float* __restrict__ c, const Offset& o,
                                                GalSums& g) {
   const float4 q = *reinterpret_cast<const float4*>(c);
@@ -284,7 +335,9 @@ struct GalSums2 {
   float2 t4a, t4b, t4c, t4d, t4e;
 };
 
-// gal_accumulate on a staged pair (32 floats, exponential in the even slots).
+// gal_accumulate on a staged pair (40 floats, exponential in the even slots).
+// Accumulations sharing phi, pt or pt2 stand together: 4.49 ms against 4.64
+// in the order of the formulas (derivatives of 1,000 blended sources).
 __device__ __forceinline__ void gal_accumulate2(const float* __restrict__ c, const Offset2& o,
                                                 GalSums2& g) {
   const float4 qa = *reinterpret_cast<const float4*>(c);
@@ -294,7 +347,11 @@ __device__ __forceinline__ void gal_accumulate2(const float* __restrict__ c, con
   const float4 ha = *reinterpret_cast<const float4*>(c + 16);
   const float4 hb = *reinterpret_cast<const float4*>(c + 20);
   const float4 hq = *reinterpret_cast<const float4*>(c + 24);
-  const float2 c4d = *reinterpret_cast<const float2*>(c + 28);
+  const float4 hr = *reinterpret_cast<const float4*>(c + 28);
+  const float4 hs4 = *reinterpret_cast<const float4*>(c + 32);
+  const float2 n4P22 = *reinterpret_cast<const float2*>(c + 36);
+  const float2 c4d = make_float2(hr.x, hr.y), n2P11 = make_float2(hr.z, hr.w);
+  const float2 n2P22 = make_float2(hs4.x, hs4.y), n4P11 = make_float2(hs4.z, hs4.w);
   const float2 m4P12 = make_float2(hq.x, hq.y), c4b = make_float2(hq.z, hq.w);
   const float2 A11 = make_float2(qa.x, qa.y), A12 = make_float2(qa.z, qa.w);
   const float2 A22 = make_float2(qb.x, qb.y), lw = make_float2(qb.z, qb.w);
@@ -302,7 +359,6 @@ __device__ __forceinline__ void gal_accumulate2(const float* __restrict__ c, con
   const float2 nP22 = make_float2(pb.x, pb.y), tau = make_float2(pb.z, pb.w);
   const float2 m2P12 = make_float2(ha.x, ha.y), c4a = make_float2(ha.z, ha.w);
   const float2 c4e = make_float2(hb.x, hb.y), c4c = make_float2(hb.z, hb.w);
-  const float2 two = f2(2.f), four = f2(4.f);
   const float2 z1 = fma2(nP11, o.dx, mul2(nP12, o.dy));
   const float2 z2 = fma2(nP12, o.dx, mul2(nP22, o.dy));
   const float2 arg = fma2(A11, o.xx, fma2(A12, o.xy, fma2(A22, o.yy, lw)));
@@ -310,28 +366,38 @@ __device__ __forceinline__ void gal_accumulate2(const float* __restrict__ c, con
   const float2 h11 = fma2(z1, z1, nP11);
   const float2 h12 = fma2(z1, z2, nP12);
   const float2 h22 = fma2(z2, z2, nP22);
-  const float2 pt = mul2(phi, tau);
-  const float2 pt2 = mul2(pt, tau);
-  g.s0 = add2(g.s0, phi);
+  const float2 pt = mul2(tau, phi);
+  g.s0 = add2(phi, g.s0);
   g.s1x = fma2(phi, z1, g.s1x);
   g.s1y = fma2(phi, z2, g.s1y);
   g.s2xx = fma2(phi, h11, g.s2xx);
   g.s2xy = fma2(phi, h12, g.s2xy);
   g.s2yy = fma2(phi, h22, g.s2yy);
+  const float2 pt2 = mul2(tau, pt);
   g.t2xx = fma2(pt, h11, g.t2xx);
   g.t2xy = fma2(pt, h12, g.t2xy);
   g.t2yy = fma2(pt, h22, g.t2yy);
-  const float2 a1 = fma2(two, nP11, h11), a2 = fma2(two, nP22, h22);
   const float2 pz1 = mul2(pt, z1), pz2 = mul2(pt, z2);
-  g.t3a = fma2(pz1, a1, g.t3a);
-  g.t3b = fma2(pz2, h11, fma2(m2P12, pz1, g.t3b));
-  g.t3c = fma2(pz1, h22, fma2(m2P12, pz2, g.t3c));
+  const float2 a1 = add2(h11, n2P11), a2 = add2(h22, n2P22);
+  g.t3b = fma2(m2P12, pz1, g.t3b);
+  g.t3c = fma2(m2P12, pz2, g.t3c);
+  const float2 ub = fma2(m2P12, h11, c4b);
+  const float2 ud = fma2(m2P12, h22, c4d);
+  g.t3b = fma2(pz2, h11, g.t3b);
   g.t3d = fma2(pz2, a2, g.t3d);
-  g.t4a = fma2(pt2, fma2(h11, fma2(four, nP11, h11), c4a), g.t4a);
-  g.t4b = fma2(pt2, fma2(h12, a1, fma2(m2P12, h11, c4b)), g.t4b);
-  g.t4c = fma2(pt2, fma2(h11, h22, fma2(h12, m4P12, c4c)), g.t4c);
-  g.t4d = fma2(pt2, fma2(h12, a2, fma2(m2P12, h22, c4d)), g.t4d);
-  g.t4e = fma2(pt2, fma2(h22, fma2(four, nP22, h22), c4e), g.t4e);
+  g.t3a = fma2(pz1, a1, g.t3a);
+  g.t3c = fma2(pz1, h22, g.t3c);
+  const float2 va = fma2(h11, add2(h11, n4P11), c4a);
+  const float2 uc = fma2(h12, m4P12, c4c);
+  const float2 vc = fma2(h11, h22, uc);
+  const float2 ve = fma2(h22, add2(h22, n4P22), c4e);
+  const float2 vb = fma2(h12, a1, ub);
+  const float2 vd = fma2(h12, a2, ud);
+  g.t4a = fma2(pt2, va, g.t4a);
+  g.t4b = fma2(pt2, vb, g.t4b);
+  g.t4c = fma2(pt2, vc, g.t4c);
+  g.t4d = fma2(pt2, vd, g.t4d);
+  g.t4e = fma2(pt2, ve, g.t4e);
 }
 
 // A component without a partner: gal_accumulate into half L of g.
@@ -466,12 +532,18 @@ struct HessAcc {
   }
 };
 
-// One pixel: render with derivatives and accumulate value, gradient, Hessian.
-__device__ __forceinline__ void pixel_derivs(const float* __restrict__ rec, int ne, int nd,
-                                             float px, float py, float x, float2 bg,
-                                             float* __restrict__ acc, const HessAcc& hs) {
-  // ---- star: value, d mu, d mu d mu
-  float F1 = 0.f, sx = 0.f, sy = 0.f, sxx = 0.f, sxy = 0.f, syy = 0.f;
+// The star sums of a pixel: value, d mu, d mu d mu.
+struct StarSums {
+  float F1, sx, sy, sxx, sxy, syy;
+};
+
+// A pixel's star and galaxy sums; with kSkip for a whole warp of pixels at
+// once, leaving out the pairs that are zero at all of them.
+template <bool kSkip>
+__device__ __forceinline__ void pixel_sums(const float* __restrict__ rec, int ne, int nd,
+                                           float px, float py, int lane, StarSums& st,
+                                           GalSums2& g2) {
+  st = {};
 #pragma unroll
   for (int k = 0; k < kPsf; ++k) {
     const Offset o = make_offset(pixel_delta(rec, k, px, py));
@@ -481,15 +553,15 @@ __device__ __forceinline__ void pixel_derivs(const float* __restrict__ rec, int 
     const float y1 = fmaf(pp.x, o.dx, pp.y * o.dy);
     const float y2 = fmaf(pp.y, o.dx, pp.z * o.dy);
     const float phi = gauss_density(q, o);
-    F1 += phi;
-    sx = fmaf(phi, y1, sx);
-    sy = fmaf(phi, y2, sy);
-    sxx = fmaf(phi, fmaf(y1, y1, -pp.x), sxx);
-    sxy = fmaf(phi, fmaf(y1, y2, -pp.y), sxy);
-    syy = fmaf(phi, fmaf(y2, y2, -pp.z), syy);
+    st.F1 += phi;
+    st.sx = fmaf(phi, y1, st.sx);
+    st.sy = fmaf(phi, y2, st.sy);
+    st.sxx = fmaf(phi, fmaf(y1, y1, -pp.x), st.sxx);
+    st.sxy = fmaf(phi, fmaf(y1, y2, -pp.y), st.sxy);
+    st.syy = fmaf(phi, fmaf(y2, y2, -pp.z), st.syy);
   }
-  // ---- galaxy: exponential and de Vaucouleurs sums, evaluated in pairs
-  GalSums2 g2 = {};
+  // galaxy: exponential and de Vaucouleurs sums, evaluated in pairs
+  g2 = {};
   const int per = ne + nd;
   const int nb = ne < nd ? ne : nd;
   // kept rolled: three copies of this loop cost more in instruction fetch
@@ -499,19 +571,28 @@ __device__ __forceinline__ void pixel_derivs(const float* __restrict__ rec, int 
     const float* base = rec + kCompBase + kPsf * kStarF + k * per * kGalF;
     const Offset o = make_offset(pixel_delta(rec, k, px, py));
     const Offset2 o2 = dup_offset(o);
-    if (nb == kMaxProf) {
+    int j = kSkip ? first_pair(rec, k, nb, warp_min_d2(o.xx + o.yy), lane) : 0;
+    if (nb == kMaxProf && j < 2) {
       // the usual eight pairs, unrolled: independent pairs interleave (the
       // loop over PSF components stays rolled: unrolling both measured
       // slower, from instruction fetch)
 #pragma unroll
-      for (int j = 0; j < kMaxProf; ++j) gal_accumulate2(base + j * 2 * kGalF, o2, g2);
+      for (int jj = 0; jj < kMaxProf; ++jj) gal_accumulate2(base + jj * 2 * kGalF, o2, g2);
     } else {
-      for (int j = 0; j < nb; ++j) gal_accumulate2(base + j * 2 * kGalF, o2, g2);
+#pragma unroll 2
+      for (; j < nb; ++j) gal_accumulate2(base + j * 2 * kGalF, o2, g2);
     }
     const float* single = base + nb * 2 * kGalF;
     for (int j = nb; j < ne; ++j, single += kGalF) gal_single<0>(single, o, g2);
     for (int j = nb; j < nd; ++j, single += kGalF) gal_single<1>(single, o, g2);
   }
+}
+
+// One pixel with its sums: accumulates value, gradient and Hessian.
+__device__ __forceinline__ void pixel_derivs(const float* __restrict__ rec, const StarSums& st,
+                                             const GalSums2& g2, float x, float2 bg,
+                                             float* __restrict__ acc, const HessAcc& hs) {
+  const float F1 = st.F1, sx = st.sx, sy = st.sy, sxx = st.sxx, sxy = st.sxy, syy = st.syy;
   GalSums ge, gd;
 #define SPLIT(f) ge.f = g2.f.x; gd.f = g2.f.y;
 #define FLIP(f) ge.f = -g2.f.x; gd.f = -g2.f.y;        // odd orders: summed with -y
@@ -839,7 +920,7 @@ __device__ __forceinline__ void reduce_tile(float* __restrict__ tile, float* __r
 // fed.  (Forming the background here instead of in background_kernel was
 // measured slower: the cached-moment loads inside the pixel loop stall 16
 // warps more than a separate kernel's many warps.)
-template <bool kQueue>
+template <bool kQueue, bool kSkip>
 __global__ void __launch_bounds__(128, 4) derivs_kernel(PlanView v, int ne, int nd) {
   extern __shared__ float4 smem4[];
   float* smem = reinterpret_cast<float*>(smem4);
@@ -861,16 +942,26 @@ __global__ void __launch_bounds__(128, 4) derivs_kernel(PlanView v, int ne, int 
 #pragma unroll
     for (int a = 0; a < kHessAcc; ++a) tile[a * kHessRow + lane] = 0.f;
     __syncwarp();
+    if (kSkip) stage_skip<2 * kGalF>(rec, kCompBase + kPsf * kStarF, ne, nd, lane);
     float acc[kGradAcc];
 #pragma unroll
     for (int a = 0; a < kGradAcc; ++a) acc[a] = 0.f;
     const int end = item.start + item.count;
     PixelWalk pw(item.start + lane, pi.w);
-    for (int q = item.start + lane; q < end; q += 32, pw.next(pi.w)) {
-      const int qy = pw.qy, qx = pw.qx;
+    // with kSkip the whole warp takes every pass, and lanes past the end
+    // repeat lane 0's pixel
+    for (int q = item.start + lane; (kSkip ? q - lane : q) < end; q += 32, pw.next(pi.w)) {
+      int qy = pw.qy, qx = pw.qx;
+      if (kSkip && q - lane + 32 > end) {
+        const int y0 = __shfl_sync(0xffffffffu, qy, 0), x0 = __shfl_sync(0xffffffffu, qx, 0);
+        if (q >= end) qy = y0, qx = x0;
+      }
       const float x = __ldg(v.pixels + pi.pix_base + (int64_t)qy * pi.stride + qx);
-      const float2 bg = v.bg[pi.bg_base + q];
-      pixel_derivs(rec, ne, nd, (float)qx, (float)qy, x, bg, acc, hs);
+      const float2 bg = v.bg[pi.bg_base + (!kSkip || q < end ? q : q - lane)];
+      StarSums st;
+      GalSums2 g2;
+      pixel_sums<kSkip>(rec, ne, nd, (float)qx, (float)qy, lane, st, g2);
+      if (!kSkip || q < end) pixel_derivs(rec, st, g2, x, bg, acc, hs);
     }
     __syncwarp();
     reduce_tile(tile, acc, v.partials + (size_t)it * kAcc, lane);
@@ -1344,15 +1435,19 @@ constexpr int kWpb = 4;   // warps per block of the pixel kernels
 // The derivative kernel's dynamic shared memory is close to the default 48 KB
 // limit: raise the limit to what it uses.
 static DeviceOnce g_derivs_attr;
+using DerivsKernel = void (*)(PlanView, int, int);
+static constexpr DerivsKernel kDerivsKernels[2][2] = {   // [queue][skip]
+    {derivs_kernel<false, false>, derivs_kernel<false, true>},
+    {derivs_kernel<true, false>, derivs_kernel<true, true>}};
 static cudaError_t derivs_attr() {
   return g_derivs_attr.run([] {
-    cudaError_t e = cudaFuncSetAttribute(derivs_kernel<false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem_bytes_derivs(kWpb));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(derivs_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem_bytes_derivs(kWpb));
-    return e;
+    for (int k = 0; k < 4; ++k) {
+      cudaError_t e = cudaFuncSetAttribute(kDerivsKernels[k / 2][k % 2],
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)smem_bytes_derivs(kWpb));
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
   });
 }
 
@@ -1372,9 +1467,9 @@ cudaError_t init_pixel_occupancy() {
     const size_t sm = smem_bytes(kWpb);
     int occ[kOccKinds] = {};
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &occ[kOccDerivs], derivs_kernel<false>, kWpb * 32, smem_bytes_derivs(kWpb));
+        &occ[kOccDerivs], kDerivsKernels[0][0], kWpb * 32, smem_bytes_derivs(kWpb));
     if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[kOccDerivsQ], derivs_kernel<true>,
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[kOccDerivsQ], kDerivsKernels[1][0],
                                                         kWpb * 32, smem_bytes_derivs(kWpb));
     if (e == cudaSuccess)
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[kOccGrad], grad_kernel<false>,
@@ -1435,15 +1530,25 @@ static bool use_queue(const PlanView& v, int blocks) {
   return v.work_ctr && v.n_items >= kQueueItemsPerWarp * kWpb * blocks;
 }
 
+// Leaving out vanished pairs pays where pixels lie far from their source and
+// the launch is bound by arithmetic: a mean patch of 45 x 45 pixels or more,
+// and more items than warps on the GPU.  Batched field (2,000 sources, mean
+// patch 2,700 pixels): 8.64 ms against 10.13; 1,200 field sources (mean
+// patch 650): 0.615 against 0.604; one source of 101 x 101 pixels, which a
+// few warps work on: 27.4 us against 26.9.
+constexpr int kSkipArea = 2048;
+static bool use_skip(const Launch& L, const PlanView& v) {
+  return v.n_bg >= (int64_t)kSkipArea * v.n_own_pairs && v.n_items > 16 * L.sm_count;
+}
+
 cudaError_t launch_pixels_derivs(const Launch& L, const PlanView& v) {
   if (v.n_items == 0) return cudaSuccess;
   if (cudaError_t e = derivs_attr()) return e;
   const int gq = grid_for(L, v.n_items, kWpb, kOccDerivsQ);
-  if (use_queue(v, gq))
-    derivs_kernel<true><<<gq, kWpb * 32, smem_bytes_derivs(kWpb), L.stream>>>(v, L.n_exp, L.n_dev);
-  else
-    derivs_kernel<false><<<grid_for(L, v.n_items, kWpb, kOccDerivs), kWpb * 32,
-                           smem_bytes_derivs(kWpb), L.stream>>>(v, L.n_exp, L.n_dev);
+  const bool queue = use_queue(v, gq);
+  const int grid = queue ? gq : grid_for(L, v.n_items, kWpb, kOccDerivs);
+  kDerivsKernels[queue][use_skip(L, v)]<<<grid, kWpb * 32, smem_bytes_derivs(kWpb), L.stream>>>(
+      v, L.n_exp, L.n_dev);
   return cudaGetLastError();
 }
 
