@@ -568,8 +568,6 @@ int celeste_plan_create(celeste_ctx* c, const celeste_problem* pr, const int32_t
   v.elbo_rel = dev_alloc<double>(p, n, &err);
   p->rel_trial = dev_alloc<double>(p, n, &err);
   v.rel_trial = p->rel_trial;
-  v.grad = dev_alloc<double>(p, (size_t)n * kTheta, &err);
-  v.hess = dev_alloc<double>(p, (size_t)n * kTheta * kTheta, &err);
   v.active = dev_alloc<uint8_t>(p, n, &err);
   if (err != CELESTE_OK) {
     celeste_plan_destroy(p);

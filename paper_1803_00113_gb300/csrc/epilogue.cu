@@ -5,6 +5,14 @@
 
 namespace celeste {
 
+struct EpiBlock {
+  EpiSmem e;
+  ModelDev::F32 f;
+};
+
+// use_trial: bit 0 evaluates theta_trial; bit 1 (value mode only) asks for
+// the pixel part alone, without the KL (the log-likelihood of the source's
+// point values relative to its absence).
 template <int kMode>
 __global__ void __launch_bounds__(kEpiThreads) epilogue_kernel(PlanView v,
                                                                const ModelDev* __restrict__ model,
@@ -12,8 +20,34 @@ __global__ void __launch_bounds__(kEpiThreads) epilogue_kernel(PlanView v,
                                                                double* grad_out, double* hess_out,
                                                                int use_trial) {
   extern __shared__ double smd[];
-  epilogue_source<kMode>(v, model, *reinterpret_cast<EpiSmem*>(smd), blockIdx.x, elbo, elbo_rel,
-                         grad_out, hess_out, use_trial);
+  EpiBlock& S = *reinterpret_cast<EpiBlock*>(smd);
+  const int j = blockIdx.x, tid = threadIdx.x;
+  if (!v.active[j]) return;
+  const bool trial = (use_trial & 1) != 0, pixel_only = kMode == 0 && (use_trial & 2) != 0;
+  const double* thd =
+      trial ? v.theta_trial + (size_t)j * kTheta : v.theta + (size_t)v.src_ids[j] * kTheta;
+  if (tid < kTheta) S.e.th[tid] = (real)thd[tid];
+  stage_model(S.f, model, tid, kEpiThreads);
+  double rel, full;
+  epilogue_source<kMode>(v, S.f, model->n_color, S.e, j, tid, pixel_only, rel, full);
+  if (tid == 0) {
+    if (elbo) elbo[j] = full;
+    if (elbo_rel) elbo_rel[j] = rel;
+    // a non-finite value at a trial point is a rejected step, not an error
+    if (!isfinite(full) && !trial) set_error(v.err, CELESTE_DERR_NONFINITE);
+  }
+  if (kMode >= 1) {
+    int bad = 0;
+    for (int e = tid; e < kTheta; e += kEpiThreads) {
+      grad_out[(size_t)j * kTheta + e] = (double)S.e.gth[e];
+      bad |= !isfinite(S.e.gth[e]);
+    }
+    for (int e = tid; e < (kMode == 2 ? kTheta * kTheta : 0); e += kEpiThreads) {
+      hess_out[(size_t)j * kTheta * kTheta + e] = (double)S.e.Hth[e];
+      bad |= !isfinite(S.e.Hth[e]);
+    }
+    if (__syncthreads_or(bad) && tid == 0) set_error(v.err, CELESTE_DERR_NONFINITE);
+  }
 }
 
 // The dynamic shared memory limit of each epilogue kernel, once per device.
@@ -22,7 +56,7 @@ static cudaError_t set_smem_attr() {
   static DeviceOnce once;
   return once.run([] {
     return cudaFuncSetAttribute(epilogue_kernel<kMode>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(EpiSmem));
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(EpiBlock));
   });
 }
 
@@ -30,7 +64,7 @@ cudaError_t launch_epilogue(const Launch& L, const PlanView& v, const ModelDev* 
                             double* elbo, double* elbo_rel, double* grad, double* hess) {
   if (v.n == 0) return cudaSuccess;
   if (cudaError_t e = set_smem_attr<2>()) return e;
-  epilogue_kernel<2><<<v.n, kEpiThreads, sizeof(EpiSmem), L.stream>>>(v, model, elbo, elbo_rel, grad,
+  epilogue_kernel<2><<<v.n, kEpiThreads, sizeof(EpiBlock), L.stream>>>(v, model, elbo, elbo_rel, grad,
                                                               hess, 0);
   return cudaGetLastError();
 }
@@ -39,7 +73,7 @@ cudaError_t launch_epilogue_grad(const Launch& L, const PlanView& v, const Model
                                  double* elbo, double* elbo_rel, double* grad) {
   if (v.n == 0) return cudaSuccess;
   if (cudaError_t e = set_smem_attr<1>()) return e;
-  epilogue_kernel<1><<<v.n, kEpiThreads, sizeof(EpiSmem), L.stream>>>(v, model, elbo, elbo_rel, grad,
+  epilogue_kernel<1><<<v.n, kEpiThreads, sizeof(EpiBlock), L.stream>>>(v, model, elbo, elbo_rel, grad,
                                                               nullptr, 0);
   return cudaGetLastError();
 }
@@ -48,7 +82,7 @@ cudaError_t launch_epilogue_value(const Launch& L, const PlanView& v, const Mode
                                   double* elbo, double* elbo_rel, bool use_trial) {
   if (v.n == 0) return cudaSuccess;
   if (cudaError_t e = set_smem_attr<0>()) return e;
-  epilogue_kernel<0><<<v.n, kEpiThreads, sizeof(EpiSmem), L.stream>>>(v, model, elbo, elbo_rel, nullptr,
+  epilogue_kernel<0><<<v.n, kEpiThreads, sizeof(EpiBlock), L.stream>>>(v, model, elbo, elbo_rel, nullptr,
                                                               nullptr, use_trial ? 1 : 0);
   return cudaGetLastError();
 }
@@ -57,7 +91,7 @@ cudaError_t launch_epilogue_loglik(const Launch& L, const PlanView& v, const Mod
                                    double* out) {
   if (v.n == 0) return cudaSuccess;
   if (cudaError_t e = set_smem_attr<0>()) return e;
-  epilogue_kernel<0><<<v.n, kEpiThreads, sizeof(EpiSmem), L.stream>>>(v, model, nullptr, out,
+  epilogue_kernel<0><<<v.n, kEpiThreads, sizeof(EpiBlock), L.stream>>>(v, model, nullptr, out,
                                                                       nullptr, nullptr, 2);
   return cudaGetLastError();
 }
@@ -72,7 +106,7 @@ __global__ void kl_kernel(PlanView v, const ModelDev* __restrict__ model, double
   const int src = v.src_ids[j];
   if (lane < kTheta) S.th[lane] = (real)v.theta[(size_t)src * kTheta + lane];
   __syncwarp();
-  kl_terms<0>(S.th, model, S, lane);
+  kl_terms<0, false>(S.th, model->f, model->n_color, S, lane);
   __syncwarp();
   if (lane == 0) kl_out[src] = (double)S.kls[0];
 }

@@ -21,8 +21,18 @@
 // the pixel kernel, so the chain rule and the KL run in FP32 ("real"), which
 // adds rounding of the same order as its inputs already carry; the value
 // sums (which include the large sky baseline) stay in FP64.  On GB300 an
-// FP64 instruction costs ~64 cycles per SM sub-partition, and this kernel
-// is on the critical path of every colour class.
+// FP64 instruction costs ~65 cycles of an SM sub-partition, whatever the
+// number of its lanes at work or of independent ones around it.
+//
+// Bound: latency.  A source is a block of four warps, on the critical path of
+// every colour class, and each stage is a short chain of loads, shared
+// memory exchanges and barriers.  So the stages that depend on theta alone
+// (KL_s, the Jacobian) run beside the reduction of the tile sums, the sums
+// come to shared memory in asynchronous copies, maps and indices are formed
+// without branches (a divergent 18-way choice of map entries alone took 4k
+// cycles a pair), and every small dense product is spread over all threads.
+// One source with one 41 x 41 patch per band: 27k cycles (53k before) for
+// value, gradient and Hessian; with two 61 x 61 patches per band: 34k (84k).
 #pragma once
 
 #include <math.h>
@@ -39,7 +49,7 @@ static __constant__ signed char kSelE[5][4] = {
 constexpr int kNu = 26;   // 20 flux moments (band b, kind e at 4b+e), u (2), Sigma_s (3), rho
 constexpr int kNuPad = 32;
 constexpr int kKlVals = 8 + 10 + 4;       // per colour component: grad, precision, diag
-constexpr int kKlSums = 64;                // per type: mean grad 8, centred outer 36, prec 10, diag 4
+constexpr int kKlSums = 64;               // per type: mean grad 8, centred outer 36, prec 10, diag 4
 
 static __device__ __forceinline__ real sigm(real t) {
   return t >= 0.f ? 1.f / (1.f + expf(-t)) : expf(t) / (1.f + expf(t));
@@ -51,17 +61,35 @@ static __device__ __forceinline__ real softplus(real t) {
 
 constexpr int kEpiThreads = 128;   // four warps per source
 constexpr int kPairThreads = kEpiThreads - 32;   // warps 1..3: the pixel sums
-constexpr int kPairGroup = 4;                    // pairs reduced together
+constexpr int kPairGroup = 12;                   // pairs reduced between barriers
+constexpr int kTileChunk = 32;                   // tiles copied to shared memory at a time
 
-// Barrier among the kPairThreads threads of warps 1..3 (named barrier 1;
-// warp 0 is busy with the KL terms meanwhile).
+// Barriers among the kPairThreads threads of warps 1..3 (named barrier 1;
+// warp 0 is busy with the KL terms meanwhile) and among warps 1 and 2
+// (named barrier 2).
 static __device__ __forceinline__ void pair_sync() {
   asm volatile("bar.sync 1, %0;" ::"n"(kPairThreads) : "memory");
 }
+static __device__ __forceinline__ void tile_sync() {
+  asm volatile("bar.sync 2, 64;" ::: "memory");
+}
+// Asynchronous copy of 16 bytes to shared memory.
+static __device__ __forceinline__ void copy_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                   (unsigned)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+
+constexpr int kGeoHess = 55;                     // upper triangle over the 10 w
 
 struct EpiSmem {
-  double Wd[kPairGroup][2];        // per pair of a group: value sums (relative, base)
-  float W[kPairGroup][kAcc];       // per pair of a group: the other sums (entries 2..63)
+  float vs[kPairGroup][4];         // per pair of a group: value sums (s, c of relative, base)
+  float W[kPairGroup][kAcc];       // per pair of a group: zero, then the other sums (2..63)
+  float T[kPairGroup][10 * 10];    // per pair of a group: affine map w <- nu (local)
+  alignas(16) float tiles[2][kTileChunk][kAcc];   // tile sums on their way in
+  int band[kPairGroup];
+  real pw[2 * kKlSums];            // colour bound: pi-weighted sums per type
   real th[kNuPad];                 // theta of the source (FP32 copy)
   real gnu[kNuPad];
   real Hnu[kNu * kNu];
@@ -71,11 +99,13 @@ struct EpiSmem {
   real Hth[kTheta * kTheta];
   real DL[20 * kTheta];            // d log kappa_a / d theta
   real D2L[20 * kTheta];           // diagonal second derivatives of log kappa_a
+  real kap[kNuPad];                // kappa_a
   real kw[kNuPad];                 // grad_nu[a] * kappa_a
+  real d2S[27];                    // second derivatives of Sigma_s
   real klc[2 * kMaxColor * kKlVals];   // colour-bound pieces per (type, component)
   real klj[2 * kMaxColor];         // log w_j - K_j
   real kls[8];                     // scalar KL pieces
-  float T[kPairGroup][10 * 10];    // per pair of a group: affine map w <- nu (local)
+  real klt[32];                    // terms of the KL's value and gradient
   double red[2][kEpiThreads / 32]; // per-warp value sums
   double vsum[2];                  // the source's value sums (relative, base)
 };
@@ -85,42 +115,56 @@ struct EpiSmem {
 static __device__ __forceinline__ int nrows(int c) {
   return c == 0 ? 20 : (c <= 20 ? 10 : (c <= 22 ? 1 : (c <= 25 ? 3 : 1)));
 }
-static __device__ __forceinline__ int rowof(int c, int k) {
-  if (c == 0) return k;
-  if (c <= 20) return 2 * k + (c <= 4 ? (c - 1) / 2 : ((c - 5) / 4) & 1);
-  if (c <= 22) return c - 1;
-  if (c <= 25) return 22 + k;
-  return 25;
+// first row and stride of column c's rows
+static __device__ __forceinline__ void rows_of(int c, int& r0, int& dr) {
+  r0 = c == 0 ? 0 : (c <= 4 ? (c - 1) / 2 : (c <= 20 ? ((c - 5) / 4) & 1 : (c <= 22 ? c - 1 : (c <= 25 ? 22 : 25))));
+  dr = c >= 1 && c <= 20 ? 2 : 1;
 }
 
-
-// d log kappa / d theta for flux-moment coordinate a (0..19): band b = a / 4,
-// kind e = a % 4 (0: kE0, 1: kE1, 2: kM0, 3: kM1).  Returns kappa.
-static __device__ real kappa_logderivs(const real* th, int a, real* dl, real* d2l) {
+// Row a (0..19) of the flux moments: band b = a / 4, kind e = a % 4 (0: kE0,
+// 1: kE1, 2: kM0, 3: kM1): kappa, d log kappa / d theta with its diagonal
+// second derivatives, and kappa's row of J.  The eleven coordinates that a
+// row depends on are written; the rest of the rows is zero on entry.
+static __device__ void kappa_row(const real* th, int a, EpiSmem& S) {
   const int b = a >> 2, e = a & 3;
   const int i = e & 1;
   const bool second = e >= 2;
   const real am = second ? 2.f : 1.f, av = second ? 2.f : 0.5f;
-  for (int c = 0; c < kTheta; ++c) dl[c] = d2l[c] = 0.f;
+  real* dl = S.DL + a * kTheta;
+  real* d2l = S.D2L + a * kTheta;
+  real* Ja = S.J + a * kTheta;
   const real q1 = sigm(th[0]), q0 = sigm(-th[0]);
   const real logq = i ? -softplus(-th[0]) : -softplus(th[0]);
-  dl[0] = i ? q0 : -q1;
-  d2l[0] = -q0 * q1;
+  const real l0 = i ? q0 : -q1;
   const int ir = 1 + 2 * i, iv = 2 + 2 * i;
   real m = th[ir], v = expf(th[iv]);
-  dl[ir] = am;
-  dl[iv] = av * v;
-  d2l[iv] = dl[iv];
+  const real lv = av * v;
+  real lm[4], lc[4];
+#pragma unroll
   for (int k = 0; k < 4; ++k) {
     const real s = (real)kSelE[b][k];
     const real cvk = expf(th[13 + 4 * i + k]);
     m += s * th[5 + 4 * i + k];
     v += s * s * cvk;
-    dl[5 + 4 * i + k] = am * s;
-    dl[13 + 4 * i + k] = av * s * s * cvk;
-    d2l[13 + 4 * i + k] = dl[13 + 4 * i + k];
+    lm[k] = am * s;
+    lc[k] = av * s * s * cvk;
   }
-  return expf(logq + am * m + av * v);
+  const real kap = expf(logq + am * m + av * v);
+  S.kap[a] = kap;
+  dl[0] = l0;
+  d2l[0] = -q0 * q1;
+  Ja[0] = kap * l0;
+  dl[ir] = am;
+  Ja[ir] = kap * am;
+  dl[iv] = d2l[iv] = lv;
+  Ja[iv] = kap * lv;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    dl[5 + 4 * i + k] = lm[k];
+    Ja[5 + 4 * i + k] = kap * lm[k];
+    dl[13 + 4 * i + k] = d2l[13 + 4 * i + k] = lc[k];
+    Ja[13 + 4 * i + k] = kap * lc[k];
+  }
 }
 
 // Derivatives of Sigma_s = (S11, S12, S22) over (angle, log radius, logit axis).
@@ -160,48 +204,88 @@ static __device__ void sigma_derivs(const real* th, real dS[3][3], real d2S[3][3
   d2S[1][2][2] = -Qtt * S2;
 }
 
-// KL_s: value into S.kls[0]; for kMode >= 1 the gradient and for kMode == 2
-// also the Hessian are ADDED (with a minus sign, since L = ... - KL) into
-// S.gth and S.Hth.
+// The terms of KL_s that stand alone, a lane each (lanes 0..8), into S.klt.
 template <int kMode>
-static __device__ void kl_terms(const real* th, const ModelDev* m, EpiSmem& S, int lane) {
+static __device__ __forceinline__ void kl_lone_terms(const real* th, const ModelDev::F32& f,
+                                                     EpiSmem& S, int lane) {
+  if (lane < 6) {
+    // softplus of -+theta_0, -+theta_25, -+theta_26
+    const int t = lane < 2 ? 0 : (lane < 4 ? 25 : 26);
+    S.klt[lane] = softplus(lane & 1 ? th[t] : -th[t]);
+  } else if (lane < 8) {
+    const int i = lane - 6;
+    const real R1 = f.prior_r[i][0], R2 = f.prior_r[i][1];
+    const real rm = th[1 + 2 * i], lrv = th[2 + 2 * i], rv = expf(lrv);
+    S.klt[6 + i] =
+        0.5f * (f.log_prior_r2[i] - lrv + (rv + (rm - R1) * (rm - R1)) / R2 - 1.f);
+    if (kMode >= 1) {
+      // gradient of K_i = KL_r + B over the mean and log variance of log r,
+      // and its second derivatives
+      S.klt[16 + 4 * i] = (rm - R1) / R2;
+      S.klt[17 + 4 * i] = 0.5f * (rv / R2 - 1.f);
+      S.klt[18 + 4 * i] = 1.f / R2;
+      S.klt[19 + 4 * i] = 0.5f * rv / R2;
+    }
+  } else if (lane == 8) {
+    const real lr = th[24], E1 = f.e_radius[0], E2 = f.e_radius[1];
+    S.klt[8] = lr + f.half_log_2pi_e2 + (lr - E1) * (lr - E1) / (2.f * E2);
+  }
+}
+
+// KL_s: value into S.kls[0]; for kMode >= 1 what depends on the type
+// probability, radius, axis and profile alone is ADDED (with a minus sign,
+// since L = ... - KL) into S.gth and S.Hth, and the rest left in S.pw and
+// S.klt for kl_scatter.  By one warp; f and J are the model's FP32 constants
+// and its number of colour components.  kApart: warp 3 forms the lone terms
+// and meets this warp at named barrier 3.
+template <int kMode, bool kApart>
+static __device__ void kl_terms(const real* th, const ModelDev::F32& f, int J, EpiSmem& S,
+                                int lane) {
   const real a = sigm(th[0]);
   const real wq = a * (1.f - a);
-  const int J = m->n_color;
+  if (!kApart) kl_lone_terms<kMode>(th, f, S, lane);
   // ---- colour bound, one lane per (type, component)
   if (lane < 2 * kMaxColor) {
     const int i = lane / kMaxColor, j = lane % kMaxColor;
     if (j < J) {
-      const float(*P)[4] = m->f.color_prec[i][j];
+      const float(*P)[4] = f.color_prec[i][j];
       const real* cm = th + 5 + 4 * i;
       const real* lcv = th + 13 + 4 * i;
       real d[4], cv[4], pd[4];
       real tr = 0.f, quad = 0.f, slv = 0.f;
+#pragma unroll
       for (int k = 0; k < 4; ++k) {
-        d[k] = cm[k] - m->f.color_mean[i][j][k];
+        d[k] = cm[k] - f.color_mean[i][j][k];
         cv[k] = expf(lcv[k]);
       }
+#pragma unroll
       for (int k = 0; k < 4; ++k) {
         real s = 0.f;
+#pragma unroll
         for (int l = 0; l < 4; ++l) s = fmaf(P[k][l], d[l], s);
         pd[k] = s;
         tr = fmaf(P[k][k], cv[k], tr);
         quad = fmaf(d[k], s, quad);
         slv += lcv[k];
       }
-      const real K = 0.5f * (tr + quad - 4.f + m->f.color_logdet[i][j] - slv);
-      S.klj[lane] = m->f.log_color_w[i][j] - K;
+      const real K = 0.5f * (tr + quad - 4.f + f.color_logdet[i][j] - slv);
+      S.klj[lane] = f.log_color_w[i][j] - K;
       if (kMode >= 1) {
         real* o = S.klc + lane * kKlVals;
         real gk[8];
+#pragma unroll
         for (int k = 0; k < 4; ++k) {
           gk[k] = pd[k];
           gk[4 + k] = 0.5f * (P[k][k] * cv[k] - 1.f);
         }
+#pragma unroll
         for (int k = 0; k < 8; ++k) o[k] = gk[k];
         int t = 8;
+#pragma unroll
         for (int k = 0; k < 4; ++k)
+#pragma unroll
           for (int l = k; l < 4; ++l) o[t++] = P[k][l];
+#pragma unroll
         for (int k = 0; k < 4; ++k) o[t++] = 0.5f * P[k][k] * cv[k];
       }
     } else {
@@ -213,26 +297,31 @@ static __device__ void kl_terms(const real* th, const ModelDev* m, EpiSmem& S, i
   if (lane < 2 * kMaxColor) {
     const int i = lane / kMaxColor;
     real mx = -INFINITY;
-    for (int j = 0; j < J; ++j) mx = fmaxf(mx, S.klj[i * kMaxColor + j]);
+#pragma unroll
+    for (int j = 0; j < kMaxColor; ++j) mx = fmaxf(mx, S.klj[i * kMaxColor + j]);
     S.kw[lane] = (lane % kMaxColor) < J ? expf(S.klj[lane] - mx) : 0.f;   // scratch
     S.kls[4 + i] = mx;
   }
   __syncwarp();
   real Bval[2], se[2];
+#pragma unroll
   for (int i = 0; i < 2; ++i) {
     se[i] = 0.f;
-    for (int j = 0; j < J; ++j) se[i] += S.kw[i * kMaxColor + j];
+#pragma unroll
+    for (int j = 0; j < kMaxColor; ++j) se[i] += S.kw[i * kMaxColor + j];
     Bval[i] = -(S.kls[4 + i] + logf(se[i]));
   }
   if (kMode >= 1) {
-    // pi-weighted sums per type (S.X as scratch, kKlSums per type): the mean
+    // pi-weighted sums per type (kKlSums per type): the mean
     // gradient, the precision block and the diagonal ...
     for (int e = lane; e < 2 * kKlVals; e += 32) {
       const int i = e / kKlVals, vv = e % kKlVals;
       real acc = 0.f;
-      for (int j = 0; j < J; ++j)
-        acc = fmaf(S.kw[i * kMaxColor + j], S.klc[(i * kMaxColor + j) * kKlVals + vv], acc);
-      S.X[i * kKlSums + (vv < 8 ? vv : 36 + vv)] = acc / se[i];
+#pragma unroll
+      for (int j = 0; j < kMaxColor; ++j)
+        if (j < J)
+          acc = fmaf(S.kw[i * kMaxColor + j], S.klc[(i * kMaxColor + j) * kKlVals + vv], acc);
+      S.pw[i * kKlSums + (vv < 8 ? vv : 36 + vv)] = acc / se[i];
     }
     __syncwarp();
     // ... then the covariance of the gradients across components in centred
@@ -242,62 +331,81 @@ static __device__ void kl_terms(const real* th, const ModelDev* m, EpiSmem& S, i
       int u = 0, rem = e % 36;
       while (rem >= 8 - u) { rem -= 8 - u; ++u; }
       const int w = u + rem;
-      const real gu = S.X[i * kKlSums + u], gw = S.X[i * kKlSums + w];
+      const real gu = S.pw[i * kKlSums + u], gw = S.pw[i * kKlSums + w];
       real acc = 0.f;
-      for (int j = 0; j < J; ++j) {
+#pragma unroll
+      for (int j = 0; j < kMaxColor; ++j) {
         const real* gj = S.klc + (i * kMaxColor + j) * kKlVals;
-        acc = fmaf(S.kw[i * kMaxColor + j], (gj[u] - gu) * (gj[w] - gw), acc);
+        if (j < J) acc = fmaf(S.kw[i * kMaxColor + j], (gj[u] - gu) * (gj[w] - gw), acc);
       }
-      S.X[i * kKlSums + 8 + (e % 36)] = acc / se[i];
+      S.pw[i * kKlSums + 8 + (e % 36)] = acc / se[i];
     }
   }
   __syncwarp();
+  if (kApart) asm volatile("bar.sync 3, 64;" ::: "memory");
   // ---- value (lane 0)
   if (lane == 0) {
-    real v = a * (-softplus(-th[0]) - m->f.log_prior_a) +
-             (1.f - a) * (-softplus(th[0]) - m->f.log1m_prior_a);
+    real v = fmaf(a, (-S.klt[0] - f.log_prior_a), __fmul_rn(1.f - a, (-S.klt[1] - f.log1m_prior_a)));
+#pragma unroll
     for (int i = 0; i < 2; ++i) {
-      const real R1 = m->f.prior_r[i][0], R2 = m->f.prior_r[i][1];
-      const real rm = th[1 + 2 * i], lrv = th[2 + 2 * i], rv = expf(lrv);
-      const real klr = 0.5f * (m->f.log_prior_r2[i] - lrv + (rv + (rm - R1) * (rm - R1)) / R2 - 1.f);
+      const real klr = S.klt[6 + i];
       S.kls[2 + i] = klr + Bval[i];
       v += (i ? a : 1.f - a) * S.kls[2 + i];
     }
-    const real lr = th[24], E1 = m->f.e_radius[0], E2 = m->f.e_radius[1];
-    v += lr + m->f.half_log_2pi_e2 + (lr - E1) * (lr - E1) / (2.f * E2);
+    v += S.klt[8];
+#pragma unroll
     for (int which = 0; which < 2; ++which) {
-      const int t = which ? 26 : 25;
-      const real b1 = (which ? m->f.e_profile[0] : m->f.e_axis[0]);
-      const real b2 = (which ? m->f.e_profile[1] : m->f.e_axis[1]);
-      v += (b1 - 1.f) * softplus(-th[t]) + (b2 - 1.f) * softplus(th[t]) +
-           (which ? m->f.log_beta_profile : m->f.log_beta_axis);
+      const real b1 = (which ? f.e_profile[0] : f.e_axis[0]);
+      const real b2 = (which ? f.e_profile[1] : f.e_axis[1]);
+      v += fmaf(b2 - 1.f, S.klt[3 + 2 * which], __fmul_rn(b1 - 1.f, S.klt[2 + 2 * which])) +
+           (which ? f.log_beta_profile : f.log_beta_axis);
     }
     S.kls[0] = v;
   }
   __syncwarp();
   if (kMode == 0) return;
+  if (lane == 0) {
+    const real la = f.logit_prior_a;
+    const real d2q = wq * (1.f - 2.f * a);
+    S.gth[0] -= wq * (th[0] - la) + wq * (S.kls[3] - S.kls[2]);
+    if (kMode == 2)
+      S.Hth[0] -= wq * ((1.f - 2.f * a) * (th[0] - la) + 1.f) + d2q * (S.kls[3] - S.kls[2]);
+  } else if (lane == 1) {
+    const real lr = th[24], E1 = f.e_radius[0], E2 = f.e_radius[1];
+    S.gth[24] -= 1.f + (lr - E1) / E2;
+    if (kMode == 2) S.Hth[24 * kTheta + 24] -= 1.f / E2;
+  } else if (lane < 4) {
+    const int which = lane - 2;
+    const int t = which ? 26 : 25;
+    const real b1 = (which ? f.e_profile[0] : f.e_axis[0]);
+    const real b2 = (which ? f.e_profile[1] : f.e_axis[1]);
+    const real sg = sigm(th[t]);
+    S.gth[t] -= -(b1 - 1.f) * (1.f - sg) + (b2 - 1.f) * sg;
+    if (kMode == 2) S.Hth[t * kTheta + t] -= (b1 + b2 - 2.f) * sg * (1.f - sg);
+  }
+  __syncwarp();
+}
+
+// The rest of the KL's gradient and Hessian, from S.pw and S.klt: the
+// blocks of each type's flux coordinates and their products with the type
+// probability, an entry a thread of the block.
+template <int kMode>
+static __device__ __forceinline__ void kl_scatter(const real* th, EpiSmem& S, int tid) {
+  const real a = sigm(th[0]);
+  const real wq = a * (1.f - a);
   // per type i, local coordinates 0 r-mean, 1 log r-var, 2..5 colour means,
   // 6..9 log colour vars; theta index of local k:
   auto tidx = [](int i, int k) {
     return k == 0 ? 1 + 2 * i : (k == 1 ? 2 + 2 * i : (k < 6 ? 5 + 4 * i + (k - 2) : 13 + 4 * i + (k - 6)));
   };
   // gradient-only mode visits the (i, k, l = 0) entries only
-  for (int e0 = lane; e0 < (kMode == 2 ? 200 : 20); e0 += 32) {
+  for (int e0 = tid; e0 < (kMode == 2 ? 200 : 20); e0 += kEpiThreads) {
     const int e = kMode == 2 ? e0 : (e0 / 10) * 100 + (e0 % 10) * 10;
     const int i = e / 100, k = (e % 100) / 10, l = e % 10;
-    const real* pw = S.X + i * kKlSums;       // grad(8), centred outer(36), prec(10), diag(4)
-    const real R2 = m->f.prior_r[i][1];
-    const real rm = th[1 + 2 * i], rv = expf(th[2 + 2 * i]);
-    // gradient of K_i = KL_r + B at local k
-    auto gK = [&](int kk) {
-      if (kk == 0) return (rm - m->f.prior_r[i][0]) / R2;
-      if (kk == 1) return 0.5f * (rv / R2 - 1.f);
-      return pw[kk - 2];
-    };
+    const real* pw = S.pw + i * kKlSums;       // grad(8), centred outer(36), prec(10), diag(4)
     real h = 0.f;
     if (k < 2 || l < 2) {
-      if (k == l && k == 0) h = 1.f / R2;
-      if (k == l && k == 1) h = 0.5f * rv / R2;
+      if (k == l) h = S.klt[18 + 4 * i + k];
     } else {
       const int u = k - 2, w = l - 2;        // colour block 0..7
       const int lo = u < w ? u : w, hi = u < w ? w : u;
@@ -315,7 +423,7 @@ static __device__ void kl_terms(const real* th, const ModelDev* m, EpiSmem& S, i
     if (kMode == 2) S.Hth[tidx(i, k) * kTheta + tidx(i, l)] -= qi * h;
     if (l == 0) {
       const real dq = i ? wq : -wq;
-      const real g = gK(k);
+      const real g = k < 2 ? S.klt[16 + 4 * i + k] : pw[k - 2];
       S.gth[tidx(i, k)] -= qi * g;
       if (kMode == 2) {
         S.Hth[tidx(i, k) * kTheta + 0] -= dq * g;
@@ -323,85 +431,75 @@ static __device__ void kl_terms(const real* th, const ModelDev* m, EpiSmem& S, i
       }
     }
   }
-  __syncwarp();
-  if (lane == 0) {
-    const real la = m->f.logit_prior_a;
-    const real d2q = wq * (1.f - 2.f * a);
-    S.gth[0] -= wq * (th[0] - la) + wq * (S.kls[3] - S.kls[2]);
-    if (kMode == 2)
-      S.Hth[0] -= wq * ((1.f - 2.f * a) * (th[0] - la) + 1.f) + d2q * (S.kls[3] - S.kls[2]);
-    const real lr = th[24], E1 = m->f.e_radius[0], E2 = m->f.e_radius[1];
-    S.gth[24] -= 1.f + (lr - E1) / E2;
-    if (kMode == 2) S.Hth[24 * kTheta + 24] -= 1.f / E2;
-    for (int which = 0; which < 2; ++which) {
-      const int t = which ? 26 : 25;
-      const real b1 = (which ? m->f.e_profile[0] : m->f.e_axis[0]);
-      const real b2 = (which ? m->f.e_profile[1] : m->f.e_axis[1]);
-      const real sg = sigm(th[t]);
-      S.gth[t] -= -(b1 - 1.f) * (1.f - sg) + (b2 - 1.f) * sg;
-      if (kMode == 2) S.Hth[t * kTheta + t] -= (b1 + b2 - 2.f) * sg * (1.f - sg);
-    }
-  }
-  __syncwarp();
 }
 
-// Slot j of the plan, by the whole block.  kMode: 0 value, 1 value + gradient, 2 value + gradient + Hessian.  Four
-// warps per source: warp 0 evaluates the KL terms while warps 1..3 reduce
-// the tile sums and apply the per-image maps; then warp 0 forms the Jacobian
-// rows and the two dense products (X = H_nu J, H_theta += J^T X) are spread
-// over the block in register-blocked chains.
+// Copies the model's FP32 constants into shared memory (threads tid, tid + n, ...).
+static __device__ __forceinline__ void stage_model(ModelDev::F32& dst, const ModelDev* model,
+                                                   int tid, int n) {
+  constexpr int kWords = sizeof(ModelDev::F32) / 4;
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(&model->f);
+  uint32_t* d = reinterpret_cast<uint32_t*>(&dst);
+  for (int e = tid; e < kWords; e += n) d[e] = src[e];
+}
+
+// Slot j of the plan, by the whole block (tid 0..127; S.th holds theta and
+// f the model's FP32 constants, both in shared memory).  kMode: 0 value,
+// 1 value + gradient, 2 value + gradient + Hessian.  Warp 0 evaluates the KL
+// terms; warps 1 and 2 add up the tile sums, a pair each at a time, while
+// warp 3 forms the Jacobian and the images' maps; then the maps are applied
+// and the two dense products (X = H_nu J, H_theta += J^T X) formed, an entry
+// a thread.  The results are left in S.gth, S.Hth; returns L_rel and L in
+// rel and full.
 template <int kMode>
 static __device__ __forceinline__ void epilogue_source(const PlanView& v,
-                                                const ModelDev* __restrict__ model,
-                                                EpiSmem& S, int j, double* elbo,
-                                                double* elbo_rel, double* grad_out,
-                                                double* hess_out, int use_trial) {
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  if (!v.active[j]) return;
-  const int src = v.src_ids[j];
-  // use_trial: bit 0 evaluates theta_trial; bit 1 (value mode only) asks
-  // for the pixel part alone, without the KL (the log-likelihood of the
-  // source's point values relative to its absence)
-  const bool trial = (use_trial & 1) != 0, pixel_only = kMode == 0 && (use_trial & 2) != 0;
-  const double* thd = trial ? v.theta_trial + (size_t)j * kTheta : v.theta + (size_t)src * kTheta;
-  if (tid < kTheta) S.th[tid] = (real)thd[tid];
+                                                const ModelDev::F32& f, int n_color,
+                                                EpiSmem& S, int j, int tid, bool pixel_only,
+                                                double& rel, double& full) {
+  const int lane = tid & 31, wid = tid >> 5;
   const real* th = S.th;
-
-  double vrel = 0.0, vbase = 0.0;
+  const int p0 = v.slot_pair_ptr[j], p1 = v.slot_pair_ptr[j + 1];
   if (kMode >= 1) {
-    // the slot's tile sums (its pairs' items are contiguous, 256 B an item)
-    // asked into L2 at once: the pair loop below then reads them from L2,
-    // not from DRAM, pair after pair
-    const int p0 = v.slot_pair_ptr[j], p1 = v.slot_pair_ptr[j + 1];
-    if (p1 > p0) {
-      const int64_t i0 = v.pairs[p0].item_begin, i1 = v.pairs[p1 - 1].item_end;
-      const char* base = reinterpret_cast<const char*>(v.partials + i0 * kAcc);
-      const int64_t lines = (i1 - i0) * (kAcc * (int64_t)sizeof(float) / 128);
-      for (int64_t l = tid; l < lines; l += kEpiThreads)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(base + 128 * l));
-    }
-    for (int e = tid; e < kNuPad; e += kEpiThreads) S.gnu[e] = 0.f;
-    for (int e = tid; e < kNuPad; e += kEpiThreads) S.gth[e] = 0.f;
+    if (tid < kNuPad) S.gnu[tid] = S.gth[tid] = 0.f;
+    for (int e = tid; e < kNu * kTheta; e += kEpiThreads) S.J[e] = 0.f;
+    for (int e = tid; e < 20 * kTheta; e += kEpiThreads) S.DL[e] = S.D2L[e] = 0.f;
   }
   if (kMode == 2) {
     for (int e = tid; e < kNu * kNu; e += kEpiThreads) S.Hnu[e] = 0.f;
     for (int e = tid; e < kTheta * kTheta; e += kEpiThreads) S.Hth[e] = 0.f;
   }
   __syncthreads();
-  // Warp 0 evaluates the KL terms, which depend on theta alone, while warps
-  // 1..3 reduce the pixel sums pair by pair (named barrier 1 among them).
   if (wid == 0) {
-    if (!pixel_only) kl_terms<kMode>(th, model, S, lane);
+    if (!pixel_only) kl_terms<kMode, (kMode >= 1)>(th, f, n_color, S, lane);
   } else {
     const int u = tid - 32;                            // 0 .. kPairThreads - 1
     double vr = 0.0, vb = 0.0;
     if (kMode == 0) {
-      // value sums of every pair's items, thread-strided, then one reduction
-      for (int pp = v.slot_pair_ptr[j]; pp < v.slot_pair_ptr[j + 1]; ++pp) {
-        const PairInfo pi = v.pairs[pp];
-        for (int it = pi.item_begin + u; it < pi.item_end; it += kPairThreads) {
-          vr += (double)v.vpartials[2 * (size_t)it];
-          vb += (double)v.vpartials[2 * (size_t)it + 1];
+      // value sums of every pair's items, thread-strided, then one reduction;
+      // eight pairs' first items are loaded together
+      for (int pg = p0; pg < p1; pg += 8) {
+        int ib[8], ie[8];
+        float2 x[8];
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+          ib[g] = ie[g] = 0;
+          if (pg + g < p1) {
+            ib[g] = v.pairs[pg + g].item_begin + u;
+            ie[g] = v.pairs[pg + g].item_end;
+          }
+        }
+#pragma unroll
+        for (int g = 0; g < 8; ++g)
+          if (ib[g] < ie[g]) x[g] = reinterpret_cast<const float2*>(v.vpartials)[ib[g]];
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+          if (ib[g] < ie[g]) {
+            vr += (double)x[g].x;
+            vb += (double)x[g].y;
+            for (int it = ib[g] + kPairThreads; it < ie[g]; it += kPairThreads) {
+              vr += (double)v.vpartials[2 * (size_t)it];
+              vb += (double)v.vpartials[2 * (size_t)it + 1];
+            }
+          }
         }
       }
       vr = warp_sum_d(vr);
@@ -412,281 +510,311 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
       }
       pair_sync();
       if (u == 0) {
-        vr = S.red[0][0] + S.red[0][1] + S.red[0][2];
-        vb = S.red[1][0] + S.red[1][1] + S.red[1][2];
+        S.vsum[0] = S.red[0][0] + S.red[0][1] + S.red[0][2];
+        S.vsum[1] = S.red[1][0] + S.red[1][1] + S.red[1][2];
       }
     } else {
-      // kPairGroup pairs at a time: their tile sums in one loop (loads of
-      // every pair in flight together) and their images' maps, then the
-      // per-pair updates in pair order; each sum below is updated by one
-      // thread, pair after pair, as with one pair at a time
-      const int pend = v.slot_pair_ptr[j + 1];
-      for (int pp = v.slot_pair_ptr[j]; pp < pend; pp += kPairGroup) {
-        const int ng = min(kPairGroup, pend - pp);
-        if (u < kAcc) {
-          // the pairs' tile sums, accumulator u: compensated (Kahan) FP32
-          // summation whose error does not grow with the number of tiles;
-          // the loads are independent of the chains, so they run ahead
-          float s0[kPairGroup], c0[kPairGroup];
-          int ib[kPairGroup], nit[kPairGroup];
-          int nmax = 0;
+      if (wid == 3) {
+        kl_lone_terms<kMode>(th, f, S, lane);
+        asm volatile("bar.arrive 3, 64;" ::: "memory");
+        if (lane < 20) {
+          kappa_row(th, lane, S);
+        } else if (lane < 22) {
+          S.J[lane * kTheta + 21 + (lane - 20)] = 1.f;
+        } else if (lane == 22) {
+          real dS[3][3], d2S[3][3][3];
+          sigma_derivs(th, dS, d2S);
 #pragma unroll
-          for (int g = 0; g < kPairGroup; ++g) {
-            s0[g] = c0[g] = 0.f;
-            ib[g] = nit[g] = 0;
-            if (g < ng && (kMode == 2 || u < kGradAcc)) {
-              ib[g] = v.pairs[pp + g].item_begin;
-              nit[g] = v.pairs[pp + g].item_end - ib[g];
-              nmax = max(nmax, nit[g]);
+          for (int e = 0; e < 3; ++e)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+              S.J[(22 + e) * kTheta + 23 + c] = dS[e][c];
+#pragma unroll
+              for (int d = 0; d < 3; ++d) S.d2S[9 * e + 3 * c + d] = d2S[e][c][d];
             }
-          }
+        } else if (lane == 25) {
+          const real r = sigm(th[26]);
+          S.J[25 * kTheta + 26] = r * (1.f - r);
+        }
+        __syncwarp();
+      }
+      // thread u's entry of H_nu (upper triangle of the ten w, u < 55) or of
+      // grad_nu (the next ten): the terms of its sum over the w, as offsets
+      // into T and W; terms it does not have multiply entry 0 of W, zero
+      auto lo = [](int a) { return a < 4 ? a : (a < 6 ? 4 : (a < 9 ? 6 : 9)); };
+      auto hi = [](int a) { return a < 4 ? a + 1 : (a < 6 ? 6 : (a < 9 ? 9 : 10)); };
+      const bool ghess = u < kGeoHess, ggrad = u >= kGeoHess && u < kGeoHess + kW;
+      int ea = ghess ? 0 : min(u - kGeoHess, kW - 1), ec = ea;
+      int tk[3], tl[3], wo[9];
+      if (ghess) {
+        int r = u;
+        while (r >= 10 - ea) { r -= 10 - ea; ++ea; }
+        ec = ea + r;
+      }
+      const int ka = lo(ea), la = lo(ec), na3 = hi(ea) - ka, nc3 = ghess ? hi(ec) - la : 1;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        tk[i] = i < na3 ? (ka + i) * 10 + ea : 99;
+        tl[i] = ghess && i < nc3 ? (la + i) * 10 + ec : 99;
+      }
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        const int k = ka + q / 3, l = la + q % 3, kk = min(k, l), ll = max(k, l);
+        const bool zero = ghess && kk >= 2 && kk <= 3 && ll <= 3;   // (cM, cM): vanish
+        const bool on = q / 3 < na3 && q % 3 < nc3 && !zero;
+        wo[q] = !on ? 0 : (ghess ? hidx(kk, ll) : 2 + k);
+      }
+      for (int pp = p0; pp < p1; pp += kPairGroup) {
+        const int ng = min(kPairGroup, p1 - pp);
+        int ib = 0, ie = 0, im = 0;
+        if (lane < ng) {
+          const PairInfo& pi = v.pairs[pp + lane];
+          ib = pi.item_begin;
+          ie = pi.item_end;
+          im = pi.image;
+          if (wid == 3) S.band[lane] = pi.band;
+        }
+        if (wid < 3) {
+          // the tile sums of the group's pairs, whose items are contiguous:
+          // chunks of kTileChunk tiles (256 B each) are copied to shared
+          // memory, one chunk ahead, and warps 1 and 2 add up a pair each at
+          // a time: lane l forms accumulators 2 l and 2 l + 1 by compensated
+          // (Kahan) FP32 summation in tile order, whose error does not grow
+          // with the number of tiles
+          const int t0 = __shfl_sync(0xffffffffu, ib, 0);
+          const int t1 = __shfl_sync(0xffffffffu, ie, ng - 1);
+          auto fetch = [&](int c) {
+            const int n16 = min(kTileChunk, t1 - t0 - c * kTileChunk) * (kAcc / 4);
+            const float* src = v.partials + (size_t)(t0 + c * kTileChunk) * kAcc;
+            float* dst = &S.tiles[c & 1][0][0];
+            for (int e = u; e < n16; e += 64) copy_async16(dst + 4 * e, src + 4 * e);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+          };
+          const int nc = (t1 - t0 + kTileChunk - 1) / kTileChunk;
+          fetch(0);
+          int g = wid - 1;
+          float2 s = make_float2(0.f, 0.f), c = s;
+          for (int ch = 0; ch < nc; ++ch) {
+            if (ch + 1 < nc) {
+              fetch(ch + 1);
+              asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+              asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            tile_sync();
+            const int c0 = t0 + ch * kTileChunk, c1 = c0 + kTileChunk;
+            const float2* x = reinterpret_cast<const float2*>(&S.tiles[ch & 1][0][0]) + lane;
+            while (g < ng) {
+              const int b = __shfl_sync(0xffffffffu, ib, g), e = __shfl_sync(0xffffffffu, ie, g);
+              if (b >= c1) break;
+              const int q1 = min(e, c1) - c0;
 #pragma unroll 4
-          for (int t = 0; t < nmax; ++t) {
-#pragma unroll
-            for (int g = 0; g < kPairGroup; ++g) {
-              if (t < nit[g]) {
-                const float y0 = v.partials[(size_t)(ib[g] + t) * kAcc + u] - c0[g];
-                const float t0 = s0[g] + y0;
-                c0[g] = (t0 - s0[g]) - y0;
-                s0[g] = t0;
+              for (int q = max(b, c0) - c0; q < q1; ++q) {
+                const float2 y = x[q * (kAcc / 2)];
+                const float ya = y.x - c.x, yb = y.y - c.y;
+                const float ta = s.x + ya, tb = s.y + yb;
+                c.x = (ta - s.x) - ya;
+                c.y = (tb - s.y) - yb;
+                s.x = ta;
+                s.y = tb;
               }
-            }
-          }
-          // the value sums go on in FP64; the others are used in FP32, and
-          // s0 - c0 rounded once to FP32 equals (float)((double)s0 -
-          // (double)c0): that double difference is exact or off s0 by far
-          // less than half an FP32 unit in the last place
-#pragma unroll
-          for (int g = 0; g < kPairGroup; ++g) {
-            if (g < ng) {
-              if (u < 2) {
-                S.Wd[g][u] = (double)s0[g] - (double)c0[g];
+              if (e > c1) break;                       // goes on in the next chunk
+              // the value sums go on in FP64; the others are used in FP32,
+              // and s - c rounded once to FP32 equals (float)((double)s -
+              // (double)c): that double difference is exact or off s by far
+              // less than half an FP32 unit in the last place
+              if (lane == 0) {
+                S.W[g][0] = 0.f;
+                S.vs[g][0] = s.x;
+                S.vs[g][1] = c.x;
+                S.vs[g][2] = s.y;
+                S.vs[g][3] = c.y;
               } else {
-                S.W[g][u] = s0[g] - c0[g];
+                S.W[g][2 * lane] = s.x - c.x;
+                S.W[g][2 * lane + 1] = s.y - c.y;
               }
+              s = c = make_float2(0.f, 0.f);
+              g += 2;
             }
+            tile_sync();                               // before the buffer is filled again
           }
         } else {
-          // each pair's local affine map, FP32: w_k = sum_a T[k][a] nu_a
-          for (int g = 0; g < ng; ++g) {
-            const celeste_image& im = v.images[v.pairs[pp + g].image];
-            const float cal = (float)im.calib;
-            const float A0 = (float)im.wcs_A[0], A1 = (float)im.wcs_A[1];
-            const float A2 = (float)im.wcs_A[2], A3 = (float)im.wcs_A[3];
-            for (int e = u - kAcc; e < 100; e += kPairThreads - kAcc) {
-              float t = 0.f;
-              switch (e) {
-                case 0: case 11: t = cal; break;
-                case 22: case 33: t = cal * cal; break;
-                case 44: t = A0; break;
-                case 45: t = A1; break;
-                case 54: t = A2; break;
-                case 55: t = A3; break;
-                case 66: t = A0 * A0; break;
-                case 67: t = 2.f * A0 * A1; break;
-                case 68: t = A1 * A1; break;
-                case 76: t = A0 * A2; break;
-                case 77: t = A0 * A3 + A1 * A2; break;
-                case 78: t = A1 * A3; break;
-                case 86: t = A2 * A2; break;
-                case 87: t = 2.f * A2 * A3; break;
-                case 88: t = A3 * A3; break;
-                case 99: t = 1.f; break;
-                default: break;
-              }
-              S.T[g][e] = t;
+          // each pair's local affine map, FP32: w_k = sum_a T[k][a] nu_a;
+          // five values of an image (calibration, A) in five lanes, so that
+          // six images share a conversion.  Lanes 0..17 form an entry each,
+          // from values i1 and i2 (three bits a lane): kind 0 the value i1, 1
+          // the product, 2 twice it, 3 A0 A3 + A1 A2, 4 one
+          constexpr uint64_t kKind = 0412113112100001100ull, kOne = 043321121143210000ull, kTwo = 044344322100000000ull;
+          const int sh = 3 * min(lane, 17), bl = lane - 8;
+          const int kind = (int)(kKind >> sh & 7), i1 = (int)(kOne >> sh & 7), i2 = (int)(kTwo >> sh & 7);
+          const int te = lane < 4 ? 11 * lane
+                                  : (lane < 8 ? 44 + ((lane - 4) >> 1) * 10 + (lane & 1)
+                                              : (lane < 17 ? 66 + bl / 3 * 10 + bl % 3 : 99));
+          for (int g0 = 0; g0 < ng; g0 += 6) {
+            const int g = g0 + lane / 5, q = lane % 5;
+            const int image = __shfl_sync(0xffffffffu, im, min(g, ng - 1));
+            float x = 0.f;
+            if (lane < 30) {
+              const celeste_image& I = v.images[image];
+              x = (float)(q == 0 ? I.calib : I.wcs_A[q - 1]);
+            }
+            for (int h = 0; h < min(6, ng - g0); ++h) {
+              const float f1 = __shfl_sync(0xffffffffu, x, 5 * h + i1);
+              const float f2 = __shfl_sync(0xffffffffu, x, 5 * h + i2);
+              const float f3 = __shfl_sync(0xffffffffu, x, 5 * h + 2);
+              const float f4 = __shfl_sync(0xffffffffu, x, 5 * h + 3);
+              float t = f1 * f2;
+              if (kind == 0) t = f1;
+              if (kind == 2) t = 2.f * f1 * f2;
+              if (kind == 3) t = f1 * f2 + f3 * f4;
+              if (kind == 4) t = 1.f;
+              if (lane < 18) S.T[g0 + h][te] = t;
             }
           }
         }
         pair_sync();
-        auto lo = [](int a) { return a < 4 ? a : (a < 6 ? 4 : (a < 9 ? 6 : 9)); };
-        auto hi = [](int a) { return a < 4 ? a + 1 : (a < 6 ? 6 : (a < 9 ? 9 : 10)); };
-        if (u < 10) {
+        // the maps applied, in pair order, an entry a thread
+        if ((kMode == 2 && ghess) || ggrad) {
           for (int g = 0; g < ng; ++g) {
-            const int b = v.pairs[pp + g].band;
             const float* T = S.T[g];
             const float* W = S.W[g];
-            float gl = 0.f;
-            for (int k = lo(u); k < hi(u); ++k) gl += T[k * 10 + u] * W[2 + k];
-            S.gnu[u < 4 ? 4 * b + u : 16 + u] += gl;    // nu of w_u (4..9 -> 20..25)
-          }
-        } else if (kMode == 2 && u >= 32 && u < 32 + 55) {
-          const int e = u - 32;
-          int a = 0, rem = e;
-          while (rem >= 10 - a) { rem -= 10 - a; ++a; }
-          const int c = a + rem;
-          for (int g = 0; g < ng; ++g) {
-            const int b = v.pairs[pp + g].band;
-            const float* T = S.T[g];
-            const float* W = S.W[g];
-            float val = 0.f;
-            for (int k = lo(a); k < hi(a); ++k)
-              for (int l = lo(c); l < hi(c); ++l) {
-                const int kk = k < l ? k : l, ll = k < l ? l : k;
-                const bool zero = (kk == 2 || kk == 3) && (ll == 2 || ll == 3);
-                const float hwv = zero ? 0.f : W[hidx(kk, ll)];
-                val = fmaf(T[k * 10 + a] * T[l * 10 + c], hwv, val);
-              }
-            const int na = a < 4 ? 4 * b + a : 16 + a, nc = c < 4 ? 4 * b + c : 16 + c;
-            S.Hnu[na * kNu + nc] += val;
-            if (na != nc) S.Hnu[nc * kNu + na] += val;
+            const int b = S.band[g];
+            float x[9], p[9], val = 0.f;
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+              x[q] = W[wo[q]];
+              p[q] = T[tk[q / 3]] * T[tl[q % 3]];    // (entry 99 of T is one)
+            }
+#pragma unroll
+            for (int q = 0; q < 9; ++q) val = fmaf(p[q], x[q], val);
+            const int na = ea < 4 ? 4 * b + ea : 16 + ea, nc = ec < 4 ? 4 * b + ec : 16 + ec;
+            if (ghess) S.Hnu[na * kNu + nc] += val;
+            else S.gnu[na] += val;                   // nu of w_a (4..9 -> 20..25)
           }
         }
-        if (u == 0) {
-          for (int g = 0; g < ng; ++g) {
-            vr += S.Wd[g][0];
-            vb += S.Wd[g][1];
+        if (wid == 1) {
+          // the value sums of the group's pairs, in pair order: lane 2 g + h
+          // holds pair g's relative (h = 0) or base sum, lanes 0 and 1 add
+          double d = 0.0;
+          if (lane < 2 * ng) {
+            const float* x = S.vs[lane >> 1] + 2 * (lane & 1);
+            d = (double)x[0] - (double)x[1];
           }
+          for (int g = 0; g < ng; ++g) vr += __shfl_sync(0xffffffffu, d, 2 * g + (lane & 1));
         }
-        pair_sync();
+        if (pp + kPairGroup < p1) pair_sync();
       }
-    }
-    if (u == 0) {
-      S.vsum[0] = vr;
-      S.vsum[1] = vb;
+      if (wid == 1 && lane < 2) S.vsum[lane] = vr;
     }
   }
   __syncthreads();
-  vrel = S.vsum[0];
-  vbase = S.vsum[1];
   const double kl = pixel_only ? 0.0 : (double)S.kls[0];
+  rel = S.vsum[0] - kl;
+  full = S.vsum[1] + S.vsum[0] - kl;
   if (kMode >= 1) {
-    if (wid == 0) {
-      // Jacobian rows: flux moments (lanes 0..19), u, Sigma_s, rho
-      for (int e = lane; e < kNu * kTheta; e += 32) S.J[e] = 0.f;
-      __syncwarp();
-      if (lane < 20) {
-        real* dl = S.DL + lane * kTheta;
-        real* d2l = S.D2L + lane * kTheta;
-        const real kap = kappa_logderivs(th, lane, dl, d2l);
-        for (int c = 0; c < kTheta; ++c) S.J[lane * kTheta + c] = kap * dl[c];
-        S.kw[lane] = S.gnu[lane] * kap;
-      } else if (lane < 22) {
-        S.J[lane * kTheta + 21 + (lane - 20)] = 1.f;
-      } else if (lane == 22) {
-        real dS[3][3], d2S[3][3][3];
-        sigma_derivs(th, dS, d2S);
-        for (int e = 0; e < 3; ++e)
-          for (int c = 0; c < 3; ++c) S.J[(22 + e) * kTheta + 23 + c] = dS[e][c];
-        real h[3][3] = {{0.f}};
-        for (int e = 0; e < 3; ++e)
-          for (int c = 0; c < 3; ++c)
-            for (int d = 0; d < 3; ++d) h[c][d] += S.gnu[22 + e] * d2S[e][c][d];
-        for (int c = 0; c < 3; ++c)
-          for (int d = 0; d < 3; ++d) S.X[8 * 64 + c * 3 + d] = h[c][d];   // parked below
-      } else if (lane == 25) {
+    kl_scatter<kMode>(th, S, tid);
+    if (kMode == 2) {
+      // the lower triangle of H_nu
+      for (int e = tid; e < kNu * kNu; e += kEpiThreads) {
+        const int a = e / kNu, c = e - a * kNu;
+        if (a > c) S.Hnu[e] = S.Hnu[c * kNu + a];
+      }
+      if (tid < 20) S.kw[tid] = S.gnu[tid] * S.kap[tid];
+      __syncthreads();
+      // X = H_nu J where J's column has support.  Columns 0..20 (ten or
+      // twenty rows): thread (c, g) forms rows a = g, g + 4, ... of column c,
+      // seven chains sharing each entry of J; the other columns (one or three
+      // rows), an entry a thread
+      if (tid < 4 * 21) {
+        const int c = tid % 21, g = tid / 21, nr = nrows(c);
+        int r, dr;
+        rows_of(c, r, dr);
+        real x[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 5
+        for (int k = 0; k < nr; ++k, r += dr) {
+          const real jv = S.J[r * kTheta + c];
+#pragma unroll
+          for (int m = 0; m < 7; ++m)
+            x[m] = fmaf(S.Hnu[min(g + 4 * m, kNu - 1) * kNu + r], jv, x[m]);
+        }
+#pragma unroll
+        for (int m = 0; m < 7; ++m)
+          if (g + 4 * m < kNu) S.X[(g + 4 * m) * kTheta + c] = x[m];
+      } else {
+        for (int e = tid - 4 * 21; e < 6 * kNu; e += kEpiThreads - 4 * 21) {
+          const int c = 21 + e % 6, a = e / 6, nr = nrows(c);
+          int r, dr;
+          rows_of(c, r, dr);
+          real x = 0.f;
+          for (int k = 0; k < nr; ++k) x = fmaf(S.Hnu[a * kNu + r + k], S.J[(r + k) * kTheta + c], x);
+          S.X[a * kTheta + c] = x;
+        }
+      }
+      if (tid < 9) {
+        // Sigma_s second-order chain term
+        real h = 0.f;
+#pragma unroll
+        for (int e = 0; e < 3; ++e) h += S.gnu[22 + e] * S.d2S[9 * e + tid];
+        S.Hth[(23 + tid / 3) * kTheta + 23 + tid % 3] += h;
+      } else if (tid == 32) {
         const real r = sigm(th[26]);
-        S.J[25 * kTheta + 26] = r * (1.f - r);
-      }
-      __syncwarp();
-      if (kMode == 2) {
-        // Sigma_s second-order chain term (parked by lane 22 in X's space)
-        if (lane < 9) S.Hth[(23 + lane / 3) * kTheta + 23 + lane % 3] += S.X[8 * 64 + lane];
-        if (lane == 0) {
-          const real r = sigm(th[26]);
-          S.Hth[26 * kTheta + 26] += S.gnu[25] * r * (1.f - r) * (1.f - 2.f * r);
-        }
-      }
-      __syncwarp();
-      // gradient: J^T grad_nu over each column's rows
-      if (lane < kTheta) {
-        const int nr = nrows(lane);
-        real gsum = 0.f;
-        for (int k = 0; k < nr; ++k) {
-          const int a = rowof(lane, k);
-          gsum = fmaf(S.J[a * kTheta + lane], S.gnu[a], gsum);
-        }
-        S.gth[lane] += gsum;
+        S.Hth[26 * kTheta + 26] += S.gnu[25] * r * (1.f - r) * (1.f - 2.f * r);
       }
     }
     __syncthreads();
+    // gradient: J^T grad_nu over each column's rows
+    if (tid >= kEpiThreads - kTheta) {
+      const int c = tid - (kEpiThreads - kTheta), nr = nrows(c);
+      int r, dr;
+      rows_of(c, r, dr);
+      real gsum = 0.f;
+#pragma unroll 5
+      for (int k = 0; k < nr; ++k, r += dr) gsum = fmaf(S.J[r * kTheta + c], S.gnu[r], gsum);
+      S.gth[c] += gsum;
+    }
     if (kMode == 2) {
-      // X = H_nu J where J's column has support: thread (c, g) forms rows
-      // a = g, g + 4, ... of column c, seven independent chains sharing
-      // each entry of J
-      if (tid < 4 * kTheta) {
-        const int c = tid % kTheta, g = tid / kTheta;
-        const int nr = nrows(c);
-        real x[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int k = 0; k < nr; ++k) {
-          const int r = rowof(c, k);
-          const real jv = S.J[r * kTheta + c];
-#pragma unroll
-          for (int m = 0; m < 7; ++m) {
-            const int a = g + 4 * m;
-            if (a < kNu) x[m] = fmaf(S.Hnu[a * kNu + r], jv, x[m]);
-          }
-        }
-#pragma unroll
-        for (int m = 0; m < 7; ++m) {
-          const int a = g + 4 * m;
-          if (a < kNu) S.X[a * kTheta + c] = x[m];
-        }
-      }
-      __syncthreads();
       // Hth += J^T X over d >= c (mirrored), plus the flux-moment
       // second-order term sum_a kw_a (dl dl^T + diag d2l): thread (c, g)
-      // takes d = c + g, c + g + 4, ...
+      // takes d = c + g, c + g + 4, ..., seven chains
       if (tid < 4 * kTheta) {
-        const int c = tid % kTheta, g = tid / kTheta;
-        const int nr = nrows(c);
+        const int c = tid % kTheta, g = tid / kTheta, nr = nrows(c);
+        int r0, dr;
+        rows_of(c, r0, dr);
         real x[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int k = 0; k < nr; ++k) {
-          const int r = rowof(c, k);
+        int d[7];
+#pragma unroll
+        for (int m = 0; m < 7; ++m) d[m] = min(c + g + 4 * m, kTheta - 1);
+        int r = r0;
+#pragma unroll 5
+        for (int k = 0; k < nr; ++k, r += dr) {
           const real jv = S.J[r * kTheta + c];
 #pragma unroll
-          for (int m = 0; m < 7; ++m) {
-            const int d = c + g + 4 * m;
-            if (d < kTheta) x[m] = fmaf(jv, S.X[r * kTheta + d], x[m]);
-          }
+          for (int m = 0; m < 7; ++m) x[m] = fmaf(jv, S.X[r * kTheta + d[m]], x[m]);
         }
         if (c <= 20) {
-          for (int k = 0; k < nr; ++k) {
-            const int a = rowof(c, k);
-            if (a >= 20) break;
-            const real kd = S.kw[a] * S.DL[a * kTheta + c];
+          r = r0;
+#pragma unroll 5
+          for (int k = 0; k < nr; ++k, r += dr) {
+            const real kd = S.kw[r] * S.DL[r * kTheta + c];
+            const real xd = fmaf(kd, S.DL[r * kTheta + d[0]], x[0]);
+            x[0] = g == 0 ? fmaf(S.kw[r], S.D2L[r * kTheta + c], xd) : (d[0] <= 20 ? xd : x[0]);
 #pragma unroll
-            for (int m = 0; m < 7; ++m) {
-              const int d = c + g + 4 * m;
-              if (d <= 20) {
-                x[m] = fmaf(kd, S.DL[a * kTheta + d], x[m]);
-                if (d == c) x[m] = fmaf(S.kw[a], S.D2L[a * kTheta + c], x[m]);
-              }
+            for (int m = 1; m < 7; ++m) {
+              const real xm = fmaf(kd, S.DL[r * kTheta + d[m]], x[m]);
+              if (d[m] <= 20) x[m] = xm;
             }
           }
         }
 #pragma unroll
         for (int m = 0; m < 7; ++m) {
-          const int d = c + g + 4 * m;
-          if (d < kTheta) {
-            S.Hth[c * kTheta + d] += x[m];
-            if (d != c) S.Hth[d * kTheta + c] += x[m];
+          if (c + g + 4 * m < kTheta) {
+            S.Hth[c * kTheta + d[m]] += x[m];
+            if (d[m] != c) S.Hth[d[m] * kTheta + c] += x[m];
           }
         }
       }
-      __syncthreads();
     }
-  }
-
-  const double Lrel = vrel - kl;
-  const double Lfull = vbase + vrel - kl;
-  if (tid == 0) {
-    if (elbo) elbo[j] = Lfull;
-    if (elbo_rel) elbo_rel[j] = Lrel;
-    // a non-finite value at a trial point is a rejected step, not an error
-    if (!isfinite(Lfull) && !trial) set_error(v.err, CELESTE_DERR_NONFINITE);
-  }
-  if (kMode >= 1) {
-    int bad = 0;
-    for (int e = tid; e < kTheta; e += kEpiThreads) {
-      grad_out[(size_t)j * kTheta + e] = (double)S.gth[e];
-      bad |= !isfinite(S.gth[e]);
-    }
-    for (int e = tid; e < (kMode == 2 ? kTheta * kTheta : 0); e += kEpiThreads) {
-      hess_out[(size_t)j * kTheta * kTheta + e] = (double)S.Hth[e];
-      bad |= !isfinite(S.Hth[e]);
-    }
-    if (__syncthreads_or(bad) && tid == 0) set_error(v.err, CELESTE_DERR_NONFINITE);
+    __syncthreads();
   }
 }
 

@@ -123,8 +123,6 @@ struct PlanView {
   double* kl_trial;           // [n] KL_s at theta_trial (the per-source Newton step)
   double* rel_trial;          // [n] L_rel at theta_trial
   double* elbo_rel;           // [n] value at the current iterate
-  double* grad;               // [n][27] scratch for newton_step
-  double* hess;               // [n][27][27]
   uint8_t* active;            // [n] 1 if the slot takes part in the evaluation
   unsigned int* err;          // device error word
   float2* cache;              // problem render cache (pool layout) or null
@@ -257,6 +255,15 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+// Thread number within a block of four warps, with the warps renumbered from
+// block to block: a kernel whose warp 0 does the serial FP64 work would
+// otherwise queue every resident block's on one sub-partition of the SM
+// (warps go to sub-partitions by their number; blocks b and b + n_sm tend to
+// share an SM).
+__device__ __forceinline__ int rotated_tid(int n_sm) {
+  return (int)((threadIdx.x + 32u * (blockIdx.x + blockIdx.x / (unsigned)n_sm)) & 127u);
 }
 
 // A slot takes part in a Newton iteration unless its source has stopped.

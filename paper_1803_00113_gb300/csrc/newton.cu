@@ -8,13 +8,14 @@ namespace celeste {
 __global__ void __launch_bounds__(kTrThreads, 4) tr_subproblem_kernel(int n, const double* g,
                                                                   const double* H,
                                                                   const double* delta, double* p,
-                                                                  double* pred) {
+                                                                  double* pred, int n_sm) {
   extern __shared__ double smd[];
   TrSmem& S = *reinterpret_cast<TrSmem*>(smd);
   const int j = blockIdx.x;
   if (j >= n) return;
-  if (!tr_solve(S, g + (size_t)j * N, H + (size_t)j * N * N, delta[j])) return;
-  const int lane = threadIdx.x & 31;
+  const int tid = rotated_tid(n_sm), lane = tid & 31;
+  tr_load(S, g + (size_t)j * N, H + (size_t)j * N * N, tid);
+  if (!tr_solve(S, delta[j], tid)) return;
   if (lane < N) p[(size_t)j * N + lane] = S.y[lane];
   if (lane == 0) pred[j] = S.red[0];
 }
@@ -32,7 +33,8 @@ cudaError_t launch_tr_subproblem(const Launch& L, int n, const double* g, const 
                                  const double* delta, double* p, double* pred) {
   if (n <= 0) return cudaSuccess;
   if (cudaError_t e = set_attrs()) return e;
-  tr_subproblem_kernel<<<n, kTrThreads, sizeof(TrSmem), L.stream>>>(n, g, H, delta, p, pred);
+  tr_subproblem_kernel<<<n, kTrThreads, sizeof(TrSmem), L.stream>>>(n, g, H, delta, p, pred,
+                                                                      L.sm_count);
   return cudaGetLastError();
 }
 

@@ -21,29 +21,75 @@ namespace celeste {
 
 static_assert(kEpiThreads == kTrThreads, "the stages share one block shape");
 
-union StepSmem {
-  EpiSmem e;
-  TrSmem t;
+struct StepSmem {
+  union {
+    EpiSmem e;
+    TrSmem t;
+  };
+  ModelDev::F32 f;
 };
 static_assert(sizeof(EpiSmem::Hnu) >= 3 * 64 * sizeof(float), "setup scratch of warps 1..3");
 
-// Five blocks per SM (96 registers, a few hundred bytes of spills): a colour
-// class of up to 760 sources runs in one round of blocks rather than two.
+// Five blocks per SM (96 registers): a colour class of up to 760 sources runs
+// in one round of blocks rather than two.
 __global__ void __launch_bounds__(kTrThreads, 5) source_step_kernel(PlanView v,
                                                                     const ModelDev* __restrict__ model,
-                                                                    double* delta, int32_t* status) {
+                                                                    const double* delta, int32_t* status,
+                                                                    int n_sm) {
   extern __shared__ double smd[];
   StepSmem& S = *reinterpret_cast<StepSmem*>(smd);
   const int j = blockIdx.x;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int tid = rotated_tid(n_sm), lane = tid & 31, wid = tid >> 5;
   if (!v.active[j]) return;
-  epilogue_source<2>(v, model, S.e, j, nullptr, v.elbo_rel, v.grad, v.hess, 0);
-  __syncthreads();
-  if (!tr_step_source(v, S.t, j, delta, status)) return;
+  const int src = v.src_ids[j], n_color = model->n_color;
+  const double Dl = delta[src];
+  if (tid < kTheta) S.e.th[tid] = (real)v.theta[(size_t)src * kTheta + tid];
+  stage_model(S.f, model, tid, kTrThreads);
+  double rel, full;
+  epilogue_source<2>(v, S.f, n_color, S.e, j, tid, false, rel, full);
+  // the Hessian (symmetric to the last bit: every term is formed once and
+  // mirrored) and gradient, held in registers while the trust-region stage
+  // takes over the shared memory
+  constexpr int kH = (kTheta * kTheta + kTrThreads - 1) / kTrThreads;
+  float h[kH];
+  int bad = 0;
+#pragma unroll
+  for (int m = 0; m < kH; ++m) {
+    const int e = tid + m * kTrThreads;
+    h[m] = e < kTheta * kTheta ? S.e.Hth[e] : 0.f;
+    bad |= !isfinite(h[m]);
+  }
+  const float g = tid < kTheta ? S.e.gth[tid] : 0.f;
+  bad |= !isfinite(g);
+  bad = __syncthreads_or(bad);
+  if (tid == 0) {
+    v.elbo_rel[j] = rel;
+    if (bad || !isfinite(full)) set_error(v.err, CELESTE_DERR_NONFINITE);
+  }
+  if (bad || !isfinite(rel)) {
+    if (tid == 0) {
+      status[src] = CELESTE_ST_FAILED;
+      v.active[j] = 0;
+    }
+    return;
+  }
+#pragma unroll
+  for (int m = 0; m < kH; ++m) {
+    const int e = tid + m * kTrThreads;
+    if (e < kTheta * kTheta) {
+      S.t.B[e] = -(double)h[m];
+      S.t.ws.f.Bf[e] = -h[m];
+    }
+  }
+  if (tid < kTheta) {
+    S.t.gh[tid] = (double)g;
+    S.t.gfr[tid] = g;
+  }
+  if (!tr_step_source(v, S.t, j, src, Dl, rel, status, tid)) return;
   if (wid == 0) {
     if (lane < kTheta) S.e.th[lane] = (real)v.theta_trial[(size_t)j * kTheta + lane];
     __syncwarp();
-    kl_terms<0>(S.e.th, model, S.e, lane);
+    kl_terms<0, false>(S.e.th, S.f, n_color, S.e, lane);
     if (lane == 0) v.kl_trial[j] = (double)S.e.kls[0];
   } else {
     // each warp's 64 floats of the Hessian scratch, which KL_s does not use
@@ -89,7 +135,8 @@ cudaError_t launch_source_step(const Launch& L, const PlanView& v, const ModelDe
                                 (int)sizeof(StepSmem));
   });
   if (e != cudaSuccess) return e;
-  source_step_kernel<<<v.n, kTrThreads, sizeof(StepSmem), L.stream>>>(v, model, delta, status);
+  source_step_kernel<<<v.n, kTrThreads, sizeof(StepSmem), L.stream>>>(v, model, delta, status,
+                                                                       L.sm_count);
   return cudaGetLastError();
 }
 

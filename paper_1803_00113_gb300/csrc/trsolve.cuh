@@ -45,21 +45,20 @@ constexpr int kTri = N * (N + 1) / 2;                        // 378 lower entrie
 
 struct TrSmem {
   double B[N * N];
-  // mixed-precision path.  The FP32 reduction (Bf), then locate32's
+  // mixed-precision path.  The FP32 copy of B (Bf), then locate32's
   // per-thread elimination factors (cps, gps: [i][thread]), then the FP64
   // factorisations (W, L) use the same memory in turn.
   union Work {
     struct Fp64 {
       double W[N * N];             // factorisation work copy of B + l I
       double L[N * N];             // unit lower factor of B + l I (strict lower part)
-      float Bf[N * N];             // FP32 copy of B, reduced to tridiagonal form
+      float Bf[N * N];             // FP32 copy of B
     } f;
     struct Sec {
       float cps[N * kTrThreads], gps[N * kTrThreads];
     } s;
   } ws;
   double Dinv[32];                 // 1 / D
-  double col[2][32];               // published pivot column, double-buffered
   double p[32];
   double lam, lo, hi;              // multiplier and its bracket (unscaled)
   double lmin_lo;                  // lower bound of lambda_min (unscaled, FP32 accuracy)
@@ -70,7 +69,6 @@ struct TrSmem {
   float betaf[32], dfr[32], efr[32], gfr[32];
   float loc[4];                    // locate32: scale, |g|^2 (scaled), |p(0)|^2
   unsigned hmask[2][4];            // locate32: probe ballots of the four warps
-  short2 tri[kTri];                // lower entry e -> (row, column)
   int mode;                        // 0 interior candidate, 1 boundary, 2 full FP64 path
   double beta[32];
   double gh[32];
@@ -83,7 +81,8 @@ struct TrSmem {
   double part[4 * 32];
   double red[8];
   float df[32], ef[32], e2f[32], gf[32];
-  float hps[32], hred[8];          // block Householder: p per row, per-warp sums
+  float hxs[32], hsq[32], hps[32], hred[8];   // block Householder: pivot column and its
+                                              // squares below the pivot, p per row, sums
   int skip[32];                    // per Householder step: column already reduced
 };
 
@@ -109,14 +108,25 @@ static __device__ __forceinline__ int sturm32(const float (&d)[N], const float (
   return cnt;
 }
 
+// 1 / x by the reciprocal instruction alone: __fdividef(1, x) for |x| in
+// (1e-30, 1e30) (and a * rcp32(x) its a / x, where that is normal: equal to
+// the last bit for every x of that range), without its range scaling, which
+// lengthens the chains below by a third.
+static __device__ __forceinline__ float rcp32(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // The same count reading d and e2 from shared memory (broadcast loads).
 static __device__ __forceinline__ int sturm32s(const float* d, const float* e2, float sigma) {
   int cnt = 0;
   float q = d[0] - sigma;
   cnt += q < 0.f;
+#pragma unroll
   for (int i = 1; i < N; ++i) {
     const float qp = q == 0.f ? 1e-30f : q;
-    q = (d[i] - sigma) - __fdividef(e2[i - 1], qp);
+    q = (d[i] - sigma) - e2[i - 1] * rcp32(qp);
     cnt += q < 0.f;
   }
   return cnt;
@@ -166,22 +176,24 @@ static __device__ __noinline__ float norm2_32(const float* d, const float* e, co
 
 // |y|^2 for (T + lam I) y = g in FP32 with the per-thread elimination
 // factors in shared memory (cps, gps: [i][thread] layout, the thread's column).
-static __device__ float norm2_32s(const float* d, const float* e, const float* g, float lam, float* cps,
+static __device__ __noinline__ float norm2_32s(const float* d, const float* e, const float* g, float lam, float* cps,
                            float* gps) {
   float m = d[0] + lam;
-  float r = __fdividef(1.f, m);
+  float r = rcp32(m);
   float c = e[0] * r, gp = g[0] * r;
   cps[0] = c;
   gps[0] = gp;
+#pragma unroll
   for (int i = 1; i < N; ++i) {
     m = (d[i] + lam) - e[i - 1] * c;
-    r = __fdividef(1.f, m);
+    r = rcp32(m);
     c = i < N - 1 ? e[i] * r : 0.f;
     gp = (g[i] - e[i - 1] * gp) * r;
     cps[i * kTrThreads] = c;
     gps[i * kTrThreads] = gp;
   }
   float y = gp, sum = y * y;
+#pragma unroll
   for (int i = N - 2; i >= 0; --i) {
     y = gps[i * kTrThreads] - cps[i * kTrThreads] * y;
     sum += y * y;
@@ -245,16 +257,9 @@ static __device__ void apply_q(TrSmem& S, double* x, bool transpose, int lane) {
 // Exact trust-region subproblem of one source, all in FP64 (the path for
 // the hard and nearly hard cases); 128 threads (4 warps) enter, warp 0
 // finishes: it returns true and holds p in S.y and the predicted gain in
-// S.red[0].  g (27) and H (27 x 27) are in global memory.
-static __device__ bool tr_solve_full(TrSmem& S, const double* __restrict__ g,
-                              const double* __restrict__ H, double Delta) {
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  for (int e = tid; e < N * N; e += kTrThreads) {
-    const int i = e / N, j = e % N;
-    S.B[e] = -0.5 * (H[i * N + j] + H[j * N + i]);
-  }
-  if (tid < N) S.gh[tid] = g[tid];
-  __syncthreads();
+// S.red[0].  B = -H is in S.B and g in S.gh (both are overwritten).
+static __device__ bool tr_solve_full(TrSmem& S, double Delta, int tid) {
+  const int lane = tid & 31, wid = tid >> 5;
   // ---- Householder tridiagonalisation; v_k stored below the diagonal of column k
   for (int k = 0; k < N - 2; ++k) {
     const int m = N - 1 - k;
@@ -536,120 +541,167 @@ static __device__ __forceinline__ double rcp64_any(double x) {
   return ldexp(r, -ex);
 }
 
-static __device__ __forceinline__ double B_diag0(const TrSmem& S, double lam) { return S.B[0] + lam; }
+// FP64 <-> FP32 conversions of positive normal values on the integer pipe
+// (an FP64-pipe conversion takes ~65 cycles of the sub-partition): to FP32
+// with round to nearest even, for values whose FP32 form is normal; to FP64
+// exactly.
+static __device__ __forceinline__ float f32_of(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned q = ((hi - ((1023u - 127u) << 20)) << 3) | (lo >> 29), rem = lo << 3;
+  return __uint_as_float(q + (rem > 0x80000000u || (rem == 0x80000000u && (q & 1u)) ? 1u : 0u));
+}
+static __device__ __forceinline__ double f64_of(float x) {
+  const unsigned b = __float_as_uint(x);
+  return __hiloint2double((int)((b >> 3) + ((1023u - 127u) << 20)), (int)(b << 29));
+}
 
 // 1/d in FP64 from an FP32 seed and one Newton step (relative error
 // ~1e-14) when d is inside the FP32 range; 0 when d is not a positive
-// finite pivot.
+// finite pivot.  (The range tests compare bits: an FP64 comparison takes the
+// FP64 pipe.)
 static __device__ __forceinline__ double pivot_rcp(double d) {
-  if (!(d > 0.0 && d < 1e300)) return 0.0;
-  if (d > 1e-30 && d < 1e30) {
-    const double r = (double)__fdividef(1.f, (float)d);   // ~1e-7 seed
-    return fma(r, fma(-d, r, 1.0), r);                     // one Newton step: ~1e-14
+  const long long b = __double_as_longlong(d);
+  if (b > __double_as_longlong(1e-30) && b < __double_as_longlong(1e30)) {
+    const double r = f64_of(rcp32(f32_of(d)));             // ~1e-7 seed
+    return fma(r, fma(-d, r, 1.0), r);                      // one Newton step: ~1e-14
   }
+  if (!(d > 0.0 && d < 1e300)) return 0.0;
   return rcp64_any(d);
 }
 
-// LDL^T of B + lam I in FP64 with all 128 threads, right-looking, one
-// barrier per column: the m(m+1)/2 entries of the trailing triangle are
-// spread evenly over the threads, each updated with the column's inverse
-// pivot applied on the fly; thread 0, which updates the next diagonal entry
-// first, takes its reciprocal right away.  The columns of L are scaled at
-// the end.  Returns false (the same on every thread) when a pivot is not
-// positive.  On success S.ws.f.L holds the unit lower factor (strictly
-// lower part) and S.Dinv the inverse pivots.  S.ws.f.W is the working copy.
-static __device__ bool ldl_factor(TrSmem& S, double lam) {
-  const int tid = threadIdx.x;
-  for (int e = tid; e < kTri; e += kTrThreads) {
-    const short2 t = S.tri[e];
-    S.ws.f.W[t.x * N + t.y] = S.B[t.x * N + t.y] + (t.x == t.y ? lam : 0.0);
+// Entries of a trailing triangle that warps 1..3 update: thread u takes
+// u + 1, u + 97, ... (entry 0 is the pivot), as (row, column).
+constexpr int kLdlThreads = kTrThreads - 32;
+constexpr int kLdlRounds = (kTri - N + kLdlThreads - 1) / kLdlThreads;   // 351 entries at first
+static __device__ __forceinline__ void ldl_entries(short2 (&rc)[kLdlRounds], int tid) {
+#pragma unroll
+  for (int m = 0; m < kLdlRounds; ++m) {
+    const int e = max(tid - 32, 0) + 1 + m * kLdlThreads;
+    // row i of lower entry e: i (i + 1) / 2 <= e < (i + 1) (i + 2) / 2
+    int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+    if (i * (i + 1) / 2 > e) --i;
+    if ((i + 1) * (i + 2) / 2 <= e) ++i;
+    rc[m] = make_short2((short)i, (short)(e - i * (i + 1) / 2));
   }
-  if (tid == 0) S.Dinv[0] = pivot_rcp(B_diag0(S, lam));
-  if (__syncthreads_or(tid == 0 && S.Dinv[0] == 0.0)) return false;
-  for (int j = 0; j < N - 1; ++j) {
-    const int m = N - 1 - j;
-    const int cnt = m * (m + 1) / 2;
-    const double dinv = S.Dinv[j];
-    int bad = 0;
-    for (int e = tid; e < cnt; e += kTrThreads) {
-      const short2 t = S.tri[e];                  // (row, col) in the trailing block
-      const int i = j + 1 + t.x, k = j + 1 + t.y;
-      const double w = fma(-(S.ws.f.W[i * N + j] * dinv), S.ws.f.W[k * N + j], S.ws.f.W[i * N + k]);
-      S.ws.f.W[i * N + k] = w;
-      if (e == 0) {                               // the next pivot
-        const double r = pivot_rcp(w);
-        S.Dinv[j + 1] = r;
-        bad = r == 0.0;
-      }
-    }
-    if (__syncthreads_or(bad)) return false;
-  }
-  for (int e = tid; e < kTri; e += kTrThreads) {
-    const short2 t = S.tri[e];
-    if (t.x > t.y) S.ws.f.L[t.x * N + t.y] = S.ws.f.W[t.x * N + t.y] * S.Dinv[t.y];
-  }
-  __syncthreads();
-  return true;
 }
 
-// Warp 0: p = (L D L^T)^{-1} rhs into out; returns |p|^2, and in *q2 (when
-// non-null) p^T (L D L^T)^{-1} p.  Rows live on lanes; each elimination step
-// broadcasts one solved entry.
-static __device__ double ldl_solve_full(TrSmem& S, const double* rhs, double* out, int lane,
-                                 double* q2) {
-  double b = lane < N ? rhs[lane] : 0.0;
-  for (int k = 0; k < N - 1; ++k) {
-    const double wk = __shfl_sync(0xffffffffu, b, k);
-    if (lane > k && lane < N) b = fma(-S.ws.f.L[lane * N + k], wk, b);
+// LDL^T of B + lam I in FP64 with all 128 threads, right-looking, one
+// barrier per column.  Bound by the chain of pivots (a product, an FMA and a
+// reciprocal each, ~5 FP64 instructions of ~65 cycles): warp 0 does nothing
+// else, one column ahead, while warps 1..3 spread the trailing triangle
+// evenly over their threads, with the column and its multiples (each
+// formed once, by the lane of its row) passed by shuffles.  17.5k cycles, 34.8k
+// with one entry's product and FMA after the other and FP64 comparisons of
+// the pivot.  Returns false
+// (the same on every thread) when a pivot is not positive.  On success
+// S.ws.f.L holds the unit lower factor (strictly lower part) and S.Dinv the
+// inverse pivots.  S.ws.f.W is the working copy.
+static __device__ bool ldl_factor(TrSmem& S, double lam, const short2 (&rc)[kLdlRounds], int tid) {
+  const int lane = tid & 31, wid = tid >> 5;
+  double* W = S.ws.f.W;
+  for (int e = tid; e < N * N; e += kTrThreads)
+    if (e % (N + 1) != 0) W[e] = S.B[e];
+  if (tid < N) W[tid * N + tid] = S.B[tid * N + tid] + lam;
+  double dinv = 0.0;
+  bool ok = true;
+  if (wid == 0) {
+    dinv = pivot_rcp(S.B[0] + lam);
+    if (lane == 0) S.Dinv[0] = dinv;
+    ok = dinv != 0.0;
   }
-  double z = lane < N ? b * S.Dinv[lane] : 0.0;
-  for (int k = N - 1; k > 0; --k) {
-    const double pk = __shfl_sync(0xffffffffu, z, k);
-    if (lane < k) z = fma(-S.ws.f.L[k * N + lane], pk, z);
-  }
-  if (lane < N) out[lane] = z;
-  const double n2 = warp_sum_d(z * z);
-  if (q2) {
-    double u = z;
-    for (int k = 0; k < N - 1; ++k) {
-      const double uk = __shfl_sync(0xffffffffu, u, k);
-      if (lane > k && lane < N) u = fma(-S.ws.f.L[lane * N + k], uk, u);
+  __syncthreads();
+  double* Wj = W + N + 1;                       // W[j + 1][j + 1]
+  for (int j = 0; j < N - 1; ++j, Wj += N + 1) {
+    if (wid == 0) {
+      const double a = Wj[-1];
+      const double d = fma(-(a * dinv), a, Wj[0]);
+      dinv = pivot_rcp(d);
+      if (lane == 0) S.Dinv[j + 1] = dinv;
+      ok &= __double_as_longlong(dinv) != 0;
+    } else {
+      const int m = N - 1 - j, cnt = m * (m + 1) / 2;
+      const double x = lane < m ? Wj[lane * N - 1] : 0.0;
+      const double l = x * S.Dinv[j];
+      if (wid == 1 && lane < m) S.ws.f.L[(j + 1 + lane) * N + j] = l;
+      const int e0 = tid - 32 + 1;
+      double w[kLdlRounds], lr[kLdlRounds], xc[kLdlRounds];
+      // (loads and shuffles of every round first; a warp leaves out the
+      // rounds that hold none of its entries)
+#pragma unroll
+      for (int r = 0; r < kLdlRounds; ++r) {
+        w[r] = Wj[e0 + r * kLdlThreads < cnt ? rc[r].x * N + rc[r].y : 0];
+        xc[r] = __shfl_sync(0xffffffffu, x, rc[r].y);
+        lr[r] = __shfl_sync(0xffffffffu, l, rc[r].x);
+      }
+#pragma unroll
+      for (int r = 0; r < kLdlRounds; ++r) {
+        if (e0 - lane + r * kLdlThreads < cnt) {
+          const double y = fma(-lr[r], xc[r], w[r]);
+          if (e0 + r * kLdlThreads < cnt) Wj[rc[r].x * N + rc[r].y] = y;
+        }
+      }
     }
-    *q2 = warp_sum_d(lane < N ? u * u * S.Dinv[lane] : 0.0);
-    if (lane < N) S.z[lane] = u;        // u = L^{-1} p, for first_order()
+    __syncthreads();
   }
+  // (a pivot that is not positive leaves zeros and a factor nobody reads)
+  return !__syncthreads_or(!ok);
+}
+
+// Warp 0: p = (L D L^T)^{-1} rhs into out; returns |p|^2.  Rows live on
+// lanes; each elimination step broadcasts one solved entry.
+static __device__ __noinline__ double back_sweep(const TrSmem& S, double z, int lane);
+static __device__ __noinline__ double fwd_sweep(const TrSmem& S, double b, int lane);
+static __device__ double ldl_solve_full(TrSmem& S, const double* rhs, double* out, int lane) {
+  const double b = fwd_sweep(S, lane < N ? rhs[lane] : 0.0, lane);
+  const double z = back_sweep(S, lane < N ? b * S.Dinv[lane] : 0.0, lane);
+  if (lane < N) out[lane] = z;
   __syncwarp();
-  return n2;
+  return warp_sum_d(z * z);
+}
+
+// Warp 0: p^T (L D L^T)^{-1} p for the p of ldl_solve_full; u = L^{-1} p
+// into S.z.
+static __device__ double ldl_curvature(TrSmem& S, const double* p, int lane) {
+  const double u = fwd_sweep(S, lane < N ? p[lane] : 0.0, lane);
+  if (lane < N) S.z[lane] = u;
+  __syncwarp();
+  return warp_sum_d(lane < N ? u * u * S.Dinv[lane] : 0.0);
 }
 
 // Warp 0: p(l + dl) = p(l) - dl (B + l I)^{-1} p(l) to first order, with
-// (B + l I)^{-1} p = L^{-T} D^{-1} u and u = L^{-1} p kept by ldl_solve_full.
+// (B + l I)^{-1} p = L^{-T} D^{-1} u and u = L^{-1} p kept by ldl_curvature.
 static __device__ void first_order(TrSmem& S, int lane, double dl) {
-  double z = lane < N ? S.z[lane] * S.Dinv[lane] : 0.0;
-  for (int k = N - 1; k > 0; --k) {
-    const double qk = __shfl_sync(0xffffffffu, z, k);
-    if (lane < k) z = fma(-S.ws.f.L[k * N + lane], qk, z);
-  }
+  const double z = back_sweep(S, lane < N ? S.z[lane] * S.Dinv[lane] : 0.0, lane);
   if (lane < N) S.p[lane] = fma(-dl, z, S.p[lane]);
   __syncwarp();
 }
 
-// Warp 0: x = L^{-T} z (rows on lanes).
-static __device__ __forceinline__ double back_sweep(const TrSmem& S, double z, int lane) {
+// Warp 0: x = L^{-T} z (rows on lanes); each elimination step broadcasts one
+// solved entry.  The lane's column of L is loaded ahead, so that a step is
+// its FMA and shuffle (~100 cycles).
+static __device__ __noinline__ double back_sweep(const TrSmem& S, double z, int lane) {
+  double l[N];
+#pragma unroll
+  for (int k = N - 1; k > 0; --k) l[k] = S.ws.f.L[k * N + min(lane, N - 1)];
+#pragma unroll
   for (int k = N - 1; k > 0; --k) {
     const double xk = __shfl_sync(0xffffffffu, z, k);
-    if (lane < k) z = fma(-S.ws.f.L[k * N + lane], xk, z);
+    if (lane < k) z = fma(-l[k], xk, z);
   }
   return z;
 }
 
-// Warp 0: x = (L D L^T)^{-1} b.
-static __device__ __forceinline__ double full_solve(const TrSmem& S, double b, int lane) {
+// Warp 0: x = L^{-1} b.
+static __device__ __noinline__ double fwd_sweep(const TrSmem& S, double b, int lane) {
+  double l[N];
+#pragma unroll
+  for (int k = 0; k < N - 1; ++k) l[k] = S.ws.f.L[min(lane, N - 1) * N + k];
+#pragma unroll
   for (int k = 0; k < N - 1; ++k) {
     const double bk = __shfl_sync(0xffffffffu, b, k);
-    if (lane > k && lane < N) b = fma(-S.ws.f.L[lane * N + k], bk, b);
+    if (lane > k && lane < N) b = fma(-l[k], bk, b);
   }
-  return back_sweep(S, lane < N ? b * S.Dinv[lane] : 0.0, lane);
+  return b;
 }
 
 // Warp 0: the step at the multiplier l0 + d with |p(l0 + d)| = Delta, from
@@ -659,34 +711,85 @@ static __device__ __forceinline__ double full_solve(const TrSmem& S, double b, i
 // pole) and A(d)^{-1} p(l0 + d) = sum_n (n + 1) (-d)^n w_{n+1}; Newton's
 // iteration on 1/|p| - 1/Delta (Nocedal & Wright, Algorithm 4.3) then runs
 // on the scalars of the Gram matrix w_i . w_j.  On entry S.p = p(l0) and
-// S.z = L^{-1} p(l0) (from ldl_solve_full); d0 is the first Newton step.
+// S.z = L^{-1} p(l0) (from ldl_curvature); d0 is the first Newton step.
 // On exit S.p is the step.
+//
+// FP64 instructions are what it costs, whatever their lanes do: the ten dot
+// products share their shuffle trees (a step of two sums in the two halves
+// of the lanes), and an iteration's two polynomials run side by side, one in
+// each half of the warp.  32k cycles (35k with one at a time), half of them
+// the five triangular sweeps.
 static __device__ void series_finish(TrSmem& S, int lane, double d0, double Delta) {
   constexpr int K = 3;
+  constexpr int kG = (K + 1) * (K + 2) / 2;   // 10 products w_i . w_j, i <= j
   double w[K + 1];
   w[0] = lane < N ? S.p[lane] : 0.0;
   w[1] = back_sweep(S, lane < N ? S.z[lane] * S.Dinv[lane] : 0.0, lane);
+#pragma unroll 1
+  for (int k = 2; k <= K; ++k) {
+    const double b = fwd_sweep(S, k == 2 ? w[1] : w[2], lane);
+    const double x = back_sweep(S, lane < N ? b * S.Dinv[lane] : 0.0, lane);
+    if (k == 2) w[2] = x;
+    else w[3] = x;
+  }
+  // sums q and q + 1 of level o: lanes with bit o clear keep q, the others
+  // q + 1; each adds its partner's half (the tree of warp_sum_d)
+  double r[kG + 2];
+  {
+    int q = 0;
 #pragma unroll
-  for (int k = 2; k <= K; ++k) w[k] = full_solve(S, w[k - 1], lane);
-  double G[K + 1][K + 1];
+    for (int i = 0; i <= K; ++i)
 #pragma unroll
-  for (int i = 0; i <= K; ++i)
+      for (int j = i; j <= K; ++j) r[q++] = w[i] * w[j];
+    r[kG] = r[kG + 1] = 0.0;
+  }
+  int n = kG;
 #pragma unroll
-    for (int j = i; j <= K; ++j) G[i][j] = G[j][i] = warp_sum_d(w[i] * w[j]);
+  for (int o = 16; o >= 2; o >>= 1) {
+    const bool up = (lane & o) != 0;
+    const int half = (n + 1) / 2;
+#pragma unroll
+    for (int q = 0; q < half; ++q) {
+      const double lo = r[2 * q], hi = 2 * q + 1 < n ? r[2 * q + 1] : lo;
+      const double give = up ? lo : hi, keep = up ? hi : lo;
+      r[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+    n = half;
+  }
+  r[0] += __shfl_xor_sync(0xffffffffu, r[0], 1);
+  // sum q of the ten is in lanes with bits 4, 3, 2, 1 = bits 0, 1, 2, 3 of q
+  if (!(lane & 1)) {
+    const int q = (lane >> 4 & 1) | (lane >> 2 & 2) | (lane & 4) | (lane << 2 & 8);
+    if (q < kG) S.part[q] = r[0];
+  }
+  __syncwarp();
+  // lanes 0..15 hold the terms of |p|^2 = sum c_i c_j G_ij, lanes 16..27
+  // those of q = sum c_i (n + 1) c_n G_i,n+1
+  const int t = lane & 15;
+  const bool second = lane >= 16;
+  const int ti = second ? min(t / K, K) : t / (K + 1), tn = second ? t % K : t % (K + 1);
+  const int tj = second ? tn + 1 : tn;
+  const int gi = min(ti, tj), gj = max(ti, tj);
+  const double gt = S.part[gi * (K + 1) - gi * (gi - 1) / 2 + gj - gi];
+  const double wt = second ? (double)(tn + 1) : 1.0;
   double d = d0;
   double c[K + 1];
   for (int it = 0; it < 8; ++it) {
     c[0] = 1.0;
 #pragma unroll
     for (int k = 1; k <= K; ++k) c[k] = -d * c[k - 1];
-    double n2 = 0.0, q = 0.0;
+    const double ci = ti == 0 ? c[0] : (ti == 1 ? c[1] : (ti == 2 ? c[2] : c[3]));
+    const double cn = tn == 0 ? c[0] : (tn == 1 ? c[1] : (tn == 2 ? c[2] : c[3]));
+    const double pt = ci * wt * cn;
+    double acc = 0.0;
 #pragma unroll
-    for (int i = 0; i <= K; ++i) {
-#pragma unroll
-      for (int j = 0; j <= K; ++j) n2 = fma(c[i] * c[j], G[i][j], n2);
-#pragma unroll
-      for (int n = 0; n < K; ++n) q = fma(c[i] * (double)(n + 1) * c[n], G[i][n + 1], q);
+    for (int e = 0; e < (K + 1) * (K + 1); ++e) {
+      const double pe = __shfl_sync(0xffffffffu, pt, (lane & 16) + e);
+      const double ge = __shfl_sync(0xffffffffu, gt, (lane & 16) + e);
+      const double a = fma(pe, ge, acc);
+      if (!second || e < K * (K + 1)) acc = a;
     }
+    const double n2 = __shfl_sync(0xffffffffu, acc, 0), q = __shfl_sync(0xffffffffu, acc, 16);
     const double step = (sqrt(n2) - Delta) / Delta * n2 / q;
     d += step;
     if (!(fabs(step) > 1e-15 * fabs(d))) break;
@@ -701,89 +804,119 @@ static __device__ void series_finish(TrSmem& S, int lane, double d0, double Delt
   __syncwarp();
 }
 
-// Householder reduction of B (FP32, in S.ws.f.Bf) to tridiagonal form by all
-// four warps: thread t owns row t / 4 of the trailing block and, in it, the
-// columns c = t (mod 4); two block barriers per reflection.  Every warp
-// reduces the pivot column itself (rows on lanes, the same shuffle tree in
-// each), so all threads take the same branch.  The reflections are applied
-// to g as they are made.  d, e into S.dfr, S.efr; Q^T g into S.gfr.
-static __device__ void householder_blk(TrSmem& S) {
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+// Householder reduction of B (FP32 copy in S.ws.f.Bf) to tridiagonal form by
+// all four warps: thread t holds, in registers, row t / 4 of the matrix at
+// the columns c = t (mod 4); the pivot column and p = bt B v pass through
+// shared memory, with two block barriers per reflection.  Every warp reduces
+// the pivot column itself (rows on lanes, the same shuffle tree in each), so
+// all threads take the same branch.  The reflections are applied to g as
+// they are made.  d, e into S.dfr, S.efr; Q^T g into S.gfr.  Bound by its
+// dependent shuffles, barriers and short instruction chains: 21k cycles (32k
+// with the matrix in shared memory).
+static __device__ void householder_blk(TrSmem& S, int tid) {
+  constexpr int kCols = (N + 3) / 4;
+  const int lane = tid & 31, wid = tid >> 5;
   const int i = tid >> 2, sub = tid & 3;
-  float* Bf = S.ws.f.Bf;
+  float r[kCols];
+#pragma unroll
+  for (int m = 0; m < kCols; ++m)
+    r[m] = i < N && sub + 4 * m < N ? S.ws.f.Bf[i * N + sub + 4 * m] : 0.f;
   float gi = i < N ? S.gfr[i] : 0.f;
-  for (int k = 0; k < N - 2; ++k) {
-    const float xl = (lane > k && lane < N) ? Bf[lane * N + k] : 0.f;
-    float nrm2 = xl * xl;
+  if (sub == 0) {
+    S.hxs[i] = r[0];
+    S.hsq[i] = i > 0 ? r[0] * r[0] : 0.f;
+  }
+  __syncthreads();
+  // columns up to 4 m0 - 1 are done in phase m0: the phases are unrolled, so
+  // that a thread touches only the registers of columns still in the block
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) nrm2 += __shfl_xor_sync(0xffffffffu, nrm2, o);
-    const float x0 = Bf[(k + 1) * N + k];
-    if (tid == 0) S.dfr[k] = Bf[k * N + k];
-    if (!(nrm2 - x0 * x0 > 1e-30f * fmaxf(nrm2, 1e-30f))) {
+  for (int m0 = 0; m0 < kCols; ++m0)
+#pragma unroll 1
+  for (int k = 4 * m0; k < min(4 * m0 + 4, N - 2); ++k) {
+    // the sum over the rows in the order of a butterfly over lanes (xor 16,
+    // 8, 4, 2, 1): its first three levels from shared memory
+    float q[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) q[t] = S.hsq[lane ^ (4 * t)];
+    float nrm2 = ((q[0] + q[4]) + (q[2] + q[6])) + ((q[1] + q[5]) + (q[3] + q[7]));
+#pragma unroll
+    for (int o = 2; o > 0; o >>= 1) nrm2 += __shfl_xor_sync(0xffffffffu, nrm2, o);
+    const float x0 = S.hxs[k + 1];
+    if (tid == 0) S.dfr[k] = S.hxs[k];
+    const bool skip = !(nrm2 - x0 * x0 > 1e-30f * fmaxf(nrm2, 1e-30f));
+    if (skip) {
       if (tid == 0) S.efr[k] = x0;
-      continue;
-    }
-    const float alpha = -copysignf(sqrtf(nrm2), x0);
-    const float bt = __fdividef(1.f, fmaf(-x0, alpha, nrm2));
-    if (tid == 0) S.efr[k] = alpha;
-    const bool row = i > k && i < N;
-    // reflector v_c = B[c][k] - alpha [c == k + 1], c > k (column k is not
-    // written during this reflection)
-    auto vof = [&](int c) { return Bf[c * N + k] - (c == k + 1 ? alpha : 0.f); };
-    const float vi = row ? vof(i) : 0.f;
-    const int c0 = k + 1 + ((sub - (k + 1)) & 3);   // first c > k with c = sub (mod 4)
-    // p = bt B v over the trailing block: this thread's columns, then the row
-    float pp = 0.f;
-    if (row) {
-      const float* r = Bf + i * N;
-      for (int c = c0; c < N; c += 4) pp = fmaf(r[c], vof(c), pp);
-    }
-    pp += __shfl_xor_sync(0xffffffffu, pp, 1);
-    pp += __shfl_xor_sync(0xffffffffu, pp, 2);
-    const float p = row ? bt * pp : 0.f;
-    // K = v.p and v.g over the rows (row values on sub 0), then the warps
-    float K = sub == 0 ? vi * p : 0.f, vg = sub == 0 ? vi * gi : 0.f;
+      __syncthreads();
+    } else {
+      const float alpha = -copysignf(sqrtf(nrm2), x0);
+      const float bt = __fdividef(1.f, fmaf(-x0, alpha, nrm2));
+      if (tid == 0) S.efr[k] = alpha;
+      const bool row = i > k && i < N;
+      // reflector v_c = B[c][k] - alpha [c == k + 1], c > k
+      const float vi = row ? S.hxs[i] - (i == k + 1 ? alpha : 0.f) : 0.f;
+      float vc[kCols];
+      // p = bt B v over the trailing block: this thread's columns, then the row
+      float pp = 0.f;
 #pragma unroll
-    for (int o = 16; o >= 4; o >>= 1) {
-      K += __shfl_xor_sync(0xffffffffu, K, o);
-      vg += __shfl_xor_sync(0xffffffffu, vg, o);
-    }
-    if (lane == 0) {
-      S.hred[wid] = K;
-      S.hred[4 + wid] = vg;
-    }
-    if (sub == 0 && row) S.hps[i] = p;
-    __syncthreads();
-    K = (S.hred[0] + S.hred[1]) + (S.hred[2] + S.hred[3]);
-    vg = (S.hred[4] + S.hred[5]) + (S.hred[6] + S.hred[7]);
-    gi = fmaf(-bt * vg, vi, gi);                  // g -= bt v (v.g)
-    // B -= v w^T + w v^T with w = p - (bt K / 2) v
-    const float hk = -0.5f * bt * K;
-    if (row) {
+      for (int m = m0; m < kCols; ++m) {
+        const int c = sub + 4 * m;
+        vc[m] = c < N ? S.hxs[c] - (c == k + 1 ? alpha : 0.f) : 0.f;
+        if ((m > m0 || c > k) && c < N && row) pp = fmaf(r[m], vc[m], pp);
+      }
+      pp += __shfl_xor_sync(0xffffffffu, pp, 1);
+      pp += __shfl_xor_sync(0xffffffffu, pp, 2);
+      const float p = row ? bt * pp : 0.f;
+      // K = v.p and v.g over the rows (row values on sub 0), then the warps
+      float K = sub == 0 ? vi * p : 0.f, vg = sub == 0 ? vi * gi : 0.f;
+#pragma unroll
+      for (int o = 16; o >= 4; o >>= 1) {
+        K += __shfl_xor_sync(0xffffffffu, K, o);
+        vg += __shfl_xor_sync(0xffffffffu, vg, o);
+      }
+      if (lane == 0) {
+        S.hred[wid] = K;
+        S.hred[4 + wid] = vg;
+      }
+      if (sub == 0 && row) S.hps[i] = p;
+      __syncthreads();
+      K = (S.hred[0] + S.hred[1]) + (S.hred[2] + S.hred[3]);
+      vg = (S.hred[4] + S.hred[5]) + (S.hred[6] + S.hred[7]);
+      gi = fmaf(-bt * vg, vi, gi);                  // g -= bt v (v.g)
+      // B -= v w^T + w v^T with w = p - (bt K / 2) v
+      const float hk = -0.5f * bt * K;
       const float wi = fmaf(hk, vi, p);
-      float* r = Bf + i * N;
-      for (int c = c0; c < N; c += 4) {
-        const float vc = vof(c);
-        const float wc = fmaf(hk, vc, S.hps[c]);
-        r[c] = fmaf(-vi, wc, fmaf(-wi, vc, r[c]));
+#pragma unroll
+      for (int m = m0; m < kCols; ++m) {
+        const int c = sub + 4 * m;
+        if ((m > m0 || c > k) && c < N && row) {
+          const float wc = fmaf(hk, vc[m], S.hps[c]);
+          r[m] = fmaf(-vi, wc, fmaf(-wi, vc[m], r[m]));
+        }
       }
     }
+    // the next pivot column
+#pragma unroll
+    for (int m = m0; m < min(m0 + 2, kCols); ++m)
+      if (sub + 4 * m == k + 1) {
+        S.hxs[i] = r[m];
+        S.hsq[i] = i > k + 1 && i < N ? r[m] * r[m] : 0.f;
+      }
     __syncthreads();
   }
   if (tid == 0) {
-    S.dfr[N - 2] = Bf[(N - 2) * N + N - 2];
-    S.dfr[N - 1] = Bf[(N - 1) * N + N - 1];
-    S.efr[N - 2] = Bf[(N - 1) * N + N - 2];
+    S.dfr[N - 2] = S.hxs[N - 2];
+    S.efr[N - 2] = S.hxs[N - 1];
     S.efr[N - 1] = 0.f;
   }
+  if (i == N - 1 && sub == ((N - 1) & 3)) S.dfr[N - 1] = r[(N - 1) / 4];
   if (sub == 0 && i < N) S.gfr[i] = gi;
   __syncthreads();
 }
 
 // The first of the block's 127 probes (threads 0..126) that is set, or 127
 // when none is; one barrier (the ballot slots alternate between rounds).
-static __device__ __forceinline__ int first_hit(TrSmem& S, bool hit, int round) {
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+static __device__ __forceinline__ int first_hit(TrSmem& S, bool hit, int round, int tid) {
+  const int lane = tid & 31, wid = tid >> 5;
   const unsigned m = __ballot_sync(0xffffffffu, hit && tid < kTrThreads - 1);
   if (lane == 0) S.hmask[round & 1][wid] = m;
   __syncthreads();
@@ -798,8 +931,8 @@ static __device__ __forceinline__ int first_hit(TrSmem& S, bool hit, int round) 
 // All four warps: from the FP32 tridiagonal form, lambda_min and the
 // multiplier to FP32 accuracy by multisection, 127 probes a round (7 bits);
 // sets S.mode, S.lam, S.lo, S.hi (unscaled).
-static __device__ void locate32(TrSmem& S, double Delta) {
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+static __device__ void locate32(TrSmem& S, double Delta, int tid) {
+  const int lane = tid & 31, wid = tid >> 5;
   constexpr float kStep = 1.f / (float)kTrThreads;
   if (wid == 0) {
     float rowf = 0.f, g2f = 0.f;
@@ -834,9 +967,10 @@ static __device__ void locate32(TrSmem& S, double Delta) {
   const float D2 = (float)(Delta * Delta);
   int round = 0;
   float fa = -1.f - 1e-6f, fb = 1.f + 1e-6f;
+#pragma unroll 1
   for (int r = 0; r < 4; ++r, ++round) {
     const float sig = fa + (fb - fa) * (float)(tid + 1) * kStep;
-    const int t = first_hit(S, sturm32s(S.df, S.e2f, sig) >= 1, round);
+    const int t = first_hit(S, sturm32s(S.df, S.e2f, sig) >= 1, round, tid);
     const float na = t == 0 ? fa : fa + (fb - fa) * (float)t * kStep;
     const float nb = t == kTrThreads - 1 ? fb : fa + (fb - fa) * (float)(t + 1) * kStep;
     fa = na;
@@ -844,13 +978,25 @@ static __device__ void locate32(TrSmem& S, double Delta) {
   }
   // lambda_min (scaled) lies in [fa, fb] up to FP32 rounding of the counts
   const float lmin = fa;
-  if (tid == 0) S.loc[2] = lmin > 0.f ? norm2_32s(S.df, S.ef, S.gf, 0.f, cps, gps) : 3.4e38f;
-  __syncthreads();
+  // boundary bracket [la, lb]; the first round of its multisection also
+  // evaluates |p(0)| (thread 127, which holds no probe)
+  const float lo = fmaxf(0.f, -lmin);
+  float la = lo, lb = lo + gnorm_s / (float)Delta * 1.01f + 1e-6f;
+  auto secular_round = [&]() {
+    const float l = la + (lb - la) * (float)(tid + 1) * kStep;
+    const float n2 = norm2_32s(S.df, S.ef, S.gf, tid < kTrThreads - 1 ? l : 0.f, cps, gps);
+    if (tid == kTrThreads - 1) S.loc[2] = lmin > 0.f ? n2 : 3.4e38f;
+    const int t = first_hit(S, tid < kTrThreads - 1 && n2 <= D2, round++, tid);
+    const float na = t == 0 ? la : la + (lb - la) * (float)t * kStep;
+    const float nb = t == kTrThreads - 1 ? lb : la + (lb - la) * (float)(t + 1) * kStep;
+    la = na;
+    lb = nb;
+  };
+  secular_round();
   const float n0 = S.loc[2];
   // mode 0: try l = 0 first (interior Newton step); mode 1: the boundary
-  // root from the bracket [la, lb]; mode 2: the all-FP64 path
+  // root from the bracket; mode 2: the all-FP64 path
   int mode = 1;
-  float la = 0.f, lb = 0.f;
   bool bracket = false;
   if (!(g2f > 0.f)) {
     mode = 2;
@@ -862,18 +1008,8 @@ static __device__ void locate32(TrSmem& S, double Delta) {
     // boundary bracket as the alternative
     if (lmin > 0.f && n0 <= D2 * 1.01f) mode = 0;
     bracket = true;
-    const float lo = fmaxf(0.f, -lmin);
-    la = lo;
-    lb = lo + gnorm_s / (float)Delta * 1.01f + 1e-6f;
-    for (int r = 0; r < 4; ++r, ++round) {
-      const float l = la + (lb - la) * (float)(tid + 1) * kStep;
-      const bool inside = tid < kTrThreads - 1 && norm2_32s(S.df, S.ef, S.gf, l, cps, gps) <= D2;
-      const int t = first_hit(S, inside, round);
-      const float na = t == 0 ? la : la + (lb - la) * (float)t * kStep;
-      const float nb = t == kTrThreads - 1 ? lb : la + (lb - la) * (float)(t + 1) * kStep;
-      la = na;
-      lb = nb;
-    }
+#pragma unroll 1
+    for (int r = 1; r < 4; ++r) secular_round();
     // near the pole (nearly hard case) the FP32 bracket is still a good
     // start; the FP64 iteration below resolves it, and a true hard case
     // (no root above the pole) ends in the all-FP64 path
@@ -895,32 +1031,32 @@ static __device__ void locate32(TrSmem& S, double Delta) {
   __syncthreads();
 }
 
-// Exact trust-region subproblem of one source; 128 threads (4 warps) enter,
-// warp 0 finishes: it returns true and holds p in S.y and the predicted
-// gain in S.red[0].  g (27) and H (27 x 27) are in global memory.
-static __device__ bool tr_solve(TrSmem& S, const double* __restrict__ g, const double* __restrict__ H,
-                         double Delta) {
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+// B = -H (symmetrised) and g of one subproblem from global memory.
+static __device__ __forceinline__ void tr_load(TrSmem& S, const double* __restrict__ g,
+                                               const double* __restrict__ H, int tid) {
   for (int e = tid; e < N * N; e += kTrThreads) {
     const int i = e / N, j = e % N;
     const double b = -0.5 * (H[i * N + j] + H[j * N + i]);
     S.B[e] = b;
     S.ws.f.Bf[e] = (float)b;
   }
-  for (int e = tid; e < kTri; e += kTrThreads) {
-    // row i of lower entry e: i (i + 1) / 2 <= e < (i + 1) (i + 2) / 2
-    int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-    if (i * (i + 1) / 2 > e) --i;
-    if ((i + 1) * (i + 2) / 2 <= e) ++i;
-    S.tri[e] = make_short2((short)i, (short)(e - i * (i + 1) / 2));
-  }
   if (tid < N) {
     S.gh[tid] = g[tid];
     S.gfr[tid] = (float)g[tid];
   }
+}
+
+// Exact trust-region subproblem of one source; 128 threads (4 warps, tid
+// 0..127) enter, warp 0 finishes: it returns true and holds p in S.y and the
+// predicted gain in S.red[0].  On entry S.B and S.ws.f.Bf hold B = -H, S.gh
+// and S.gfr hold g.
+static __device__ bool tr_solve(TrSmem& S, double Delta, int tid) {
+  const int lane = tid & 31, wid = tid >> 5;
+  short2 rc[kLdlRounds];
+  ldl_entries(rc, tid);
   __syncthreads();
-  householder_blk(S);
-  locate32(S, Delta);
+  householder_blk(S, tid);
+  locate32(S, Delta, tid);
   const double D2 = Delta * Delta;
   bool done = false;
   if (S.mode != 2) {
@@ -929,7 +1065,7 @@ static __device__ bool tr_solve(TrSmem& S, const double* __restrict__ g, const d
     // warp 0 lane 0 only between barriers
     for (int it = 0; it < 8 && !done; ++it) {
       const double lam = S.lam;
-      const bool ok = ldl_factor(S, lam);
+      const bool ok = ldl_factor(S, lam, rc, tid);
       if (wid == 0) {
         // Bounds known in FP64 (the FP32 estimates only pick the start):
         // lo, a multiplier too small (indefinite, or |p| > Delta), < 0 for
@@ -949,8 +1085,7 @@ static __device__ bool tr_solve(TrSmem& S, const double* __restrict__ g, const d
           }
           mode = 1;
         } else {
-          double q2;
-          const double n2 = ldl_solve_full(S, S.gh, S.p, lane, &q2);
+          const double n2 = ldl_solve_full(S, S.gh, S.p, lane);
           const double np = sqrt(n2);
           if (lam == 0.0 && n2 <= D2) {
             fin = true;                 // interior Newton step
@@ -962,6 +1097,7 @@ static __device__ bool tr_solve(TrSmem& S, const double* __restrict__ g, const d
             if (mode == 0 && S.lam_b > lo && (hi < 0.0 || S.lam_b < hi)) {
               next = S.lam_b;           // l = 0 was not interior: start on the boundary
             } else {
+              const double q2 = ldl_curvature(S, S.p, lane);
               const double dl = (np - Delta) / Delta * n2 / q2;
               double ln = lam + dl;
               // a correction far below the distance to the pole: the
@@ -1012,13 +1148,14 @@ static __device__ bool tr_solve(TrSmem& S, const double* __restrict__ g, const d
   }
   if (!done) {
     __syncthreads();
-    return tr_solve_full(S, g, H, Delta);
+    return tr_solve_full(S, Delta, tid);
   }
   if (wid != 0) return false;
   // predicted gain g.p - p.B.p / 2 in FP64 on the full matrix, one row per lane
   double term = 0.0;
   if (lane < N) {
     double bp = 0.0;
+#pragma unroll 9
     for (int k = 0; k < N; ++k) bp = fma(S.B[lane * N + k], S.p[k], bp);
     term = S.p[lane] * fma(-0.5, bp, S.gh[lane]);
   }
@@ -1029,39 +1166,22 @@ static __device__ bool tr_solve(TrSmem& S, const double* __restrict__ g, const d
   return true;
 }
 
-// The step of slot j of the plan from its gradient and Hessian (v.grad,
-// v.hess), by the whole block: non-finite derivatives fail the source, a
-// predicted gain below kFtol (1 + |L|) or a radius below kDeltaMin
-// converges it (both leave the active set); otherwise the step, its
-// predicted gain and theta_trial are written.  Returns true, in every
-// thread, when a trial point was formed.
-static __device__ __forceinline__ bool tr_step_source(const PlanView& v, TrSmem& S, int j,
-                                               const double* delta, int32_t* status) {
-  const int tid = threadIdx.x, lane = tid & 31;
-  if (!v.active[j]) return false;
-  const int src = v.src_ids[j];
-  const double Dl = delta[src];
-  const double* g = v.grad + (size_t)j * N;
-  const double* H = v.hess + (size_t)j * N * N;
-  bool finite = true;
-  for (int e = tid; e < N * N; e += kTrThreads) finite &= isfinite(H[e]);
-  if (tid < N) finite &= isfinite(g[tid]);
-  finite = __syncthreads_and(finite) && isfinite(v.elbo_rel[j]);
-  if (!finite) {
-    if (tid == 0) {
-      status[src] = CELESTE_ST_FAILED;
-      v.active[j] = 0;
-    }
-    return false;
-  }
+// The step of slot j of the plan, source src, with radius Dl and value rel
+// (S loaded as for tr_solve; finite): a predicted gain below kFtol (1 + |L|)
+// or a radius below kDeltaMin converges the source (it leaves the active
+// set); otherwise the step, its predicted gain and theta_trial are written.
+// Returns true, in every thread, when a trial point was formed.
+static __device__ __forceinline__ bool tr_step_source(const PlanView& v, TrSmem& S, int j, int src,
+                                               double Dl, double rel, int32_t* status, int tid) {
+  const int lane = tid & 31;
   int formed = 0;
-  if (tr_solve(S, g, H, Dl)) {
+  if (tr_solve(S, Dl, tid)) {
     // warp 0
     double* p = v.step + (size_t)j * N;
     if (lane < N) p[lane] = S.y[lane];
     const double pred = S.red[0];
     if (lane == 0) v.pred[j] = pred;
-    if (pred <= kFtol * (1.0 + fabs(v.elbo_rel[j])) || Dl < kDeltaMin) {
+    if (pred <= kFtol * (1.0 + fabs(rel)) || Dl < kDeltaMin) {
       if (lane == 0) {
         status[src] = CELESTE_ST_CONVERGED;
         v.active[j] = 0;
