@@ -19,6 +19,8 @@
 // kernel only needs the Hermite polynomials of orders 0..4 in y = P (p - mu).
 #include <math.h>
 
+#include <type_traits>
+
 #include "device_once.h"
 #include "internal.cuh"
 #include "setup.cuh"
@@ -142,20 +144,18 @@ __device__ __forceinline__ void stage_record(float* __restrict__ dst, const floa
 }
 
 // Skip radii of the staged galaxy pairs, after stage_record and a warp
-// barrier (kPairF floats a pair, its first eight {A11, A12, A22, lw} in both
-// layouts): for d^2 beyond rec[kSkipBase + k kMaxProf + j] both halves of pair
+// barrier (derivs layout: a pair's first eight floats are its {A11, A12, A22,
+// lw}): for d^2 beyond rec[kSkipBase + k kMaxProf + j] both halves of pair
 // j have log2 phi <= lw - lambda_min(-A) d^2 < -128, where exp2 (which
 // flushes denormals here) returns zero, so the pair would add exact zeros.
 // 0.1 % on the radius and two powers of two of slack cover the rounding of
 // the bound and of the exponent; an ill-conditioned or non-finite form is
 // never skipped.
-template <int kPairF>
-__device__ __forceinline__ void stage_skip(float* __restrict__ rec, int base, int ne, int nd,
-                                           int lane) {
+__device__ __forceinline__ void stage_skip(float* __restrict__ rec, int ne, int nd, int lane) {
   const int nb = ne < nd ? ne : nd;
   if (lane < kPsf * nb) {
     const int k = lane / nb, j = lane - k * nb;
-    const float* c = rec + base + k * (ne + nd) * (kPairF / 2) + j * kPairF;
+    const float* c = rec + kCompBase + kPsf * kStarF + (k * (ne + nd) + 2 * j) * kGalF;
     float r = 0.f;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -417,44 +417,17 @@ __device__ __forceinline__ void gal_single(const float* __restrict__ c, const Of
 #undef GET
 }
 
-// Galaxy (rho-mixed) and star profile densities of one pair at a pixel
-// (value layout): the galaxy pairs in packed two-wide instructions, the
-// exponential and de Vaucouleurs sums in the two halves (each half adds its
-// components in the order of the derivative kernel's sums).
-__device__ __forceinline__ void profiles_value(const float* __restrict__ rec, int ne, int nd,
-                                               float px, float py, float& F0, float& F1) {
-  const float4* q4 = reinterpret_cast<const float4*>(rec + kCompBase);
-  float fs = 0.f;
-  float2 f = make_float2(0.f, 0.f);
-  const int per = ne + nd;
-  const int nb = ne < nd ? ne : nd;
-#pragma unroll
-  for (int k = 0; k < kPsf; ++k) {
-    const Offset o = make_offset(pixel_delta(rec, k, px, py));
-    fs += gauss_density(q4[k], o);
-    const Offset2 o2 = dup_offset(o);
-    const float4* g = q4 + kPsf + k * per;
-    for (int j = 0; j < nb; ++j) {
-      const float4 a = g[2 * j], b = g[2 * j + 1];
-      const float2 arg = fma2(make_float2(a.x, a.y), o2.xx,
-                              fma2(make_float2(a.z, a.w), o2.xy,
-                                   fma2(make_float2(b.x, b.y), o2.yy, make_float2(b.z, b.w))));
-      f = add2(f, make_float2(exp2f(arg.x), exp2f(arg.y)));
-    }
-    const float4* single = g + 2 * nb;
-    for (int j = nb; j < ne; ++j) f.x += gauss_density(*single++, o);
-    for (int j = nb; j < nd; ++j) f.y += gauss_density(*single++, o);
-  }
-  F0 = fmaf(rec[H_RHO], f.x, rec[H_RHO1] * f.y);
-  F1 = fs;
-}
-
-// profiles_value at two pixels (a and b), each with exactly the
-// instructions of profiles_value, reading each staged component once.
+// Galaxy (rho-mixed) and star profile densities of one pair at two pixels a
+// and b (value layout), reading each staged component once: the galaxy pairs
+// in packed two-wide instructions, the exponential and de Vaucouleurs sums in
+// the two halves (each half adds its components in the order of the
+// derivative kernel's sums).  (Leaving out vanished pairs, as the derivative
+// kernel does, costs more than it saves here: 1.64 ms against 1.62 for a
+// value pass of 2,000 blended sources, 1.40 against 1.28 for renders and
+// backgrounds of 500.)
 __device__ __forceinline__ void profiles_value2(const float* __restrict__ rec, int ne, int nd,
                                                 float pxa, float pya, float pxb, float pyb,
-                                                float& F0a, float& F1a, float& F0b,
-                                                float& F1b) {
+                                                float& F0a, float& F1a, float& F0b, float& F1b) {
   const float4* q4 = reinterpret_cast<const float4*>(rec + kCompBase);
   float fsa = 0.f, fsb = 0.f;
   float2 fa = make_float2(0.f, 0.f), fb = make_float2(0.f, 0.f);
@@ -469,6 +442,7 @@ __device__ __forceinline__ void profiles_value2(const float* __restrict__ rec, i
     fsb += gauss_density(qs, ob);
     const Offset2 a2 = dup_offset(oa), b2 = dup_offset(ob);
     const float4* g = q4 + kPsf + k * per;
+#pragma unroll 4
     for (int j = 0; j < nb; ++j) {
       const float4 a = g[2 * j], b = g[2 * j + 1];
       const float2 A11 = make_float2(a.x, a.y), A12 = make_float2(a.z, a.w);
@@ -942,7 +916,7 @@ __global__ void __launch_bounds__(128, 4) derivs_kernel(PlanView v, int ne, int 
 #pragma unroll
     for (int a = 0; a < kHessAcc; ++a) tile[a * kHessRow + lane] = 0.f;
     __syncwarp();
-    if (kSkip) stage_skip<2 * kGalF>(rec, kCompBase + kPsf * kStarF, ne, nd, lane);
+    if (kSkip) stage_skip(rec, ne, nd, lane);
     float acc[kGradAcc];
 #pragma unroll
     for (int a = 0; a < kGradAcc; ++a) acc[a] = 0.f;
@@ -1008,6 +982,47 @@ __global__ void __launch_bounds__(128) grad_kernel(PlanView v, int ne, int nd) {
   wq.done(lane);
 }
 
+// Stages a record for value-only passes.
+__device__ __forceinline__ void stage_value(float* rec, const PlanView& v, int pair, int lane,
+                                            int ne, int nd) {
+  __syncwarp();
+  stage_record<false>(rec, v.records + (size_t)pair * kRecF, kPsf * (1 + ne + nd), lane, ne);
+  __syncwarp();
+}
+
+// The own moments at pixels [begin, end) (row-major) of a rectangle w
+// columns wide: f(pre(q, column, row), q, column, row, E, V) for each, a
+// lane's pixels in ascending order; pre runs before the densities are
+// formed, so that what it loads is on its way meanwhile.  A lane takes pixels q and q + 32 in one pass over the
+// staged components.  The whole warp takes every pass; lanes past the end
+// repeat lane 0's pixel.  dx, dy: from the rectangle to the record's frame.
+template <class P, class F>
+__device__ __forceinline__ void for_moments(const float* __restrict__ rec, int begin, int end, int w,
+                                            int dx, int dy, int lane, int ne, int nd, P&& pre,
+                                            F&& f) {
+  PixelWalk pa(begin + lane, w, 64), pb(begin + lane + 32, w, 64);
+  for (int q = begin + lane; q - lane < end; q += 64, pa.next(w), pb.next(w)) {
+    int xa = pa.qx, ya = pa.qy, xb = pb.qx, yb = pb.qy;
+    if (q - lane + 64 > end) {
+      const int x0 = __shfl_sync(0xffffffffu, xa, 0), y0 = __shfl_sync(0xffffffffu, ya, 0);
+      if (q >= end) xa = x0, ya = y0;
+      if (q + 32 >= end) xb = x0, yb = y0;
+    }
+    const bool in_a = q < end, in_b = q + 32 < end;
+    const auto la = pre(in_a ? q : q - lane, xa, ya), lb = pre(in_b ? q + 32 : q - lane, xb, yb);
+    float F0[2], F1[2];
+    profiles_value2(rec, ne, nd, (float)(xa + dx), (float)(ya + dy), (float)(xb + dx),
+                    (float)(yb + dy), F0[0], F1[0], F0[1], F1[1]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (q + 32 * h >= end) break;
+      float Es, Vs;
+      own_moments(rec, F0[h], F1[h], Es, Vs);
+      f(h ? lb : la, q + 32 * h, h ? xb : xa, h ? yb : ya, Es, Vs);
+    }
+  }
+}
+
 // Value-only pass over one item: the pixel term at the record's point
 // (relative and baseline sums into the item's slot of vpartials); with
 // render set, the own moments are also stored there (row-major over the
@@ -1015,34 +1030,21 @@ __global__ void __launch_bounds__(128) grad_kernel(PlanView v, int ne, int nd) {
 __device__ __forceinline__ void value_item(const PlanView& v, int it, const Item& item,
                                            const PairInfo& pi, float* rec, int lane, int ne,
                                            int nd, float2* render) {
-  __syncwarp();
-  stage_record<false>(rec, v.records + (size_t)item.pair * kRecF, kPsf * (1 + ne + nd), lane, ne);
-  __syncwarp();
+  stage_value(rec, v, item.pair, lane, ne, nd);
   float rel = 0.f, base = 0.f;
-  const int end = item.start + item.count;
-  // a lane's pixels q and q + 32 in one pass over the staged components; the
-  // sums take pixel q, then q + 32, as one pixel per pass would
-  PixelWalk pa(item.start + lane, pi.w, 64), pb(item.start + lane + 32, pi.w, 64);
-  for (int q = item.start + lane; q < end; q += 64, pa.next(pi.w), pb.next(pi.w)) {
-    const bool has_b = q + 32 < end;
-    float F0[2], F1[2];
-    profiles_value2(rec, ne, nd, (float)pa.qx, (float)pa.qy, (float)pb.qx, (float)pb.qy, F0[0],
-                    F1[0], F0[1], F1[1]);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (h == 1 && !has_b) break;
-      const int qq = q + 32 * h, qx = h ? pb.qx : pa.qx, qy = h ? pb.qy : pa.qy;
-      const float x = __ldg(v.pixels + pi.pix_base + (int64_t)qy * pi.stride + qx);
-      const float2 bg = v.bg[pi.bg_base + qq];
-      float Es, Vs;
-      own_moments(rec, F0[h], F1[h], Es, Vs);
-      if (render) render[qq] = make_float2(Es, Vs);
-      const float E = bg.x + Es, V = bg.y + Vs;
-      const float r = __frcp_rn(E), rb = __frcp_rn(bg.x);
-      rel += fmaf(x, log1pf(Es * rb) - 0.5f * V * r * r + 0.5f * bg.y * rb * rb, -Es);
-      base += fmaf(x, __logf(bg.x) - 0.5f * bg.y * rb * rb, -bg.x);
-    }
-  }
+  for_moments(rec, item.start, item.start + item.count, pi.w, 0, 0, lane, ne, nd,
+                     [&](int q, int qx, int qy) {
+    const float2 bg = v.bg[pi.bg_base + q];
+    return make_float3(__ldg(v.pixels + pi.pix_base + (int64_t)qy * pi.stride + qx), bg.x, bg.y);
+  }, [&](float3 in, int q, int, int, float Es, float Vs) {
+    const float x = in.x;
+    const float2 bg = make_float2(in.y, in.z);
+    if (render) render[q] = make_float2(Es, Vs);
+    const float E = bg.x + Es, V = bg.y + Vs;
+    const float r = __frcp_rn(E), rb = __frcp_rn(bg.x);
+    rel += fmaf(x, log1pf(Es * rb) - 0.5f * V * r * r + 0.5f * bg.y * rb * rb, -Es);
+    base += fmaf(x, __logf(bg.x) - 0.5f * bg.y * rb * rb, -bg.x);
+  });
   rel = warp_sum(rel);
   base = warp_sum(base);
   if (lane == 0) {
@@ -1082,113 +1084,192 @@ __global__ void __launch_bounds__(128, 8) value_kernel(PlanView v, int ne, int n
   wq.done(lane);
 }
 
-// Stages neighbour pairs [c0, c0 + cnt) of own pair pi: rectangle and offset
-// of the neighbour's patch in the render cache (in its current half).
-__device__ __forceinline__ void stage_neighbours(const PlanView& v, const PairInfo& pi, int c0,
-                                                 int cnt, int4* srect, int64_t* soff, int lane) {
-  if (lane < cnt) {
-    const PairInfo qn = v.pairs[v.pair_nbr[pi.nbr_begin + c0 + lane]];
-    srect[lane] = make_int4(qn.x0, qn.y0, qn.w, qn.h);
-    soff[lane] = v.patches[qn.patch].pool_offset + cache_base(v, qn.source);
-  }
+// ---- backgrounds, kBgChunk pixels of an item at a time: sky plus each
+// neighbour's E and V where the pixel lies in that neighbour's patch (support
+// rule, Sec. 2.2.3), in neighbour order.
+constexpr int kBgChunk = 256;
+constexpr int kBgWarpF = kValRecF + 2 * kBgChunk;          // a staged record, the chunk's sums
+constexpr int kBgStages = 4;
+constexpr int kBgCacheF = kBgStages * 2 * kBgChunk;        // cached moments on their way in
+
+__device__ __forceinline__ float sky_checked(const PlanView& v, const celeste_image& im, float x,
+                                             float y) {
+  const float s = sky_value(im, v.sky, x, y);
+  if (!(s > 0.f)) set_error(v.err, CELESTE_DERR_SKY);
+  return s;
 }
 
-// Adds the cached moments of the staged neighbours whose patches hold the
-// pixel (gx, gy) of the image, in staging order.
-__device__ __forceinline__ float2 add_neighbours(const PlanView& v, float2 b, int gx, int gy,
-                                                 int cnt, const int4* srect,
-                                                 const int64_t* soff) {
-  for (int k = 0; k < cnt; ++k) {
-    const int4 r = srect[k];
-    const int lx = gx - r.x, ly = gy - r.y;
-    if (lx < 0 || ly < 0 || lx >= r.z || ly >= r.w) continue;
-    const float2 c = v.cache[soff[k] + ly * r.z + lx];
-    b.x += c.x;
-    b.y += c.y;
-  }
-  return b;
-}
-
-// Background of item it's pixels (own pair pi): sky plus each neighbour's E
-// and V where the pixel lies in that neighbour's patch (support rule, Sec.
-// 2.2.3).  rec: the warp's staging area (kValRecF floats).
-__device__ __forceinline__ void background_item(const PlanView& v, const Item& item,
-                                                const PairInfo& pi, float* rec, int lane, int ne,
-                                                int nd) {
+// Without a render cache the neighbours are rendered: the lanes go over the
+// pixels of each neighbour's overlap with the chunk, two a lane (not over
+// the chunk, where lanes outside the overlap would idle), and add to sums in
+// the warp's shared memory (rec: kBgWarpF floats).  300 blended sources:
+// 755 us, 1,008 with a pixel a lane over the whole chunk and sums in L2; the
+// 1,024 sources of a field 68 -> 42 us.
+__device__ __forceinline__ void background_rendered(const PlanView& v, const Item& item,
+                                                    const PairInfo& pi, float* rec, int lane,
+                                                    int ne, int nd) {
   const celeste_image& im = v.images[pi.image];
+  float2* sum = reinterpret_cast<float2*>(rec + kValRecF);
   const int end = item.start + item.count;
-  if (v.cache) {
-    // sky plus the neighbours' cached moments (the values the render
-    // below would produce, added in the same order), 32 neighbour pairs
-    // at a time staged in the warp's shared memory; the first 32 are
-    // added in the pass that evaluates the sky
-    int4* srect = reinterpret_cast<int4*>(rec);
-    int64_t* soff = reinterpret_cast<int64_t*>(rec + 4 * 32);
-    const int nn = pi.nbr_end - pi.nbr_begin;
-    for (int c0 = 0; c0 == 0 || c0 < nn; c0 += 32) {
-      const int cnt = max(0, min(32, nn - c0));
-      __syncwarp();
-      stage_neighbours(v, pi, c0, cnt, srect, soff, lane);
-      __syncwarp();
-      PixelWalk pw(item.start + lane, pi.w);
-      for (int q = item.start + lane; q < end; q += 32, pw.next(pi.w)) {
-        const int gx = pi.x0 + pw.qx, gy = pi.y0 + pw.qy;
-        float2 b;
-        if (c0 == 0) {
-          const float s = sky_value(im, v.sky, (float)gx, (float)gy);
-          if (!(s > 0.f)) set_error(v.err, CELESTE_DERR_SKY);
-          b = make_float2(s, 0.f);
-        } else {
-          b = v.bg[pi.bg_base + q];
-        }
-        v.bg[pi.bg_base + q] = add_neighbours(v, b, gx, gy, cnt, srect, soff);
+  const int nn = pi.nbr_end - pi.nbr_begin;
+  for (int c0 = item.start; c0 < end; c0 += kBgChunk) {
+    const int c1 = min(c0 + kBgChunk, end);
+    __syncwarp();
+    PixelWalk pw(c0 + lane, pi.w);
+    for (int q = c0 + lane; q < c1; q += 32, pw.next(pi.w))
+      sum[q - c0] =
+          make_float2(sky_checked(v, im, (float)(pi.x0 + pw.qx), (float)(pi.y0 + pw.qy)), 0.f);
+    const int r0 = c0 / pi.w, r1 = (c1 - 1) / pi.w + 1;   // the chunk's rows
+    for (int g0 = 0; g0 < nn; g0 += 32) {
+      // the overlaps of up to 32 neighbours, one in each lane
+      int np = 0, ox = 0, oy = 0, ow = 0, oh = 0, nx = 0, ny = 0;
+      if (g0 + lane < nn) {
+        np = v.pair_nbr[pi.nbr_begin + g0 + lane];
+        const PairInfo& qn = v.pairs[np];
+        nx = pi.x0 - qn.x0;                    // from the own patch to the neighbour's
+        ny = pi.y0 - qn.y0;
+        ox = max(0, -nx);
+        ow = min(pi.w, qn.w - nx) - ox;
+        oy = max(r0, -ny);
+        oh = min(r1, qn.h - ny) - oy;
+      }
+      unsigned todo = __ballot_sync(0xffffffffu, ow > 0 && oh > 0);
+      for (; todo; todo &= todo - 1) {
+        const int g = __ffs(todo) - 1;
+        const int bx = __shfl_sync(0xffffffffu, ox, g), by = __shfl_sync(0xffffffffu, oy, g);
+        const int bw = __shfl_sync(0xffffffffu, ow, g);
+        const int n = bw * __shfl_sync(0xffffffffu, oh, g);
+        const int mx = __shfl_sync(0xffffffffu, nx, g), my = __shfl_sync(0xffffffffu, ny, g);
+        stage_value(rec, v, __shfl_sync(0xffffffffu, np, g), lane, ne, nd);
+        for_moments(rec, 0, n, bw, bx + mx, by + my, lane, ne, nd,
+                           [](int, int, int) { return 0; },
+                           [&](int, int, int qx, int qy, float Es, float Vs) {
+          const int q = (by + qy) * pi.w + bx + qx - c0;
+          if (q < 0 || q >= c1 - c0) return;
+          const float2 b = sum[q];
+          sum[q] = make_float2(b.x + Es, b.y + Vs);
+        });
       }
     }
-    return;
-  }
-  PixelWalk pw(item.start + lane, pi.w);
-  for (int q = item.start + lane; q < end; q += 32, pw.next(pi.w)) {
-    const float s = sky_value(im, v.sky, (float)(pi.x0 + pw.qx), (float)(pi.y0 + pw.qy));
-    if (!(s > 0.f)) set_error(v.err, CELESTE_DERR_SKY);
-    v.bg[pi.bg_base + q] = make_float2(s, 0.f);
-  }
-  for (int nb = pi.nbr_begin; nb < pi.nbr_end; ++nb) {
-    const int np = v.pair_nbr[nb];
-    const PairInfo qn = v.pairs[np];
     __syncwarp();
-    stage_record<false>(rec, v.records + (size_t)np * kRecF, kPsf * (1 + ne + nd), lane, ne);
-    __syncwarp();
-    for (int q = item.start + lane; q < end; q += 32) {
-      const int qy = q / pi.w;
-      const int gx = pi.x0 + (q - qy * pi.w), gy = pi.y0 + qy;
-      const int lx = gx - qn.x0, ly = gy - qn.y0;
-      if (lx < 0 || ly < 0 || lx >= qn.w || ly >= qn.h) continue;
-      float F0, F1, Es, Vs;
-      profiles_value(rec, ne, nd, (float)lx, (float)ly, F0, F1);
-      own_moments(rec, F0, F1, Es, Vs);
-      float2 b = v.bg[pi.bg_base + q];
-      b.x += Es;
-      b.y += Vs;
-      v.bg[pi.bg_base + q] = b;
-    }
+    for (int q = c0 + lane; q < c1; q += 32) v.bg[pi.bg_base + q] = sum[q - c0];
   }
 }
 
-__global__ void __launch_bounds__(128) background_kernel(PlanView v, int ne, int nd) {
+// With a render cache the neighbours' moments are gathered from it (the
+// values the rendering would produce, added in the same order): the lane's
+// eight pixels of the chunk stay in registers, and the neighbours' values
+// come through asynchronous copies to shared memory (st: kBgCacheF floats of
+// the warp), kBgStages - 1 neighbours ahead of the one being added, zeros
+// where the pixel is not in the neighbour's patch.  Bound by memory latency:
+// loads that a lane waits for, one neighbour or one pixel at a time, reach
+// 1.6-1.9 TB/s (a Newton pass over 2,000 blended sources: 1.02 ms of
+// preparation launches, 1.58 with a pixel's neighbours one after another).
+__device__ __forceinline__ void copy_async8(unsigned dst, const void* src, bool valid) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src),
+               "r"(valid ? 8 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void background_cached(const PlanView& v, const Item& item,
+                                                  const PairInfo& pi, float* st, int lane) {
+  constexpr int kPix = kBgChunk / 32;
+  const celeste_image& im = v.images[pi.image];
+  const float2* stage = reinterpret_cast<const float2*>(st) + lane;
+  const unsigned dst0 = (unsigned)__cvta_generic_to_shared(st) + lane * sizeof(float2);
+  const int end = item.start + item.count;
+  const int nn = pi.nbr_end - pi.nbr_begin;
+  for (int c0 = item.start; c0 < end; c0 += kBgChunk) {
+    const int c1 = min(c0 + kBgChunk, end);
+    int x[kPix], y[kPix];
+    float2 b[kPix];
+    PixelWalk pw(c0 + lane, pi.w);
+#pragma unroll
+    for (int u = 0; u < kPix; ++u, pw.next(pi.w)) {
+      const bool in = c0 + lane + 32 * u < c1;
+      x[u] = in ? pw.qx : -(1 << 20);          // (outside every patch)
+      y[u] = pw.qy;
+      if (in) b[u] = make_float2(sky_checked(v, im, (float)(pi.x0 + pw.qx), (float)(pi.y0 + pw.qy)), 0.f);
+    }
+    const int r0 = c0 / pi.w, r1 = (c1 - 1) / pi.w + 1;   // the chunk's rows
+    for (int g0 = 0; g0 < nn; g0 += 32) {
+      // up to 32 neighbours, one in each lane
+      int nx = 0, ny = 0, nw = 0, nh = 0;
+      int64_t off = 0;
+      if (g0 + lane < nn) {
+        const PairInfo& qn = v.pairs[v.pair_nbr[pi.nbr_begin + g0 + lane]];
+        nx = pi.x0 - qn.x0;                    // from the own patch to the neighbour's
+        ny = pi.y0 - qn.y0;
+        nw = qn.w;
+        nh = qn.h;
+        off = v.patches[qn.patch].pool_offset + cache_base(v, qn.source);
+      }
+      unsigned todo = __ballot_sync(0xffffffffu, min(r1, nh - ny) > max(r0, -ny) &&
+                                                     min(pi.w, nw - nx) > max(0, -nx));
+      const int cnt = __popc(todo);
+      for (int k = 0; k < cnt + kBgStages - 1; ++k) {
+        if (k < cnt) {
+          const int g = __ffs(todo) - 1;
+          todo &= todo - 1;
+          const int mx = __shfl_sync(0xffffffffu, nx, g), my = __shfl_sync(0xffffffffu, ny, g);
+          const int mw = __shfl_sync(0xffffffffu, nw, g), mh = __shfl_sync(0xffffffffu, nh, g);
+          const float2* src = v.cache + __shfl_sync(0xffffffffu, off, g);
+          const unsigned dst = dst0 + (k % kBgStages) * (kBgChunk * sizeof(float2));
+#pragma unroll
+          for (int u = 0; u < kPix; ++u) {
+            const int lx = x[u] + mx, ly = y[u] + my;
+            const bool in = (unsigned)lx < (unsigned)mw && (unsigned)ly < (unsigned)mh;
+            copy_async8(dst + u * 32 * sizeof(float2), src + (in ? ly * mw + lx : 0), in);
+          }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (k >= kBgStages - 1) {
+          // each lane reads only what it copied itself
+          asm volatile("cp.async.wait_group %0;" ::"n"(kBgStages - 1) : "memory");
+          const float2* c = stage + ((k + 1) % kBgStages) * kBgChunk;
+#pragma unroll
+          for (int u = 0; u < kPix; ++u) {
+            const float2 a = c[32 * u];
+            b[u].x += a.x;
+            b[u].y += a.y;
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kPix; ++u)
+      if (c0 + lane + 32 * u < c1) v.bg[pi.bg_base + c0 + lane + 32 * u] = b[u];
+  }
+}
+
+// Five blocks per SM (102 registers): 5-18 % faster than eight at 64.
+template <bool kQueue>
+__global__ void __launch_bounds__(128, 5) background_kernel(PlanView v, int ne, int nd) {
   extern __shared__ float4 smem4[];
   float* smem = reinterpret_cast<float*>(smem4);
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
-  float* rec = smem + wib * kValRecF;
-  WarpQueue wq(nullptr);   // grid stride (short units, as in prepare_kernel)
+  float* rec = smem + wib * kBgWarpF;
+  WarpQueue wq(kQueue ? v.work_ctr : nullptr);
   for (; wq.it < v.n_items; wq.advance()) {
     wq.ask(lane);
     const Item item = v.items[wq.it];
     const PairInfo pi = v.pairs[item.pair];
     if (!v.active[pi.slot]) continue;
-    background_item(v, item, pi, rec, lane, ne, nd);
+    background_rendered(v, item, pi, rec, lane, ne, nd);
   }
   wq.done(lane);
+}
+
+__global__ void __launch_bounds__(128) background_cached_kernel(PlanView v) {
+  extern __shared__ float4 smem4[];
+  const int lane = threadIdx.x & 31;
+  float* st = reinterpret_cast<float*>(smem4) + (threadIdx.x >> 5) * kBgCacheF;
+  const int nwarps = gridDim.x * (blockDim.x >> 5);
+  for (int it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < v.n_items; it += nwarps) {
+    const Item item = v.items[it];
+    const PairInfo pi = v.pairs[item.pair];
+    if (v.active[pi.slot]) background_cached(v, item, pi, st, lane);
+  }
 }
 
 // The start of a Newton iteration of a colour class, one warp per unit of
@@ -1198,12 +1279,12 @@ __global__ void __launch_bounds__(128) background_kernel(PlanView v, int ne, int
 // neighbours, so the own records are all it needs).
 __global__ void __launch_bounds__(128) prepare_kernel(PlanView v, const ModelDev* __restrict__ model,
                                                       const int32_t* __restrict__ status,
-                                                      int n_setup, int bg, int ne, int nd) {
+                                                      int n_setup, int bg) {
   extern __shared__ float4 smem4[];
   float* smem = reinterpret_cast<float*>(smem4);
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
-  float* rec = smem + wib * kValRecF;
+  float* rec = smem + wib * kBgCacheF;
   const int n_mark = (v.n + 31) / 32;
   const int units = n_mark + n_setup + (bg ? v.n_items : 0);
   // grid stride: its units are short, so a queue's claim would not return
@@ -1221,71 +1302,59 @@ __global__ void __launch_bounds__(128) prepare_kernel(PlanView v, const ModelDev
       const Item item = v.items[u - n_mark - n_setup];
       const PairInfo pi = v.pairs[item.pair];
       if (!active_of(status[pi.source])) continue;
-      background_item(v, item, pi, rec, lane, ne, nd);
+      background_cached(v, item, pi, rec, lane);
     }
   }
   wq.done(lane);
 }
 
+// The loop of the render kernels: f(item, pair info) for every item.
+template <bool kQueue, class F>
+__device__ __forceinline__ void for_items(const PlanView& v, int lane, F&& f) {
+  WarpQueue wq(kQueue ? v.work_ctr : nullptr);
+  for (; wq.it < v.n_items; wq.advance()) {
+    wq.ask(lane);
+    const Item item = v.items[wq.it];
+    f(item, v.pairs[item.pair]);
+  }
+  wq.done(lane);
+}
+
 // Own E_s and V_s of every plan pair, scattered to the caller's pool layout.
-__global__ void __launch_bounds__(128) render_kernel(PlanView v, int ne, int nd, float* E_out,
-                                                     float* V_out,
-                                                     const celeste_patch* __restrict__ patches) {
+template <bool kQueue>
+__global__ void __launch_bounds__(128, 8) render_kernel(PlanView v, int ne, int nd, float* E_out,
+                                                        float* V_out,
+                                                        const celeste_patch* __restrict__ patches) {
   extern __shared__ float4 smem4[];
-  float* smem = reinterpret_cast<float*>(smem4);
   const int lane = threadIdx.x & 31;
-  const int wib = threadIdx.x >> 5;
-  float* rec = smem + wib * kValRecF;
-  const int nwarps = gridDim.x * (blockDim.x >> 5);
-  for (int it = blockIdx.x * (blockDim.x >> 5) + wib; it < v.n_items; it += nwarps) {
-    const Item item = v.items[it];
-    const PairInfo pi = v.pairs[item.pair];
+  float* rec = reinterpret_cast<float*>(smem4) + (threadIdx.x >> 5) * kValRecF;
+  for_items<kQueue>(v, lane, [&](const Item& item, const PairInfo& pi) {
     const int64_t off = patches[pi.patch].pool_offset;
-    __syncwarp();
-    stage_record<false>(rec, v.records + (size_t)item.pair * kRecF,
-                        kPsf * (1 + ne + nd), lane, ne);
-    __syncwarp();
-    const int end = item.start + item.count;
-    for (int q = item.start + lane; q < end; q += 32) {
-      const int qy = q / pi.w;
-      const int qx = q - qy * pi.w;
-      float F0, F1, Es, Vs;
-      profiles_value(rec, ne, nd, (float)qx, (float)qy, F0, F1);
-      own_moments(rec, F0, F1, Es, Vs);
+    stage_value(rec, v, item.pair, lane, ne, nd);
+    for_moments(rec, item.start, item.start + item.count, pi.w, 0, 0, lane, ne, nd,
+                       [](int, int, int) { return 0; }, [&](int, int q, int, int, float Es, float Vs) {
       if (E_out) E_out[off + q] = Es;
       if (V_out) V_out[off + q] = Vs;
-    }
-  }
+    });
+  });
 }
 
 // Own E_s and V_s of the plan's pairs into the problem's render cache.
-__global__ void __launch_bounds__(128) render_cache_kernel(PlanView v, int ne, int nd,
-                                                           const int32_t* __restrict__ status) {
+template <bool kQueue>
+__global__ void __launch_bounds__(128, 8) render_cache_kernel(PlanView v, int ne, int nd,
+                                                              const int32_t* __restrict__ status) {
   extern __shared__ float4 smem4[];
-  float* smem = reinterpret_cast<float*>(smem4);
   const int lane = threadIdx.x & 31;
-  const int wib = threadIdx.x >> 5;
-  float* rec = smem + wib * kValRecF;
-  const int nwarps = gridDim.x * (blockDim.x >> 5);
-  for (int it = blockIdx.x * (blockDim.x >> 5) + wib; it < v.n_items; it += nwarps) {
-    const Item item = v.items[it];
-    const PairInfo pi = v.pairs[item.pair];
-    if (status && status[pi.source] != CELESTE_ST_ACCEPTED) continue;
+  float* rec = reinterpret_cast<float*>(smem4) + (threadIdx.x >> 5) * kValRecF;
+  for_items<kQueue>(v, lane, [&](const Item& item, const PairInfo& pi) {
+    if (status && status[pi.source] != CELESTE_ST_ACCEPTED) return;
     float2* out = v.cache + cache_base(v, pi.source) + v.patches[pi.patch].pool_offset;
-    __syncwarp();
-    stage_record<false>(rec, v.records + (size_t)item.pair * kRecF,
-                        kPsf * (1 + ne + nd), lane, ne);
-    __syncwarp();
-    const int end = item.start + item.count;
-    for (int q = item.start + lane; q < end; q += 32) {
-      const int qy = q / pi.w;
-      const int qx = q - qy * pi.w;
-      float F0, F1, Es, Vs;
-      profiles_value(rec, ne, nd, (float)qx, (float)qy, F0, F1);
-      own_moments(rec, F0, F1, Es, Vs);
+    stage_value(rec, v, item.pair, lane, ne, nd);
+    for_moments(rec, item.start, item.start + item.count, pi.w, 0, 0, lane, ne, nd,
+                       [](int, int, int) { return 0; }, [&](int, int q, int, int, float Es, float Vs) {
       out[q] = make_float2(Es, Vs);
-    }
-  }
+    });
+  });
 }
 
 // A copy: every lane loads up to eight pixels before it stores any, so that
@@ -1317,33 +1386,21 @@ __global__ void __launch_bounds__(128) commit_render_kernel(PlanView v,
 // Adds the plan's own moments into per-image buffers in the pixel-pool
 // layout.  Plain read-modify-write: sources of one colour class never share
 // a pixel, and classes are launched one after another.
-__global__ void __launch_bounds__(128) accumulate_kernel(PlanView v, int ne, int nd, float* Eimg,
-                                                         float* Vimg) {
+template <bool kQueue>
+__global__ void __launch_bounds__(128, 8) accumulate_kernel(PlanView v, int ne, int nd, float* Eimg,
+                                                            float* Vimg) {
   extern __shared__ float4 smem4[];
-  float* smem = reinterpret_cast<float*>(smem4);
   const int lane = threadIdx.x & 31;
-  const int wib = threadIdx.x >> 5;
-  float* rec = smem + wib * kValRecF;
-  const int nwarps = gridDim.x * (blockDim.x >> 5);
-  for (int it = blockIdx.x * (blockDim.x >> 5) + wib; it < v.n_items; it += nwarps) {
-    const Item item = v.items[it];
-    const PairInfo pi = v.pairs[item.pair];
-    __syncwarp();
-    stage_record<false>(rec, v.records + (size_t)item.pair * kRecF,
-                        kPsf * (1 + ne + nd), lane, ne);
-    __syncwarp();
-    const int end = item.start + item.count;
-    for (int q = item.start + lane; q < end; q += 32) {
-      const int qy = q / pi.w;
-      const int qx = q - qy * pi.w;
-      float F0, F1, Es, Vs;
-      profiles_value(rec, ne, nd, (float)qx, (float)qy, F0, F1);
-      own_moments(rec, F0, F1, Es, Vs);
+  float* rec = reinterpret_cast<float*>(smem4) + (threadIdx.x >> 5) * kValRecF;
+  for_items<kQueue>(v, lane, [&](const Item& item, const PairInfo& pi) {
+    stage_value(rec, v, item.pair, lane, ne, nd);
+    for_moments(rec, item.start, item.start + item.count, pi.w, 0, 0, lane, ne, nd,
+                       [](int, int, int) { return 0; }, [&](int, int, int qx, int qy, float Es, float Vs) {
       const int64_t m = pi.pix_base + (int64_t)qy * pi.stride + qx;
       Eimg[m] += Es;
       Vimg[m] += Vs;
-    }
-  }
+    });
+  });
 }
 
 // Pixel term -E + x (log E - V / (2 E^2)) (Eq. eq:log_p_last, without
@@ -1410,23 +1467,36 @@ __global__ void __launch_bounds__(256) field_sum_kernel(const double* parts, int
   }
 }
 
-__global__ void bg_scatter_kernel(PlanView v, float* bgE, float* bgV,
-                                  const celeste_patch* __restrict__ patches) {
+// Backgrounds from the plan's pool to the caller's, eight loads in flight per
+// lane (a copy: 167 us for 12.8 M pixels with one).
+__global__ void __launch_bounds__(128) bg_scatter_kernel(PlanView v, float* bgE, float* bgV,
+                                                         const celeste_patch* __restrict__ patches) {
   const int nwarps = gridDim.x * (blockDim.x >> 5);
   const int lane = threadIdx.x & 31;
   for (int it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < v.n_items; it += nwarps) {
     const Item item = v.items[it];
     const PairInfo pi = v.pairs[item.pair];
-    const int64_t off = patches[pi.patch].pool_offset;
-    for (int q = item.start + lane; q < item.start + item.count; q += 32) {
-      const float2 b = v.bg[pi.bg_base + q];
-      if (bgE) bgE[off + q] = b.x;
-      if (bgV) bgV[off + q] = b.y;
+    const int64_t off = patches[pi.patch].pool_offset + item.start;
+    const float2* __restrict__ src = v.bg + pi.bg_base + item.start;
+    for (int q0 = lane; q0 < item.count; q0 += 8 * 32) {
+      float2 b[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (q0 + 32 * u < item.count) b[u] = __ldcs(src + q0 + 32 * u);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (q0 + 32 * u < item.count) {
+          if (bgE) bgE[off + q0 + 32 * u] = b[u].x;
+          if (bgV) bgV[off + q0 + 32 * u] = b[u].y;
+        }
+      }
     }
   }
 }
 
 static size_t smem_bytes(int wpb) { return (size_t)wpb * kValRecF * sizeof(float); }
+static size_t smem_bytes_bg(int wpb) { return (size_t)wpb * kBgWarpF * sizeof(float); }
+static size_t smem_bytes_cached(int wpb) { return (size_t)wpb * kBgCacheF * sizeof(float); }
 static size_t smem_bytes_derivs(int wpb) { return (size_t)wpb * kDerivWarpF * sizeof(float); }
 static size_t smem_bytes_grad(int wpb) { return (size_t)wpb * kDerivRecF * sizeof(float); }
 
@@ -1455,7 +1525,7 @@ static cudaError_t derivs_attr() {
 // until measured on that device).
 enum {
   kOccDerivs, kOccGrad, kOccValue, kOccDerivsQ, kOccGradQ, kOccValueQ, kOccBackground, kOccRender,
-  kOccCommit, kOccPrepare, kOccKinds
+  kOccCommit, kOccPrepare, kOccCached, kOccKinds
 };
 static std::atomic<int> g_occ[kMaxDevices][kOccKinds] = {};
 static DeviceOnce g_occ_once;
@@ -1484,17 +1554,22 @@ cudaError_t init_pixel_occupancy() {
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[kOccValueQ], value_kernel<true>,
                                                         kWpb * 32, sm);
     if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[kOccBackground], background_kernel,
-                                                        kWpb * 32, sm);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[kOccBackground],
+                                                        background_kernel<true>, kWpb * 32,
+                                                        smem_bytes_bg(kWpb));
     if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[kOccRender], render_cache_kernel,
-                                                        kWpb * 32, sm);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[kOccRender],
+                                                        render_cache_kernel<true>, kWpb * 32,
+                                                        sm);
     if (e == cudaSuccess)
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[kOccCommit], commit_render_kernel,
                                                         kWpb * 32, 0);
     if (e == cudaSuccess)
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[kOccPrepare], prepare_kernel,
-                                                        kWpb * 32, sm);
+                                                        kWpb * 32, smem_bytes_cached(kWpb));
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[kOccCached], background_cached_kernel,
+                                                        kWpb * 32, smem_bytes_cached(kWpb));
     if (e == cudaSuccess)
       for (int k = 0; k < kOccKinds; ++k) g_occ[dev][k].store(occ[k], std::memory_order_relaxed);
     return e;
@@ -1515,13 +1590,6 @@ static int grid_for(const Launch& L, int n_items, int wpb, int occ_kind = -1) {
   return blocks < needed ? blocks : (needed > 0 ? needed : 1);
 }
 
-cudaError_t launch_background(const Launch& L, const PlanView& v) {
-  if (v.n_items == 0) return cudaSuccess;
-  background_kernel<<<grid_for(L, v.n_items, kWpb, kOccBackground), kWpb * 32, smem_bytes(kWpb), L.stream>>>(
-      v, L.n_exp, L.n_dev);
-  return cudaGetLastError();
-}
-
 // The work queue pays when a launch has many items per warp (its claims
 // then balance the warps' finishing times); with few, the grid-stride form
 // (fewer registers, no claims) is faster.
@@ -1539,6 +1607,30 @@ static bool use_queue(const PlanView& v, int blocks) {
 constexpr int kSkipArea = 2048;
 static bool use_skip(const Launch& L, const PlanView& v) {
   return v.n_bg >= (int64_t)kSkipArea * v.n_own_pairs && v.n_items > 16 * L.sm_count;
+}
+
+// A launch over items of a value-only kernel, kernel(queue, grid) with queue
+// a compile-time constant: with the work queue where the grid has many items
+// per warp (occ_q: that form's occupancy).
+template <class F>
+static cudaError_t launch_items(const Launch& L, const PlanView& v, int occ, int occ_q, F&& kernel) {
+  if (v.n_items == 0) return cudaSuccess;
+  const int gq = grid_for(L, v.n_items, kWpb, occ_q);
+  if (use_queue(v, gq)) kernel(std::true_type(), gq);
+  else kernel(std::false_type(), grid_for(L, v.n_items, kWpb, occ));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_background(const Launch& L, const PlanView& v) {
+  if (v.cache && v.n_items) {
+    background_cached_kernel<<<grid_for(L, v.n_items, kWpb, kOccCached), kWpb * 32,
+                               smem_bytes_cached(kWpb), L.stream>>>(v);
+    return cudaGetLastError();
+  }
+  return launch_items(L, v, kOccBackground, kOccBackground, [&](auto q, int grid) {
+    background_kernel<decltype(q)::value>
+        <<<grid, kWpb * 32, smem_bytes_bg(kWpb), L.stream>>>(v, L.n_exp, L.n_dev);
+  });
 }
 
 cudaError_t launch_pixels_derivs(const Launch& L, const PlanView& v) {
@@ -1566,21 +1658,18 @@ cudaError_t launch_pixels_grad(const Launch& L, const PlanView& v) {
 cudaError_t launch_pixels_value(const Launch& L, const PlanView& v, bool keep_render) {
   if (v.n_items == 0) return cudaSuccess;
   const int mode = !keep_render || !v.cache ? 0 : (v.cache_half ? 2 : 1);
-  const int gq = grid_for(L, v.n_items, kWpb, kOccValueQ);
-  if (use_queue(v, gq))
-    value_kernel<true><<<gq, kWpb * 32, smem_bytes(kWpb), L.stream>>>(v, L.n_exp, L.n_dev, mode);
-  else
-    value_kernel<false><<<grid_for(L, v.n_items, kWpb, kOccValue), kWpb * 32, smem_bytes(kWpb),
-                          L.stream>>>(v, L.n_exp, L.n_dev, mode);
-  return cudaGetLastError();
+  return launch_items(L, v, kOccValue, kOccValueQ, [&](auto q, int grid) {
+    value_kernel<decltype(q)::value>
+        <<<grid, kWpb * 32, smem_bytes(kWpb), L.stream>>>(v, L.n_exp, L.n_dev, mode);
+  });
 }
 
 cudaError_t launch_prepare(const Launch& L, const PlanView& v, const ModelDev* model,
                            const int32_t* status, int n_setup, bool background) {
   const int units = (v.n + 31) / 32 + n_setup + (background ? v.n_items : 0);
   if (units == 0) return cudaSuccess;
-  prepare_kernel<<<grid_for(L, units, kWpb, kOccPrepare), kWpb * 32, smem_bytes(kWpb),
-                   L.stream>>>(v, model, status, n_setup, background ? 1 : 0, L.n_exp, L.n_dev);
+  prepare_kernel<<<grid_for(L, units, kWpb, kOccPrepare), kWpb * 32, smem_bytes_cached(kWpb),
+                   L.stream>>>(v, model, status, n_setup, background ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -1593,24 +1682,25 @@ cudaError_t launch_commit_render(const Launch& L, const PlanView& v, const int32
 
 cudaError_t launch_render(const Launch& L, const PlanView& v, float* E_out, float* V_out,
                           const celeste_patch* patches) {
-  if (v.n_items == 0) return cudaSuccess;
-  render_kernel<<<grid_for(L, v.n_items, kWpb), kWpb * 32, smem_bytes(kWpb), L.stream>>>(
-      v, L.n_exp, L.n_dev, E_out, V_out, patches);
-  return cudaGetLastError();
+  return launch_items(L, v, kOccRender, kOccRender, [&](auto q, int grid) {
+    render_kernel<decltype(q)::value>
+        <<<grid, kWpb * 32, smem_bytes(kWpb), L.stream>>>(v, L.n_exp, L.n_dev, E_out, V_out, patches);
+  });
 }
 
 cudaError_t launch_render_cache(const Launch& L, const PlanView& v, const int32_t* status) {
-  if (v.n_items == 0 || !v.cache) return cudaSuccess;
-  render_cache_kernel<<<grid_for(L, v.n_items, kWpb, kOccRender), kWpb * 32, smem_bytes(kWpb), L.stream>>>(
-      v, L.n_exp, L.n_dev, status);
-  return cudaGetLastError();
+  if (!v.cache) return cudaSuccess;
+  return launch_items(L, v, kOccRender, kOccRender, [&](auto q, int grid) {
+    render_cache_kernel<decltype(q)::value>
+        <<<grid, kWpb * 32, smem_bytes(kWpb), L.stream>>>(v, L.n_exp, L.n_dev, status);
+  });
 }
 
 cudaError_t launch_accumulate(const Launch& L, const PlanView& v, float* Eimg, float* Vimg) {
-  if (v.n_items == 0) return cudaSuccess;
-  accumulate_kernel<<<grid_for(L, v.n_items, kWpb, kOccRender), kWpb * 32, smem_bytes(kWpb),
-                      L.stream>>>(v, L.n_exp, L.n_dev, Eimg, Vimg);
-  return cudaGetLastError();
+  return launch_items(L, v, kOccRender, kOccRender, [&](auto q, int grid) {
+    accumulate_kernel<decltype(q)::value>
+        <<<grid, kWpb * 32, smem_bytes(kWpb), L.stream>>>(v, L.n_exp, L.n_dev, Eimg, Vimg);
+  });
 }
 
 cudaError_t launch_field_terms(const Launch& L, const celeste_image* images, int n_images,
@@ -1632,8 +1722,8 @@ cudaError_t launch_field_sum(const Launch& L, const double* parts, int n_parts, 
 cudaError_t launch_background_out(const Launch& L, const PlanView& v, float* bgE, float* bgV,
                                   const celeste_patch* patches) {
   if (v.n_items == 0) return cudaSuccess;
-  bg_scatter_kernel<<<grid_for(L, v.n_items, kWpb), kWpb * 32, 0, L.stream>>>(v, bgE, bgV,
-                                                                              patches);
+  bg_scatter_kernel<<<grid_for(L, v.n_items, kWpb, kOccCommit), kWpb * 32, 0, L.stream>>>(v, bgE, bgV,
+                                                                                          patches);
   return cudaGetLastError();
 }
 
