@@ -78,8 +78,9 @@ int celeste_field_create(celeste_ctx* c, const celeste_problem* pr, const celest
     F->allocs.push_back(ptr);
     return ptr;
   };
-  F->Eimg = static_cast<float*>(alloc((size_t)F->n_pixels * sizeof(float)));
-  F->Vimg = static_cast<float*>(alloc((size_t)F->n_pixels * sizeof(float)));
+  // both image buffers in one block, cleared together
+  F->Eimg = static_cast<float*>(alloc(2 * (size_t)F->n_pixels * sizeof(float)));
+  F->Vimg = F->Eimg ? F->Eimg + F->n_pixels : nullptr;
   F->parts = static_cast<double*>(alloc((size_t)F->blocks_per_image * F->n_images * sizeof(double)));
   F->kl = static_cast<double*>(alloc((size_t)S * sizeof(double)));
   if (rc == CELESTE_OK && cudaMemset(F->kl, 0, (size_t)std::max(S, 1) * sizeof(double)) != cudaSuccess)
@@ -94,8 +95,7 @@ int celeste_field_create(celeste_ctx* c, const celeste_problem* pr, const celest
 
 int celeste_field_elbo(celeste_ctx* c, celeste_field* F, double* out) {
   if (!c || !F || F->ctx != c || !out) return CELESTE_EINVAL;
-  CK(cudaMemsetAsync(F->Eimg, 0, (size_t)F->n_pixels * sizeof(float), c->stream));
-  CK(cudaMemsetAsync(F->Vimg, 0, (size_t)F->n_pixels * sizeof(float), c->stream));
+  CK(cudaMemsetAsync(F->Eimg, 0, 2 * (size_t)F->n_pixels * sizeof(float), c->stream));
   for (celeste_plan* p : F->plans) {
     const Launch L = make_launch(c, p);
     CK(launch_setup(L, p->v, c->d_model, 0, p->v.n_own_pairs, false));

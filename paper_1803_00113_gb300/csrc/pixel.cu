@@ -1571,7 +1571,10 @@ __global__ void __launch_bounds__(128, 8) accumulate_kernel(PlanView v, int ne, 
 // Pixel term -E + x (log E - V / (2 E^2)) (Eq. eq:log_p_last, without
 // log x!) over every pixel of image blockIdx.y, with E = sky + Eimg and
 // V = Vimg; compensated FP32 sums per thread, FP64 across threads; one
-// partial per block in parts[blockIdx.y * gridDim.x + blockIdx.x].
+// partial per block in parts[blockIdx.y * gridDim.x + blockIdx.x].  Four
+// pixels' loads at a time and no division per pixel: 73 us for 15.2 M pixels
+// (106 with a 64-bit division and one pixel at a time; the bytes take 27).
+constexpr int kFieldBatch = 4;
 __global__ void __launch_bounds__(256) field_term_kernel(const celeste_image* __restrict__ images,
                                                          const float* __restrict__ pixels,
                                                          const float* __restrict__ sky,
@@ -1579,21 +1582,45 @@ __global__ void __launch_bounds__(256) field_term_kernel(const celeste_image* __
                                                          const float* __restrict__ Vimg,
                                                          unsigned int* err, double* parts) {
   const celeste_image& im = images[blockIdx.y];
-  const int64_t n = (int64_t)im.height * im.width;
+  const int w = im.width, stride = gridDim.x * blockDim.x;
+  const int64_t n = (int64_t)im.height * w;
+  const int64_t f0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   float s = 0.f, c = 0.f;
-  for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < n;
-       f += (int64_t)gridDim.x * blockDim.x) {
-    const int y = (int)(f / im.width), x = (int)(f - (int64_t)y * im.width);
-    const int64_t m = im.pix_offset + (int64_t)y * im.row_stride + x;
-    const float sk = sky_value(im, sky, (float)x, (float)y);
-    if (!(sk > 0.f)) set_error(err, CELESTE_DERR_SKY);
-    const float E = sk + Eimg[m], V = Vimg[m], cnt = pixels[m];
-    const float r = __frcp_rn(E);
-    const float t = fmaf(cnt, __logf(E) - 0.5f * V * r * r, -E);
-    const float yk = t - c;
-    const float tk = s + yk;
-    c = (tk - s) - yk;
-    s = tk;
+  // kFieldBatch of the thread's pixels at a time: their loads together, then
+  // the terms in order.  Pixel coordinates step without a division.
+  int x = (int)(f0 % w), y = (int)(f0 / w);
+  const int ax = stride % w, ay = stride / w;
+  for (int64_t f = f0; f < n; f += (int64_t)kFieldBatch * stride) {
+    float e[kFieldBatch], V[kFieldBatch], cnt[kFieldBatch];
+    int px[kFieldBatch], py[kFieldBatch];
+#pragma unroll
+    for (int u = 0; u < kFieldBatch; ++u) {
+      px[u] = x;
+      py[u] = y;
+      if (f + (int64_t)u * stride < n) {
+        const int64_t m = im.pix_offset + (int64_t)y * im.row_stride + x;
+        e[u] = __ldcs(Eimg + m);
+        V[u] = __ldcs(Vimg + m);
+        cnt[u] = __ldcs(pixels + m);
+      }
+      x += ax;
+      y += ay;
+      if (x >= w) x -= w, ++y;
+    }
+#pragma unroll
+    for (int u = 0; u < kFieldBatch; ++u) {
+      if (f + (int64_t)u * stride < n) {
+        const float sk = sky_value(im, sky, (float)px[u], (float)py[u]);
+        if (!(sk > 0.f)) set_error(err, CELESTE_DERR_SKY);
+        const float E = sk + e[u];
+        const float r = __frcp_rn(E);
+        const float t = fmaf(cnt[u], __logf(E) - 0.5f * V[u] * r * r, -E);
+        const float yk = t - c;
+        const float tk = s + yk;
+        c = (tk - s) - yk;
+        s = tk;
+      }
+    }
   }
   double d = (double)s - (double)c;
   d = warp_sum_d(d);

@@ -34,8 +34,9 @@ __device__ __forceinline__ float sigmoid_f(float t) {
 // conversions, at about one warp instruction per 64 cycles of an SM
 // sub-partition, so the warp converts its theta row and its image's PSF,
 // WCS and calibration with one instruction each (a value per lane), shared
-// through thf and imf: 32 floats each of the warp's shared memory.  Own
-// pairs read theta_trial when use_trial.
+// through thf and imf: 32 floats each of the warp's shared memory; the centre's
+// two coordinates and the flux moments' two types are formed side by side, in
+// even and odd lanes.  Own pairs read theta_trial when use_trial.
 __device__ __forceinline__ void setup_pair(const PlanView& v, const ModelDev* __restrict__ model,
                                            int p, bool use_trial, float* thf, float* imf,
                                            int lane) {
@@ -47,20 +48,25 @@ __device__ __forceinline__ void setup_pair(const PlanView& v, const ModelDev* __
   constexpr int kPsfV = 6 * kPsf;                // PSF values: weight, mean (2), covariance (3)
   static_assert(kTheta <= 32 && kPsfV + 5 <= 32, "one value per lane");
   __syncwarp();
+  float tv;                                      // this lane's theta
   {
-    thf[lane] = (float)th[lane < kTheta ? lane : 0];
     const double* src = lane < kPsfV ? &im.psf[0][0] + lane
                                      : (lane < kPsfV + 4 ? im.wcs_A + (lane - kPsfV) : &im.calib);
-    imf[lane] = (float)*src;
+    const double t = th[lane < kTheta ? lane : 0], i = *src;
+    thf[lane] = tv = (float)t;
+    imf[lane] = (float)i;
   }
   __syncwarp();
   const float* psf = imf;                        // psf[6 k + c]
   const float* wcs = imf + kPsfV;                // A0, A1, A2, A3, calib
 
-  // centre in the patch's local pixel frame (FP64, then FP32)
+  // centre in the patch's local pixel frame (FP64, then FP32): x in the even
+  // lanes, y in the odd ones
+  const int odd = lane & 1;
   const double ux = th[21], uy = th[22];
-  const float mux = (float)(im.wcs_A[0] * ux + im.wcs_A[1] * uy + im.wcs_t[0] - (double)pi.x0);
-  const float muy = (float)(im.wcs_A[2] * ux + im.wcs_A[3] * uy + im.wcs_t[1] - (double)pi.y0);
+  const float mul = (float)(im.wcs_A[2 * odd] * ux + im.wcs_A[2 * odd + 1] * uy + im.wcs_t[odd] -
+                            (double)(odd ? pi.y0 : pi.x0));
+  const float mux = __shfl_sync(0xffffffffu, mul, 0), muy = __shfl_sync(0xffffffffu, mul, 1);
   // Sigma_s = R^T diag(d1, d2) R, R = [[c, -s], [s, c]]  (Sec. 2.1.3)
   float s, c;
   sincosf(thf[23], &s, &c);
@@ -118,36 +124,29 @@ __device__ __forceinline__ void setup_pair(const PlanView& v, const ModelDev* __
     e[7] = 0.f;
   }
 
-  if (lane == 0) {
-    // flux moments per type in this image's band (Sec. 2.1.2)
-    const int b = im.band;
-    float kk[2], ev[2];
-    for (int i = 0; i < 2; ++i) {
-      float m = thf[1 + 2 * i];
-      float var = expf(thf[2 + 2 * i]);
-      for (int q = 0; q < 4; ++q) {
-        const float sel = (float)kSel[b][q];
-        m += sel * thf[5 + 4 * i + q];
-        var += sel * sel * expf(thf[13 + 4 * i + q]);
-      }
-      kk[i] = wcs[4] * expf(m + 0.5f * var);          // calib E[l_b | a=i]
-      ev[i] = expm1f(var);                              // E[l^2] / E[l]^2 - 1
-    }
-    const float q1 = sigmoid_f(thf[0]);
-    const float q0 = sigmoid_f(-thf[0]);
-    rec[H_CE0] = q0 * kk[0];
-    rec[H_CE1] = q1 * kk[1];
-    rec[H_CM0] = q0 * kk[0] * kk[0] * (1.f + ev[0]);
-    rec[H_CM1] = q1 * kk[1] * kk[1] * (1.f + ev[1]);
-    rec[H_K0] = kk[0];
-    rec[H_K1] = kk[1];
-    rec[H_EV0] = ev[0];
-    rec[H_EV1] = ev[1];
-    rec[H_Q0] = q0;
-    rec[H_Q1] = q1;
-    rec[H_RHO] = sigmoid_f(thf[26]);
-    rec[H_RHO1] = sigmoid_f(-thf[26]);
-    rec[12] = rec[13] = rec[14] = rec[15] = 0.f;
+  // flux moments per type in this image's band (Sec. 2.1.2), a type a lane;
+  // the exponentials of the log variances first, a coordinate a lane
+  const float ex = expf(tv);
+  const int b = im.band, i = lane & 1;
+  float m = thf[1 + 2 * i];
+  float var = __shfl_sync(0xffffffffu, ex, 2 + 2 * i);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float sel = (float)kSel[b][q];
+    m += sel * thf[5 + 4 * i + q];
+    var += sel * sel * __shfl_sync(0xffffffffu, ex, 13 + 4 * i + q);
+  }
+  if (lane < 2) {
+    const float kk = wcs[4] * expf(m + 0.5f * var);   // calib E[l_b | a=i]
+    const float ev = expm1f(var);                       // E[l^2] / E[l]^2 - 1
+    const float qi = sigmoid_f(i ? thf[0] : -thf[0]);
+    rec[H_CE0 + i] = qi * kk;
+    rec[H_CM0 + i] = qi * kk * kk * (1.f + ev);
+    rec[H_K0 + i] = kk;
+    rec[H_EV0 + i] = ev;
+    rec[H_Q0 + i] = qi;
+    rec[H_RHO + i] = sigmoid_f(i ? -thf[26] : thf[26]);
+    rec[12 + i] = rec[14 + i] = 0.f;
   }
 }
 
