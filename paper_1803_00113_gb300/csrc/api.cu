@@ -116,11 +116,26 @@ cudaError_t derivs_launch(celeste_ctx* c, celeste_plan* p, const Launch& L) {
   return timed(c, CELESTE_K_DERIVS, p->visits, L.stream, [&] { return launch_pixels_derivs(L, p->v); });
 }
 
-int run_setup(celeste_ctx* c, celeste_plan* p, int first, int n, bool trial) {
+// The start of an evaluation of every slot: active set and records, and the
+// backgrounds where asked for.  With a render cache the background comes from
+// cached moments, so only the own pairs need records, and it joins their
+// launch.
+int run_start(celeste_ctx* c, celeste_plan* p, bool background) {
   Launch L = make_launch(c, p);
+  const PlanView& v = p->v;
   ++c->launches;
-  return to_status(timed(c, CELESTE_K_SETUP, 0, L.stream,
-                         [&] { return launch_setup(L, p->v, c->d_model, first, n, trial); }));
+  if (background && v.cache) {
+    return to_status(timed(c, CELESTE_K_BACKGROUND, p->visits, L.stream, [&] {
+      return launch_prepare(L, v, c->d_model, nullptr, v.n_own_pairs);
+    }));
+  }
+  const int n = background ? v.n_pairs : v.n_own_pairs;
+  const int rc = to_status(timed(c, CELESTE_K_SETUP, 0, L.stream,
+                                 [&] { return launch_setup(L, v, c->d_model, 0, n, false, 1); }));
+  if (rc || !background) return rc;
+  ++c->launches;
+  return to_status(timed(c, CELESTE_K_BACKGROUND, p->visits, L.stream,
+                         [&] { return launch_background(L, v); }));
 }
 
 }  // namespace
@@ -289,7 +304,7 @@ bool prepare_model(const celeste_model* m, ModelDev* md) {
 cudaError_t celeste::enqueue_iteration(celeste_ctx* c, celeste_plan* p, const Launch& L,
                                      double* delta, int32_t* status) {
   PlanView& v = p->v;
-  cudaError_t e = launch_prepare(L, v, c->d_model, status, v.n_own_pairs, false);
+  cudaError_t e = launch_setup(L, v, c->d_model, 0, v.n_own_pairs, false, 2, status);
   if (e == cudaSuccess) e = launch_pixels_derivs(L, v);
   if (e == cudaSuccess) e = launch_source_step(L, v, c->d_model, delta, status);
   if (e == cudaSuccess) e = launch_pixels_value(L, v, false);
@@ -611,13 +626,9 @@ int64_t celeste_plan_visits(const celeste_plan* p) { return p ? p->visits : -1; 
 
 static int eval_common(celeste_ctx* c, celeste_plan* p, bool derivs) {
   Launch L = make_launch(c, p);
-  CK(cudaMemsetAsync(p->v.active, 1, p->v.n > 0 ? p->v.n : 1, c->stream));
-  // with a render cache the background comes from cached moments, so only
-  // the own pairs need records
-  int rc = run_setup(c, p, 0, p->v.cache ? p->v.n_own_pairs : p->v.n_pairs, false);
+  const int rc = run_start(c, p, true);
   if (rc) return rc;
-  c->launches += 2;
-  CK(timed(c, CELESTE_K_BACKGROUND, p->visits, L.stream, [&] { return launch_background(L, p->v); }));
+  ++c->launches;
   CK(derivs ? derivs_launch(c, p, L)
             : timed(c, CELESTE_K_VALUE, p->visits, L.stream, [&] { return launch_pixels_value(L, p->v); }));
   return CELESTE_OK;
@@ -645,11 +656,9 @@ int celeste_elbo_grad(celeste_ctx* c, const celeste_plan* pc, double* elbo, doub
   if (p->v.n == 0) return CELESTE_OK;
   if (!grad) return CELESTE_EINVAL;
   Launch L = make_launch(c, p);
-  CK(cudaMemsetAsync(p->v.active, 1, p->v.n > 0 ? p->v.n : 1, c->stream));
-  int rc = run_setup(c, p, 0, p->v.n_pairs, false);
+  const int rc = run_start(c, p, true);
   if (rc) return rc;
-  c->launches += 3;
-  CK(timed(c, CELESTE_K_BACKGROUND, p->visits, L.stream, [&] { return launch_background(L, p->v); }));
+  c->launches += 2;
   CK(timed(c, CELESTE_K_GRAD, p->visits, L.stream, [&] { return launch_pixels_grad(L, p->v); }));
   return to_status(timed(c, CELESTE_K_EPILOGUE, 0, L.stream, [&] {
     return launch_epilogue_grad(L, p->v, c->d_model, elbo, elbo_rel, grad);
@@ -695,8 +704,8 @@ int celeste_newton_step(celeste_ctx* c, const celeste_plan* pc, double* delta, i
   c->launches += 1;
   CK(timed(c, cached ? CELESTE_K_BACKGROUND : CELESTE_K_SETUP, cached ? p->visits : 0, L.stream,
            [&] {
-             return launch_prepare(L, v, c->d_model, status, cached ? v.n_own_pairs : v.n_pairs,
-                                   cached);
+             return cached ? launch_prepare(L, v, c->d_model, status, v.n_own_pairs)
+                           : launch_setup(L, v, c->d_model, 0, v.n_pairs, false, 2, status);
            }));
   if (!cached) {
     c->launches += 1;
@@ -726,8 +735,7 @@ int celeste_render_cache(celeste_ctx* c, const celeste_plan* pc) {
   if (!c || !p || p->ctx != c) return CELESTE_EINVAL;
   if (p->v.n == 0 || !p->v.cache) return CELESTE_OK;
   Launch L = make_launch(c, p);
-  CK(cudaMemsetAsync(p->v.active, 1, p->v.n, c->stream));
-  int rc = run_setup(c, p, 0, p->v.n_own_pairs, false);
+  const int rc = run_start(c, p, false);
   if (rc) return rc;
   ++c->launches;
   return to_status(timed(c, CELESTE_K_RENDER, p->visits, L.stream,
@@ -746,8 +754,7 @@ int celeste_render(celeste_ctx* c, const celeste_plan* pc, float* E_out, float* 
   celeste_plan* p = const_cast<celeste_plan*>(pc);
   if (!c || !p || p->ctx != c || (!E_out && !V_out) || !p->d_patches) return CELESTE_EINVAL;
   Launch L = make_launch(c, p);
-  CK(cudaMemsetAsync(p->v.active, 1, p->v.n > 0 ? p->v.n : 1, c->stream));
-  int rc = run_setup(c, p, 0, p->v.n_own_pairs, false);
+  const int rc = run_start(c, p, false);
   if (rc) return rc;
   ++c->launches;
   return to_status(launch_render(L, p->v, E_out, V_out, p->d_patches));
@@ -757,11 +764,9 @@ int celeste_background(celeste_ctx* c, const celeste_plan* pc, float* bgE, float
   celeste_plan* p = const_cast<celeste_plan*>(pc);
   if (!c || !p || p->ctx != c || (!bgE && !bgV) || !p->d_patches) return CELESTE_EINVAL;
   Launch L = make_launch(c, p);
-  CK(cudaMemsetAsync(p->v.active, 1, p->v.n > 0 ? p->v.n : 1, c->stream));
-  int rc = run_setup(c, p, 0, p->v.n_pairs, false);
+  const int rc = run_start(c, p, true);
   if (rc) return rc;
-  c->launches += 2;
-  CK(launch_background(L, p->v));
+  ++c->launches;
   return to_status(launch_background_out(L, p->v, bgE, bgV, p->d_patches));
 }
 

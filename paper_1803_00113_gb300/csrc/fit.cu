@@ -317,9 +317,9 @@ int fit_build(celeste_fit* F) {
     // render cache the background needs no records: one launch)
     CK(begin());
     if (p->v.cache) {
-      e = launch_prepare(L, p->v, c->d_model, f.status, 0, true);
+      e = launch_prepare(L, p->v, c->d_model, f.status, 0);
     } else {
-      e = launch_prepare(L, p->v, c->d_model, f.status, p->v.n_pairs, false);
+      e = launch_setup(L, p->v, c->d_model, 0, p->v.n_pairs, false, 2, f.status);
       if (e == cudaSuccess) e = launch_background(L, p->v);
     }
     e2 = end();

@@ -145,9 +145,12 @@ struct Launch {
 };
 
 // ---- kernel launchers (one per translation unit) ------------------------
-// setup.cu: per-pair records; own pairs read theta_trial when use_trial.
+// setup.cu: per-pair records; own pairs read theta_trial when use_trial.  With
+// mark the plan's active set as well, 1 every slot, 2 from status (by source
+// id).
 cudaError_t launch_setup(const Launch& L, const PlanView& v, const ModelDev* model,
-                         int first_pair, int n_pairs, bool use_trial);
+                         int first_pair, int n_pairs, bool use_trial, int mark = 0,
+                         const int32_t* status = nullptr);
 // pixel.cu
 // Measures the resident blocks per SM of the pixel kernels (once, before any
 // stream capture; launches made earlier use 3 blocks per SM).
@@ -179,11 +182,11 @@ cudaError_t launch_field_sum(const Launch& L, const double* parts, int n_parts, 
                              int n_kl, double* out);
 // epilogue.cu: KL_s of each slot's source at theta into kl_out[source id].
 cudaError_t launch_kl(const Launch& L, const PlanView& v, const ModelDev* model, double* kl_out);
-// The start of a Newton iteration of a colour class in one launch: the
-// active set from status, the records of pairs [0, n_setup) at theta and,
-// with background (render cache only), the backgrounds of the active slots.
+// With a render cache, in one launch: the active set (from status; every slot
+// if null), the records of pairs [0, n_setup) at theta and the backgrounds of
+// the active slots.
 cudaError_t launch_prepare(const Launch& L, const PlanView& v, const ModelDev* model,
-                           const int32_t* status, int n_setup, bool background);
+                           const int32_t* status, int n_setup);
 // Copies v.trial_render into the render cache for slots whose source's
 // status is CELESTE_ST_ACCEPTED.
 cudaError_t launch_commit_render(const Launch& L, const PlanView& v, const int32_t* status);

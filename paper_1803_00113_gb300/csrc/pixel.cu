@@ -1437,40 +1437,38 @@ __global__ void __launch_bounds__(128) background_cached_kernel(PlanView v) {
   }
 }
 
-// The start of a Newton iteration of a colour class, one warp per unit of
-// work: the active set from the sources' status (a warp per 32 slots), the
-// records of pairs [0, n_setup) at theta, and, with bg set, the background
-// of every item of an active slot (the render cache supplies the
-// neighbours, so the own records are all it needs).
+// The start of an evaluation or of a Newton iteration of a colour class with
+// a render cache, one warp per unit of work: the active set (a warp per 32
+// slots; from the sources' status, every slot if that is null), the records
+// of pairs [0, n_setup) at theta, and the background of every item of an
+// active slot (the cache supplies the neighbours, so the own records are all
+// it needs).
 __global__ void __launch_bounds__(128) prepare_kernel(PlanView v, const ModelDev* __restrict__ model,
                                                       const int32_t* __restrict__ status,
-                                                      int n_setup, int bg) {
+                                                      int n_setup) {
   extern __shared__ float4 smem4[];
   float* smem = reinterpret_cast<float*>(smem4);
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
   float* rec = smem + wib * kBgCacheF;
   const int n_mark = (v.n + 31) / 32;
-  const int units = n_mark + n_setup + (bg ? v.n_items : 0);
+  const int units = n_mark + n_setup + v.n_items;
   // grid stride: its units are short, so a queue's claim would not return
   // before the next unit (measured 11 % slower)
-  WarpQueue wq(nullptr);
-  for (; wq.it < units; wq.advance()) {
-    wq.ask(lane);
-    const int u = wq.it;
+  const int nwarps = gridDim.x * (blockDim.x >> 5);
+  for (int u = blockIdx.x * (blockDim.x >> 5) + wib; u < units; u += nwarps) {
     if (u < n_mark) {
       const int j = 32 * u + lane;
-      if (j < v.n) v.active[j] = active_of(status[v.src_ids[j]]);
+      if (j < v.n) v.active[j] = status ? active_of(status[v.src_ids[j]]) : 1;
     } else if (u < n_mark + n_setup) {
       setup_pair(v, model, u - n_mark, false, rec, rec + 32, lane);
     } else {
       const Item item = v.items[u - n_mark - n_setup];
       const PairInfo pi = v.pairs[item.pair];
-      if (!active_of(status[pi.source])) continue;
+      if (status && !active_of(status[pi.source])) continue;
       background_cached(v, item, pi, rec, lane);
     }
   }
-  wq.done(lane);
 }
 
 // The loop of the render kernels: f(item, pair info) for every item.
@@ -1784,10 +1782,14 @@ static int grid_for(const Launch& L, int n_items, int wpb, int occ_kind = -1) {
 
 // The work queue pays when a launch has many items per warp (its claims
 // then balance the warps' finishing times); with few, the grid-stride form
-// (fewer registers, no claims) is faster.
-constexpr int kQueueItemsPerWarp = 8;
-static bool use_queue(const PlanView& v, int blocks) {
-  return v.work_ctr && v.n_items >= kQueueItemsPerWarp * kWpb * blocks;
+// (fewer registers, no claims) is faster: from five items a warp in the
+// derivative and value passes (batched field 12.57 -> 12.48 ms a pass for
+// 2,000 sources against a line at eight; at three the sampler's value pass
+// of 800 chains loses 4 %), from three in the gradient and rendering kernels
+// (1,024 field sources: gradient 138 -> 129 us, backgrounds 50 -> 45).
+constexpr int kQueueItems = 5, kQueueItemsRender = 3;
+static bool use_queue(const PlanView& v, int blocks, int per_warp = kQueueItems) {
+  return v.work_ctr && v.n_items >= per_warp * kWpb * blocks;
 }
 
 // Leaving out vanished pairs pays where pixels lie far from their source and
@@ -1805,10 +1807,11 @@ static bool use_skip(const Launch& L, const PlanView& v) {
 // a compile-time constant: with the work queue where the grid has many items
 // per warp (occ_q: that form's occupancy).
 template <class F>
-static cudaError_t launch_items(const Launch& L, const PlanView& v, int occ, int occ_q, F&& kernel) {
+static cudaError_t launch_items(const Launch& L, const PlanView& v, int occ, int occ_q,
+                                int per_warp, F&& kernel) {
   if (v.n_items == 0) return cudaSuccess;
   const int gq = grid_for(L, v.n_items, kWpb, occ_q);
-  if (use_queue(v, gq)) kernel(std::true_type(), gq);
+  if (use_queue(v, gq, per_warp)) kernel(std::true_type(), gq);
   else kernel(std::false_type(), grid_for(L, v.n_items, kWpb, occ));
   return cudaGetLastError();
 }
@@ -1819,7 +1822,7 @@ cudaError_t launch_background(const Launch& L, const PlanView& v) {
                                smem_bytes_cached(kWpb), L.stream>>>(v);
     return cudaGetLastError();
   }
-  return launch_items(L, v, kOccBackground, kOccBackground, [&](auto q, int grid) {
+  return launch_items(L, v, kOccBackground, kOccBackground, kQueueItemsRender, [&](auto q, int grid) {
     background_kernel<decltype(q)::value>
         <<<grid, kWpb * 32, smem_bytes_bg(kWpb), L.stream>>>(v, L.n_exp, L.n_dev);
   });
@@ -1850,7 +1853,7 @@ cudaError_t launch_pixels_derivs(const Launch& L, const PlanView& v) {
 cudaError_t launch_pixels_grad(const Launch& L, const PlanView& v) {
   if (v.n_items == 0) return cudaSuccess;
   const int gq = grid_for(L, v.n_items, kWpb, kOccGradQ);
-  if (use_queue(v, gq))
+  if (use_queue(v, gq, kQueueItemsRender))
     grad_kernel<true><<<gq, kWpb * 32, smem_bytes_grad(kWpb), L.stream>>>(v, L.n_exp, L.n_dev);
   else
     grad_kernel<false><<<grid_for(L, v.n_items, kWpb, kOccGrad), kWpb * 32, smem_bytes_grad(kWpb),
@@ -1865,18 +1868,18 @@ cudaError_t launch_pixels_value(const Launch& L, const PlanView& v, bool keep_re
     value_coop_kernel<<<v.n_items, kCoopThreads, 0, L.stream>>>(v, L.n_exp, L.n_dev, mode);
     return cudaGetLastError();
   }
-  return launch_items(L, v, kOccValue, kOccValueQ, [&](auto q, int grid) {
+  return launch_items(L, v, kOccValue, kOccValueQ, kQueueItems, [&](auto q, int grid) {
     value_kernel<decltype(q)::value>
         <<<grid, kWpb * 32, smem_bytes(kWpb), L.stream>>>(v, L.n_exp, L.n_dev, mode);
   });
 }
 
 cudaError_t launch_prepare(const Launch& L, const PlanView& v, const ModelDev* model,
-                           const int32_t* status, int n_setup, bool background) {
-  const int units = (v.n + 31) / 32 + n_setup + (background ? v.n_items : 0);
+                           const int32_t* status, int n_setup) {
+  const int units = (v.n + 31) / 32 + n_setup + v.n_items;
   if (units == 0) return cudaSuccess;
   prepare_kernel<<<grid_for(L, units, kWpb, kOccPrepare), kWpb * 32, smem_bytes_cached(kWpb),
-                   L.stream>>>(v, model, status, n_setup, background ? 1 : 0);
+                   L.stream>>>(v, model, status, n_setup);
   return cudaGetLastError();
 }
 
@@ -1889,7 +1892,7 @@ cudaError_t launch_commit_render(const Launch& L, const PlanView& v, const int32
 
 cudaError_t launch_render(const Launch& L, const PlanView& v, float* E_out, float* V_out,
                           const celeste_patch* patches) {
-  return launch_items(L, v, kOccRender, kOccRender, [&](auto q, int grid) {
+  return launch_items(L, v, kOccRender, kOccRender, kQueueItemsRender, [&](auto q, int grid) {
     render_kernel<decltype(q)::value>
         <<<grid, kWpb * 32, smem_bytes(kWpb), L.stream>>>(v, L.n_exp, L.n_dev, E_out, V_out, patches);
   });
@@ -1897,14 +1900,14 @@ cudaError_t launch_render(const Launch& L, const PlanView& v, float* E_out, floa
 
 cudaError_t launch_render_cache(const Launch& L, const PlanView& v, const int32_t* status) {
   if (!v.cache) return cudaSuccess;
-  return launch_items(L, v, kOccRender, kOccRender, [&](auto q, int grid) {
+  return launch_items(L, v, kOccRender, kOccRender, kQueueItemsRender, [&](auto q, int grid) {
     render_cache_kernel<decltype(q)::value>
         <<<grid, kWpb * 32, smem_bytes(kWpb), L.stream>>>(v, L.n_exp, L.n_dev, status);
   });
 }
 
 cudaError_t launch_accumulate(const Launch& L, const PlanView& v, float* Eimg, float* Vimg) {
-  return launch_items(L, v, kOccRender, kOccRender, [&](auto q, int grid) {
+  return launch_items(L, v, kOccRender, kOccRender, kQueueItemsRender, [&](auto q, int grid) {
     accumulate_kernel<decltype(q)::value>
         <<<grid, kWpb * 32, smem_bytes(kWpb), L.stream>>>(v, L.n_exp, L.n_dev, Eimg, Vimg);
   });

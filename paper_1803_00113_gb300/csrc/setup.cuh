@@ -36,14 +36,11 @@ __device__ __forceinline__ float sigmoid_f(float t) {
 // WCS and calibration with one instruction each (a value per lane), shared
 // through thf and imf: 32 floats each of the warp's shared memory; the centre's
 // two coordinates and the flux moments' two types are formed side by side, in
-// even and odd lanes.  Own pairs read theta_trial when use_trial.
+// even and odd lanes.  image, x0, y0: the pair's; th: its source's theta.
 __device__ __forceinline__ void setup_pair(const PlanView& v, const ModelDev* __restrict__ model,
-                                           int p, bool use_trial, float* thf, float* imf,
-                                           int lane) {
-  const PairInfo pi = v.pairs[p];
-  const celeste_image& im = v.images[pi.image];
-  const double* th = (use_trial && pi.slot >= 0) ? v.theta_trial + (size_t)pi.slot * kTheta
-                                                 : v.theta + (size_t)pi.source * kTheta;
+                                           int p, int image, int x0, int y0, const double* th,
+                                           float* thf, float* imf, int lane) {
+  const celeste_image& im = v.images[image];
   float* rec = v.records + (size_t)p * kRecF;
   constexpr int kPsfV = 6 * kPsf;                // PSF values: weight, mean (2), covariance (3)
   static_assert(kTheta <= 32 && kPsfV + 5 <= 32, "one value per lane");
@@ -65,7 +62,7 @@ __device__ __forceinline__ void setup_pair(const PlanView& v, const ModelDev* __
   const int odd = lane & 1;
   const double ux = th[21], uy = th[22];
   const float mul = (float)(im.wcs_A[2 * odd] * ux + im.wcs_A[2 * odd + 1] * uy + im.wcs_t[odd] -
-                            (double)(odd ? pi.y0 : pi.x0));
+                            (double)(odd ? y0 : x0));
   const float mux = __shfl_sync(0xffffffffu, mul, 0), muy = __shfl_sync(0xffffffffu, mul, 1);
   // Sigma_s = R^T diag(d1, d2) R, R = [[c, -s], [s, c]]  (Sec. 2.1.3)
   float s, c;
@@ -148,6 +145,15 @@ __device__ __forceinline__ void setup_pair(const PlanView& v, const ModelDev* __
     rec[H_RHO + i] = sigmoid_f(i ? -thf[26] : thf[26]);
     rec[12 + i] = rec[14 + i] = 0.f;
   }
+}
+
+__device__ __forceinline__ void setup_pair(const PlanView& v, const ModelDev* __restrict__ model,
+                                           int p, bool use_trial, float* thf, float* imf,
+                                           int lane) {
+  const PairInfo& pi = v.pairs[p];
+  const double* th = use_trial && pi.slot >= 0 ? v.theta_trial + (size_t)pi.slot * kTheta
+                                               : v.theta + (size_t)pi.source * kTheta;
+  setup_pair(v, model, p, pi.image, pi.x0, pi.y0, th, thf, imf, lane);
 }
 
 }  // namespace celeste

@@ -92,10 +92,28 @@ __global__ void __launch_bounds__(kTrThreads, 5) source_step_kernel(PlanView v,
     kl_terms<0, false>(S.e.th, S.f, n_color, S.e, lane);
     if (lane == 0) v.kl_trial[j] = (double)S.e.kls[0];
   } else {
-    // each warp's 64 floats of the Hessian scratch, which KL_s does not use
+    // each warp's 64 floats of the Hessian scratch, which KL_s does not use.
+    // A warp's pairs (every third) are looked up a lane each, and their images
+    // asked into the cache, before the first is set up.
     float* scratch = S.e.Hnu + (wid - 1) * 64;
-    for (int p = v.slot_pair_ptr[j] + wid - 1; p < v.slot_pair_ptr[j + 1]; p += 3)
-      setup_pair(v, model, p, true, scratch, scratch + 32, lane);
+    const double* th = v.theta_trial + (size_t)j * kTheta;
+    const int p1 = v.slot_pair_ptr[j + 1];
+    for (int pb = v.slot_pair_ptr[j] + wid - 1; pb < p1; pb += 96) {
+      int image = 0, x0 = 0, y0 = 0;
+      if (pb + 3 * lane < p1) {
+        const PairInfo& pi = v.pairs[pb + 3 * lane];
+        image = pi.image;
+        x0 = pi.x0;
+        y0 = pi.y0;
+        const char* im = reinterpret_cast<const char*>(v.images + image);
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(im));
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(im + 128));
+      }
+      for (int m = 0; m < 32 && pb + 3 * m < p1; ++m)
+        setup_pair(v, model, pb + 3 * m, __shfl_sync(0xffffffffu, image, m),
+                   __shfl_sync(0xffffffffu, x0, m), __shfl_sync(0xffffffffu, y0, m), th, scratch,
+                   scratch + 32, lane);
+    }
   }
 }
 
