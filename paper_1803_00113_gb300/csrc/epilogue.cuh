@@ -31,8 +31,8 @@
 // come to shared memory in asynchronous copies, maps and indices are formed
 // without branches (a divergent 18-way choice of map entries alone took 4k
 // cycles a pair), and every small dense product is spread over all threads.
-// One source with one 41 x 41 patch per band: 27k cycles (53k before) for
-// value, gradient and Hessian; with two 61 x 61 patches per band: 34k (84k).
+// One source with one 41 x 41 patch per band: 25k cycles (53k before) for
+// value, gradient and Hessian; with two 61 x 61 patches per band: 31k (84k).
 #pragma once
 
 #include <math.h>
@@ -42,9 +42,6 @@
 namespace celeste {
 
 typedef float real;
-
-static __constant__ signed char kSelE[5][4] = {
-    {-1, -1, 0, 0}, {0, -1, 0, 0}, {0, 0, 0, 0}, {0, 0, 1, 0}, {0, 0, 1, 1}};
 
 constexpr int kNu = 26;   // 20 flux moments (band b, kind e at 4b+e), u (2), Sigma_s (3), rho
 constexpr int kNuPad = 32;
@@ -88,16 +85,17 @@ struct EpiSmem {
   float W[kPairGroup][kAcc];       // per pair of a group: zero, then the other sums (2..63)
   float T[kPairGroup][10 * 10];    // per pair of a group: affine map w <- nu (local)
   alignas(16) float tiles[2][kTileChunk][kAcc];   // tile sums on their way in
+  float img[5 * kPairGroup];       // per pair of a group: calibration and A, FP32
   int band[kPairGroup];
   real pw[2 * kKlSums];            // colour bound: pi-weighted sums per type
   real th[kNuPad];                 // theta of the source (FP32 copy)
   real gnu[kNuPad];
   real Hnu[kNu * kNu];
   real J[kNu * kTheta];
-  real X[kNu * kTheta];
+  real X[kNu * kTheta + kTheta];   // (padded: read, not used, past the last row)
   real gth[kNuPad];
   real Hth[kTheta * kTheta];
-  real DL[20 * kTheta];            // d log kappa_a / d theta
+  real DL[20 * kTheta + kTheta];   // d log kappa_a / d theta (padded)
   real D2L[20 * kTheta];           // diagonal second derivatives of log kappa_a
   real kap[kNuPad];                // kappa_a
   real kw[kNuPad];                 // grad_nu[a] * kappa_a
@@ -142,7 +140,7 @@ static __device__ void kappa_row(const real* th, int a, EpiSmem& S) {
   real lm[4], lc[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const real s = (real)kSelE[b][k];
+    const real s = colour_select(b, k);
     const real cvk = expf(th[13 + 4 * i + k]);
     m += s * th[5 + 4 * i + k];
     v += s * s * cvk;
@@ -236,7 +234,7 @@ static __device__ __forceinline__ void kl_lone_terms(const real* th, const Model
 // probability, radius, axis and profile alone is ADDED (with a minus sign,
 // since L = ... - KL) into S.gth and S.Hth, and the rest left in S.pw and
 // S.klt for kl_scatter.  By one warp; f and J are the model's FP32 constants
-// and its number of colour components.  kApart: warp 3 forms the lone terms
+// and its number of colour components.  kApart: warp 2 forms the lone terms
 // and meets this warp at named barrier 3.
 template <int kMode, bool kApart>
 static __device__ void kl_terms(const real* th, const ModelDev::F32& f, int J, EpiSmem& S,
@@ -388,9 +386,9 @@ static __device__ void kl_terms(const real* th, const ModelDev::F32& f, int J, E
 
 // The rest of the KL's gradient and Hessian, from S.pw and S.klt: the
 // blocks of each type's flux coordinates and their products with the type
-// probability, an entry a thread of the block.
+// probability, an entry a lane.
 template <int kMode>
-static __device__ __forceinline__ void kl_scatter(const real* th, EpiSmem& S, int tid) {
+static __device__ __forceinline__ void kl_scatter(const real* th, EpiSmem& S, int lane) {
   const real a = sigm(th[0]);
   const real wq = a * (1.f - a);
   // per type i, local coordinates 0 r-mean, 1 log r-var, 2..5 colour means,
@@ -399,7 +397,7 @@ static __device__ __forceinline__ void kl_scatter(const real* th, EpiSmem& S, in
     return k == 0 ? 1 + 2 * i : (k == 1 ? 2 + 2 * i : (k < 6 ? 5 + 4 * i + (k - 2) : 13 + 4 * i + (k - 6)));
   };
   // gradient-only mode visits the (i, k, l = 0) entries only
-  for (int e0 = tid; e0 < (kMode == 2 ? 200 : 20); e0 += kEpiThreads) {
+  for (int e0 = lane; e0 < (kMode == 2 ? 200 : 20); e0 += 32) {
     const int e = kMode == 2 ? e0 : (e0 / 10) * 100 + (e0 % 10) * 10;
     const int i = e / 100, k = (e % 100) / 10, l = e % 10;
     const real* pw = S.pw + i * kKlSums;       // grad(8), centred outer(36), prec(10), diag(4)
@@ -469,7 +467,10 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
   }
   __syncthreads();
   if (wid == 0) {
-    if (!pixel_only) kl_terms<kMode, (kMode >= 1)>(th, f, n_color, S, lane);
+    if (!pixel_only) {
+      kl_terms<kMode, (kMode >= 1)>(th, f, n_color, S, lane);
+      if (kMode >= 1) kl_scatter<kMode>(th, S, lane);
+    }
   } else {
     const int u = tid - 32;                            // 0 .. kPairThreads - 1
     double vr = 0.0, vb = 0.0;
@@ -514,30 +515,6 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
         S.vsum[1] = S.red[1][0] + S.red[1][1] + S.red[1][2];
       }
     } else {
-      if (wid == 3) {
-        kl_lone_terms<kMode>(th, f, S, lane);
-        asm volatile("bar.arrive 3, 64;" ::: "memory");
-        if (lane < 20) {
-          kappa_row(th, lane, S);
-        } else if (lane < 22) {
-          S.J[lane * kTheta + 21 + (lane - 20)] = 1.f;
-        } else if (lane == 22) {
-          real dS[3][3], d2S[3][3][3];
-          sigma_derivs(th, dS, d2S);
-#pragma unroll
-          for (int e = 0; e < 3; ++e)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              S.J[(22 + e) * kTheta + 23 + c] = dS[e][c];
-#pragma unroll
-              for (int d = 0; d < 3; ++d) S.d2S[9 * e + 3 * c + d] = d2S[e][c][d];
-            }
-        } else if (lane == 25) {
-          const real r = sigm(th[26]);
-          S.J[25 * kTheta + 26] = r * (1.f - r);
-        }
-        __syncwarp();
-      }
       // thread u's entry of H_nu (upper triangle of the ten w, u < 55) or of
       // grad_nu (the next ten): the terms of its sum over the w, as offsets
       // into T and W; terms it does not have multiply entry 0 of W, zero
@@ -564,6 +541,33 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
         const bool on = q / 3 < na3 && q % 3 < nc3 && !zero;
         wo[q] = !on ? 0 : (ghess ? hidx(kk, ll) : 2 + k);
       }
+      // what depends on theta alone, while the first loads are on their way:
+      // the KL's lone terms (warp 2), the geometric rows of J (warp 1) and its
+      // flux rows (warp 3)
+      auto apart = [&] {
+        if (wid == 2) {
+          kl_lone_terms<kMode>(th, f, S, lane);
+          asm volatile("bar.arrive 3, 64;" ::: "memory");
+        } else if (wid == 3) {
+          if (lane < 20) kappa_row(th, lane, S);
+        } else if (lane == 0) {
+          real dS[3][3], d2S[3][3][3];
+          sigma_derivs(th, dS, d2S);
+#pragma unroll
+          for (int e = 0; e < 3; ++e)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+              S.J[(22 + e) * kTheta + 23 + c] = dS[e][c];
+#pragma unroll
+              for (int d = 0; d < 3; ++d) S.d2S[9 * e + 3 * c + d] = d2S[e][c][d];
+            }
+          S.J[20 * kTheta + 21] = S.J[21 * kTheta + 22] = 1.f;
+          const real r = sigm(th[26]);
+          S.J[25 * kTheta + 26] = r * (1.f - r);
+        }
+        __syncwarp();
+      };
+      if (p0 == p1) apart();
       for (int pp = p0; pp < p1; pp += kPairGroup) {
         const int ng = min(kPairGroup, p1 - pp);
         int ib = 0, ie = 0, im = 0;
@@ -592,6 +596,7 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
           };
           const int nc = (t1 - t0 + kTileChunk - 1) / kTileChunk;
           fetch(0);
+          if (pp == p0) apart();
           int g = wid - 1;
           float2 s = make_float2(0.f, 0.f), c = s;
           for (int ch = 0; ch < nc; ++ch) {
@@ -641,35 +646,39 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
         } else {
           // each pair's local affine map, FP32: w_k = sum_a T[k][a] nu_a;
           // five values of an image (calibration, A) in five lanes, so that
-          // six images share a conversion.  Lanes 0..17 form an entry each,
-          // from values i1 and i2 (three bits a lane): kind 0 the value i1, 1
-          // the product, 2 twice it, 3 A0 A3 + A1 A2, 4 one
-          constexpr uint64_t kKind = 0412113112100001100ull, kOne = 043321121143210000ull, kTwo = 044344322100000000ull;
-          const int sh = 3 * min(lane, 17), bl = lane - 8;
-          const int kind = (int)(kKind >> sh & 7), i1 = (int)(kOne >> sh & 7), i2 = (int)(kTwo >> sh & 7);
-          const int te = lane < 4 ? 11 * lane
-                                  : (lane < 8 ? 44 + ((lane - 4) >> 1) * 10 + (lane & 1)
-                                              : (lane < 17 ? 66 + bl / 3 * 10 + bl % 3 : 99));
-          for (int g0 = 0; g0 < ng; g0 += 6) {
-            const int g = g0 + lane / 5, q = lane % 5;
-            const int image = __shfl_sync(0xffffffffu, im, min(g, ng - 1));
-            float x = 0.f;
-            if (lane < 30) {
-              const celeste_image& I = v.images[image];
-              x = (float)(q == 0 ? I.calib : I.wcs_A[q - 1]);
-            }
-            for (int h = 0; h < min(6, ng - g0); ++h) {
-              const float f1 = __shfl_sync(0xffffffffu, x, 5 * h + i1);
-              const float f2 = __shfl_sync(0xffffffffu, x, 5 * h + i2);
-              const float f3 = __shfl_sync(0xffffffffu, x, 5 * h + 2);
-              const float f4 = __shfl_sync(0xffffffffu, x, 5 * h + 3);
-              float t = f1 * f2;
-              if (kind == 0) t = f1;
-              if (kind == 2) t = 2.f * f1 * f2;
-              if (kind == 3) t = f1 * f2 + f3 * f4;
-              if (kind == 4) t = 1.f;
-              if (lane < 18) S.T[g0 + h][te] = t;
-            }
+          // six images share a conversion; then an entry (of the eighteen that
+          // are not zero) of a pair a lane, from two of the values (three bits
+          // an entry in kOne, kTwo): kind 0 the first, 1 the product, 2 twice
+          // it, 3 A0 A3 + A1 A2, 4 one
+          static_assert(kPairGroup == 12, "two conversions");
+          double raw[2];
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const int q = lane % 5;
+            const int image = __shfl_sync(0xffffffffu, im, min(6 * c + min(lane / 5, 5), ng - 1));
+            const celeste_image& I = v.images[image];
+            raw[c] = q == 0 ? I.calib : I.wcs_A[q - 1];
+          }
+          if (pp == p0) apart();
+#pragma unroll
+          for (int c = 0; c < 2; ++c)
+            if (lane < 30) S.img[30 * c + lane] = (float)raw[c];
+          __syncwarp();
+          constexpr uint64_t kKind = 0412113112100001100ull, kOne = 043321121143210000ull,
+                             kTwo = 044344322100000000ull;
+          for (int q = lane; q < 18 * ng; q += 32) {
+            const int g = q / 18, e = q - 18 * g, sh = 3 * e;
+            const int kind = (int)(kKind >> sh & 7);
+            const float* I = S.img + 5 * g;
+            const float f1 = I[kOne >> sh & 7], f2 = I[kTwo >> sh & 7], f3 = I[2], f4 = I[3];
+            const float t = kind == 0 ? f1
+                                      : (kind == 1 ? f1 * f2
+                                                   : (kind == 2 ? 2.f * f1 * f2
+                                                                : (kind == 3 ? fmaf(f3, f4, __fmul_rn(f1, f2)) : 1.f)));
+            const int te = e < 4 ? 11 * e
+                                 : (e < 8 ? 44 + ((e - 4) >> 1) * 10 + (e & 1)
+                                          : (e < 17 ? 66 + (e - 8) / 3 * 10 + (e - 8) % 3 : 99));
+            S.T[g][te] = t;
           }
         }
         pair_sync();
@@ -704,6 +713,18 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
         }
         if (pp + kPairGroup < p1) pair_sync();
       }
+      // the lower triangle of H_nu, by the threads that formed the upper one
+      if (kMode == 2 && ghess && ea != ec) {
+        if (ea >= 4) {
+          S.Hnu[(16 + ec) * kNu + 16 + ea] = S.Hnu[(16 + ea) * kNu + 16 + ec];
+        } else {
+#pragma unroll
+          for (int b = 0; b < 5; ++b) {
+            const int na = 4 * b + ea, nc = ec < 4 ? 4 * b + ec : 16 + ec;
+            S.Hnu[nc * kNu + na] = S.Hnu[na * kNu + nc];
+          }
+        }
+      }
       if (wid == 1 && lane < 2) S.vsum[lane] = vr;
     }
   }
@@ -712,13 +733,7 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
   rel = S.vsum[0] - kl;
   full = S.vsum[1] + S.vsum[0] - kl;
   if (kMode >= 1) {
-    kl_scatter<kMode>(th, S, tid);
     if (kMode == 2) {
-      // the lower triangle of H_nu
-      for (int e = tid; e < kNu * kNu; e += kEpiThreads) {
-        const int a = e / kNu, c = e - a * kNu;
-        if (a > c) S.Hnu[e] = S.Hnu[c * kNu + a];
-      }
       if (tid < 20) S.kw[tid] = S.gnu[tid] * S.kap[tid];
       __syncthreads();
       // X = H_nu J where J's column has support.  Columns 0..20 (ten or
@@ -774,44 +789,62 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
     }
     if (kMode == 2) {
       // Hth += J^T X over d >= c (mirrored), plus the flux-moment
-      // second-order term sum_a kw_a (dl dl^T + diag d2l): thread (c, g)
-      // takes d = c + g, c + g + 4, ..., seven chains
-      if (tid < 4 * kTheta) {
-        const int c = tid % kTheta, g = tid / kTheta, nr = nrows(c);
+      // second-order term sum_a kw_a (dl dl^T + diag d2l).  Column 0 (twenty
+      // rows) has a thread for each d; thread (c, g) of the others takes d =
+      // c + g, c + g + 3, ..., nine chains sharing the entries of column c.
+      auto entry = [&](int c, int d, real x) {
+        S.Hth[c * kTheta + d] += x;
+        if (d != c) S.Hth[d * kTheta + c] += x;
+      };
+      if (tid < kTheta) {
+        const int d = tid;
+        real x = 0.f;
+#pragma unroll 10
+        for (int r = 0; r < 20; ++r) x = fmaf(S.J[r * kTheta], S.X[r * kTheta + d], x);
+        if (d <= 20) {
+#pragma unroll 10
+          for (int r = 0; r < 20; ++r) {
+            const real kd = S.kw[r] * S.DL[r * kTheta];
+            x = fmaf(kd, S.DL[r * kTheta + d], x);
+            if (d == 0) x = fmaf(S.kw[r], S.D2L[r * kTheta], x);
+          }
+        }
+        entry(0, d, x);
+      } else if (tid < kTheta + 3 * (kTheta - 1)) {
+        constexpr int kCh = 9;
+        const int c = 1 + (tid - kTheta) % (kTheta - 1), g = (tid - kTheta) / (kTheta - 1);
+        const int nr = nrows(c);
         int r0, dr;
         rows_of(c, r0, dr);
-        real x[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        int d[7];
+        const int step = dr * kTheta;
+        real x[kCh];
 #pragma unroll
-        for (int m = 0; m < 7; ++m) d[m] = min(c + g + 4 * m, kTheta - 1);
-        int r = r0;
-#pragma unroll 5
-        for (int k = 0; k < nr; ++k, r += dr) {
-          const real jv = S.J[r * kTheta + c];
+        for (int m = 0; m < kCh; ++m) x[m] = 0.f;
+        // (chains with d past the last column run on what follows and are
+        // dropped; DL's columns beyond 20 are zero)
+        const real* Jc = S.J + r0 * kTheta + c;
+        const real* Xd = S.X + r0 * kTheta + c + g;
+#pragma unroll 2
+        for (int k = 0; k < nr; ++k, Jc += step, Xd += step) {
+          const real jv = *Jc;
 #pragma unroll
-          for (int m = 0; m < 7; ++m) x[m] = fmaf(jv, S.X[r * kTheta + d[m]], x[m]);
+          for (int m = 0; m < kCh; ++m) x[m] = fmaf(jv, Xd[3 * m], x[m]);
         }
         if (c <= 20) {
-          r = r0;
-#pragma unroll 5
-          for (int k = 0; k < nr; ++k, r += dr) {
-            const real kd = S.kw[r] * S.DL[r * kTheta + c];
-            const real xd = fmaf(kd, S.DL[r * kTheta + d[0]], x[0]);
-            x[0] = g == 0 ? fmaf(S.kw[r], S.D2L[r * kTheta + c], xd) : (d[0] <= 20 ? xd : x[0]);
+          const real* kw = S.kw + r0;
+          const real* Lc = S.DL + r0 * kTheta + c;
+          const real* L2 = S.D2L + r0 * kTheta + c;
+#pragma unroll 2
+          for (int k = 0; k < nr; ++k, kw += dr, Lc += step, L2 += step) {
+            const real kd = *kw * *Lc;
 #pragma unroll
-            for (int m = 1; m < 7; ++m) {
-              const real xm = fmaf(kd, S.DL[r * kTheta + d[m]], x[m]);
-              if (d[m] <= 20) x[m] = xm;
-            }
+            for (int m = 0; m < kCh; ++m) x[m] = fmaf(kd, Lc[g + 3 * m], x[m]);
+            if (g == 0) x[0] = fmaf(*kw, *L2, x[0]);
           }
         }
 #pragma unroll
-        for (int m = 0; m < 7; ++m) {
-          if (c + g + 4 * m < kTheta) {
-            S.Hth[c * kTheta + d[m]] += x[m];
-            if (d[m] != c) S.Hth[d[m] * kTheta + c] += x[m];
-          }
-        }
+        for (int m = 0; m < kCh; ++m)
+          if (c + g + 3 * m < kTheta) entry(c, c + g + 3 * m, x[m]);
       }
     }
     __syncthreads();

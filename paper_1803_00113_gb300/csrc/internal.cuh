@@ -275,6 +275,13 @@ __device__ __forceinline__ uint8_t active_of(int32_t st) {
                                                                                              : 1;
 }
 
+// l_b = r * exp(sum_k colour_select(b, k) c_k), colours c_k = log(l_{k+1} /
+// l_k), r = l_2.  (Computed: a table in constant memory costs its reader a
+// miss per block.)
+__device__ __forceinline__ float colour_select(int b, int k) {
+  return k < 2 ? (b <= k ? -1.f : 0.f) : (b > k ? 1.f : 0.f);
+}
+
 // Offset of source s's current half of the render cache.
 __device__ __forceinline__ int64_t cache_base(const PlanView& v, int s) {
   return v.cache_half && v.cache_half[s] ? v.cache_n_pool : 0;

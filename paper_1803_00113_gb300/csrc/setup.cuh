@@ -19,10 +19,6 @@
 
 namespace celeste {
 
-// l_b = r * exp(sum_k kSel[b][k] c_k), colours c_k = log(l_{k+1} / l_k), r = l_2
-static __constant__ signed char kSel[5][4] = {
-    {-1, -1, 0, 0}, {0, -1, 0, 0}, {0, 0, 0, 0}, {0, 0, 1, 0}, {0, 0, 1, 1}};
-
 __device__ __forceinline__ float sigmoid_f(float t) {
   return t >= 0.f ? 1.f / (1.f + expf(-t)) : expf(t) / (1.f + expf(t));
 }
@@ -129,7 +125,7 @@ __device__ __forceinline__ void setup_pair(const PlanView& v, const ModelDev* __
   float var = __shfl_sync(0xffffffffu, ex, 2 + 2 * i);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const float sel = (float)kSel[b][q];
+    const float sel = colour_select(b, q);
     m += sel * thf[5 + 4 * i + q];
     var += sel * sel * __shfl_sync(0xffffffffu, ex, 13 + 4 * i + q);
   }
