@@ -272,7 +272,7 @@ int celeste_lbfgs_step(celeste_ctx* c, celeste_lbfgs* B, int32_t* status, const 
   CK(launch_epilogue_value(L, v, c->d_model, nullptr, B->rel_trial, true));
   lbfgs_accept_kernel<<<nb, 128, 0, L.stream>>>(v, B->L, B->rel_trial, target, status);
   CK(cudaGetLastError());
-  c->launches += 11;
+  c->launches += v.nbr_render ? 12 : 11;
   return CELESTE_OK;
 }
 

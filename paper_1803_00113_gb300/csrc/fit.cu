@@ -429,12 +429,13 @@ int fit_pass_finish(celeste_ctx* c, celeste_fit* F, int* n_active) {
   *n_active = 0;
   if (f.n_region == 0) return CELESTE_OK;
   CK(cudaStreamSynchronize(c->stream));
-  // launches of the pass: reset and summary, per class 2 (with a render
-  // cache: 1, and 2 to refresh it at the end) + the loop trips
+  // launches of the pass: reset and summary, per class 2 (3 where neighbours
+  // are rendered once; with a render cache 1, and 2 to refresh it at the end)
+  // + the loop trips
   int64_t nl = 2;
   const int per_class = F->plans.empty() || !F->plans[0]->v.cache ? 2 : 3;
   for (int k = 0; k < f.n_classes; ++k)
-    nl += per_class + (int64_t)F->h_summary[1 + k] * kIterationLaunches;
+    nl += per_class + (F->plans[k]->v.nbr_render ? 1 : 0) + (int64_t)F->h_summary[1 + k] * kIterationLaunches;
   c->launches += nl;
   *n_active = F->h_summary[0];
   return CELESTE_OK;

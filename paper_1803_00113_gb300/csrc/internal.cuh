@@ -53,8 +53,10 @@ struct PairInfo {
   int64_t pix_base;    // index of pixel (x0, y0) in the pixel pool
   int32_t stride;
   int32_t band;
-  int64_t bg_base;     // own pairs: offset in the plan's background pool
-  int32_t nbr_begin, nbr_end;  // own pairs: neighbour pairs in pair_nbr[]
+  int64_t bg_base;     // own pairs: offset in the plan's background pool;
+                       // neighbour pairs: offset in nbr_render
+  int32_t nbr_begin, nbr_end;  // own pairs: neighbour pairs in pair_nbr[]; with
+                               // nbr_render, neighbour pairs: slots that use it
   int32_t item_begin, item_end;
 };
 
@@ -130,6 +132,9 @@ struct PlanView {
                               //     current moments (two halves of cache_n_pool), or null
   int64_t cache_n_pool;       // float2 per half
   float2* trial_render;       // [n_bg] own moments at the trial point (with a cache)
+  float2* nbr_render;         // neighbour pairs' moments over their whole patches, or null
+  const Item* nbr_items;      // [n_nbr_items] their work items
+  int32_t n_nbr_items;
   const celeste_patch* patches;  // problem patches (pool offsets)
   int32_t n, n_pairs, n_own_pairs, n_items;
   int64_t n_bg;

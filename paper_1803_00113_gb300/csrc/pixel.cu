@@ -1321,8 +1321,8 @@ __device__ __forceinline__ void background_rendered(const PlanView& v, const Ite
   }
 }
 
-// With a render cache the neighbours' moments are gathered from it (the
-// values the rendering would produce, added in the same order): the lane's
+// With a render cache (kOwn: with the plan's own renders of its neighbours)
+// the neighbours' moments are gathered from it (the values the rendering would produce, added in the same order): the lane's
 // eight pixels of the chunk stay in registers, and the neighbours' values
 // come through asynchronous copies to shared memory (st: kBgCacheF floats of
 // the warp), kBgStages - 1 neighbours ahead of the one being added, zeros
@@ -1335,6 +1335,7 @@ __device__ __forceinline__ void copy_async8(unsigned dst, const void* src, bool 
                "r"(valid ? 8 : 0)
                : "memory");
 }
+template <bool kOwn>
 __device__ __forceinline__ void background_cached(const PlanView& v, const Item& item,
                                                   const PairInfo& pi, float* st, int lane) {
   constexpr int kPix = kBgChunk / 32;
@@ -1366,7 +1367,7 @@ __device__ __forceinline__ void background_cached(const PlanView& v, const Item&
         ny = pi.y0 - qn.y0;
         nw = qn.w;
         nh = qn.h;
-        off = v.patches[qn.patch].pool_offset + cache_base(v, qn.source);
+        off = kOwn ? qn.bg_base : v.patches[qn.patch].pool_offset + cache_base(v, qn.source);
       }
       unsigned todo = __ballot_sync(0xffffffffu, min(r1, nh - ny) > max(r0, -ny) &&
                                                      min(pi.w, nw - nx) > max(0, -nx));
@@ -1377,7 +1378,7 @@ __device__ __forceinline__ void background_cached(const PlanView& v, const Item&
           todo &= todo - 1;
           const int mx = __shfl_sync(0xffffffffu, nx, g), my = __shfl_sync(0xffffffffu, ny, g);
           const int mw = __shfl_sync(0xffffffffu, nw, g), mh = __shfl_sync(0xffffffffu, nh, g);
-          const float2* src = v.cache + __shfl_sync(0xffffffffu, off, g);
+          const float2* src = (kOwn ? v.nbr_render : v.cache) + __shfl_sync(0xffffffffu, off, g);
           const unsigned dst = dst0 + (k % kBgStages) * (kBgChunk * sizeof(float2));
 #pragma unroll
           for (int u = 0; u < kPix; ++u) {
@@ -1425,6 +1426,7 @@ __global__ void __launch_bounds__(128, 5) background_kernel(PlanView v, int ne, 
   wq.done(lane);
 }
 
+template <bool kOwn>
 __global__ void __launch_bounds__(128) background_cached_kernel(PlanView v) {
   extern __shared__ float4 smem4[];
   const int lane = threadIdx.x & 31;
@@ -1433,7 +1435,7 @@ __global__ void __launch_bounds__(128) background_cached_kernel(PlanView v) {
   for (int it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < v.n_items; it += nwarps) {
     const Item item = v.items[it];
     const PairInfo pi = v.pairs[item.pair];
-    if (v.active[pi.slot]) background_cached(v, item, pi, st, lane);
+    if (v.active[pi.slot]) background_cached<kOwn>(v, item, pi, st, lane);
   }
 }
 
@@ -1466,21 +1468,46 @@ __global__ void __launch_bounds__(128) prepare_kernel(PlanView v, const ModelDev
       const Item item = v.items[u - n_mark - n_setup];
       const PairInfo pi = v.pairs[item.pair];
       if (status && !active_of(status[pi.source])) continue;
-      background_cached(v, item, pi, rec, lane);
+      background_cached<false>(v, item, pi, rec, lane);
     }
   }
 }
 
 // The loop of the render kernels: f(item, pair info) for every item.
 template <bool kQueue, class F>
-__device__ __forceinline__ void for_items(const PlanView& v, int lane, F&& f) {
+__device__ __forceinline__ void for_items(const PlanView& v, const Item* __restrict__ items, int n,
+                                          int lane, F&& f) {
   WarpQueue wq(kQueue ? v.work_ctr : nullptr);
-  for (; wq.it < v.n_items; wq.advance()) {
+  for (; wq.it < n; wq.advance()) {
     wq.ask(lane);
-    const Item item = v.items[wq.it];
+    const Item item = items[wq.it];
     f(item, v.pairs[item.pair]);
   }
   wq.done(lane);
+}
+
+// Moments of the plan's neighbour pairs over their whole patches, once each,
+// for the backgrounds to gather (into v.nbr_render); those that no active slot
+// uses are passed by.  Bound by FP32 issue like
+// the other renders; one pass over the patches instead of one an overlap
+// (300 blended sources: render and gather 276 us, overlaps 750).
+template <bool kQueue>
+__global__ void __launch_bounds__(128, 8) render_neighbours_kernel(PlanView v, int ne, int nd) {
+  extern __shared__ float4 smem4[];
+  const int lane = threadIdx.x & 31;
+  float* rec = reinterpret_cast<float*>(smem4) + (threadIdx.x >> 5) * kValRecF;
+  for_items<kQueue>(v, v.nbr_items, v.n_nbr_items, lane, [&](const Item& item, const PairInfo& pi) {
+    bool used = false;                       // by an active slot
+    for (int k = pi.nbr_begin; k < pi.nbr_end && !used; k += 32)
+      used = __any_sync(0xffffffffu, k + lane < pi.nbr_end && v.active[v.pair_nbr[k + lane]]);
+    if (!used) return;
+    float2* out = v.nbr_render + pi.bg_base;
+    stage_value(rec, v, item.pair, lane, ne, nd);
+    for_moments(rec, item.start, item.start + item.count, pi.w, 0, 0, lane, ne, nd,
+                [](int, int, int) { return 0; }, [&](int, int q, int, int, float Es, float Vs) {
+      out[q] = make_float2(Es, Vs);
+    });
+  });
 }
 
 // Own E_s and V_s of every plan pair, scattered to the caller's pool layout.
@@ -1491,7 +1518,7 @@ __global__ void __launch_bounds__(128, 8) render_kernel(PlanView v, int ne, int 
   extern __shared__ float4 smem4[];
   const int lane = threadIdx.x & 31;
   float* rec = reinterpret_cast<float*>(smem4) + (threadIdx.x >> 5) * kValRecF;
-  for_items<kQueue>(v, lane, [&](const Item& item, const PairInfo& pi) {
+  for_items<kQueue>(v, v.items, v.n_items, lane, [&](const Item& item, const PairInfo& pi) {
     const int64_t off = patches[pi.patch].pool_offset;
     stage_value(rec, v, item.pair, lane, ne, nd);
     for_moments(rec, item.start, item.start + item.count, pi.w, 0, 0, lane, ne, nd,
@@ -1509,7 +1536,7 @@ __global__ void __launch_bounds__(128, 8) render_cache_kernel(PlanView v, int ne
   extern __shared__ float4 smem4[];
   const int lane = threadIdx.x & 31;
   float* rec = reinterpret_cast<float*>(smem4) + (threadIdx.x >> 5) * kValRecF;
-  for_items<kQueue>(v, lane, [&](const Item& item, const PairInfo& pi) {
+  for_items<kQueue>(v, v.items, v.n_items, lane, [&](const Item& item, const PairInfo& pi) {
     if (status && status[pi.source] != CELESTE_ST_ACCEPTED) return;
     float2* out = v.cache + cache_base(v, pi.source) + v.patches[pi.patch].pool_offset;
     stage_value(rec, v, item.pair, lane, ne, nd);
@@ -1555,7 +1582,7 @@ __global__ void __launch_bounds__(128, 8) accumulate_kernel(PlanView v, int ne, 
   extern __shared__ float4 smem4[];
   const int lane = threadIdx.x & 31;
   float* rec = reinterpret_cast<float*>(smem4) + (threadIdx.x >> 5) * kValRecF;
-  for_items<kQueue>(v, lane, [&](const Item& item, const PairInfo& pi) {
+  for_items<kQueue>(v, v.items, v.n_items, lane, [&](const Item& item, const PairInfo& pi) {
     stage_value(rec, v, item.pair, lane, ne, nd);
     for_moments(rec, item.start, item.start + item.count, pi.w, 0, 0, lane, ne, nd,
                        [](int, int, int) { return 0; }, [&](int, int, int qx, int qy, float Es, float Vs) {
@@ -1758,7 +1785,8 @@ cudaError_t init_pixel_occupancy() {
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[kOccPrepare], prepare_kernel,
                                                         kWpb * 32, smem_bytes_cached(kWpb));
     if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[kOccCached], background_cached_kernel,
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[kOccCached],
+                                                        background_cached_kernel<true>,
                                                         kWpb * 32, smem_bytes_cached(kWpb));
     if (e == cudaSuccess)
       for (int k = 0; k < kOccKinds; ++k) g_occ[dev][k].store(occ[k], std::memory_order_relaxed);
@@ -1788,8 +1816,8 @@ static int grid_for(const Launch& L, int n_items, int wpb, int occ_kind = -1) {
 // of 800 chains loses 4 %), from three in the gradient and rendering kernels
 // (1,024 field sources: gradient 138 -> 129 us, backgrounds 50 -> 45).
 constexpr int kQueueItems = 5, kQueueItemsRender = 3;
-static bool use_queue(const PlanView& v, int blocks, int per_warp = kQueueItems) {
-  return v.work_ctr && v.n_items >= per_warp * kWpb * blocks;
+static bool use_queue(const PlanView& v, int n_items, int blocks, int per_warp) {
+  return v.work_ctr && n_items >= per_warp * kWpb * blocks;
 }
 
 // Leaving out vanished pairs pays where pixels lie far from their source and
@@ -1807,22 +1835,35 @@ static bool use_skip(const Launch& L, const PlanView& v) {
 // a compile-time constant: with the work queue where the grid has many items
 // per warp (occ_q: that form's occupancy).
 template <class F>
-static cudaError_t launch_items(const Launch& L, const PlanView& v, int occ, int occ_q,
+static cudaError_t launch_items(const Launch& L, const PlanView& v, int n_items, int occ, int occ_q,
                                 int per_warp, F&& kernel) {
+  if (n_items == 0) return cudaSuccess;
+  const int gq = grid_for(L, n_items, kWpb, occ_q);
+  if (use_queue(v, n_items, gq, per_warp)) kernel(std::true_type(), gq);
+  else kernel(std::false_type(), grid_for(L, n_items, kWpb, occ));
+  return cudaGetLastError();
+}
+
+template <bool kOwn>
+static cudaError_t launch_gather(const Launch& L, const PlanView& v) {
   if (v.n_items == 0) return cudaSuccess;
-  const int gq = grid_for(L, v.n_items, kWpb, occ_q);
-  if (use_queue(v, gq, per_warp)) kernel(std::true_type(), gq);
-  else kernel(std::false_type(), grid_for(L, v.n_items, kWpb, occ));
+  background_cached_kernel<kOwn><<<grid_for(L, v.n_items, kWpb, kOccCached), kWpb * 32,
+                                   smem_bytes_cached(kWpb), L.stream>>>(v);
   return cudaGetLastError();
 }
 
 cudaError_t launch_background(const Launch& L, const PlanView& v) {
-  if (v.cache && v.n_items) {
-    background_cached_kernel<<<grid_for(L, v.n_items, kWpb, kOccCached), kWpb * 32,
-                               smem_bytes_cached(kWpb), L.stream>>>(v);
-    return cudaGetLastError();
+  if (v.cache) return launch_gather<false>(L, v);
+  if (v.nbr_render) {
+    const cudaError_t e = launch_items(
+        L, v, v.n_nbr_items, kOccRender, kOccRender, kQueueItemsRender, [&](auto q, int grid) {
+          render_neighbours_kernel<decltype(q)::value>
+              <<<grid, kWpb * 32, smem_bytes(kWpb), L.stream>>>(v, L.n_exp, L.n_dev);
+        });
+    return e == cudaSuccess ? launch_gather<true>(L, v) : e;
   }
-  return launch_items(L, v, kOccBackground, kOccBackground, kQueueItemsRender, [&](auto q, int grid) {
+  return launch_items(L, v, v.n_items, kOccBackground, kOccBackground, kQueueItemsRender,
+                      [&](auto q, int grid) {
     background_kernel<decltype(q)::value>
         <<<grid, kWpb * 32, smem_bytes_bg(kWpb), L.stream>>>(v, L.n_exp, L.n_dev);
   });
@@ -1843,7 +1884,7 @@ cudaError_t launch_pixels_derivs(const Launch& L, const PlanView& v) {
   }
   if (cudaError_t e = derivs_attr()) return e;
   const int gq = grid_for(L, v.n_items, kWpb, kOccDerivsQ);
-  const bool queue = use_queue(v, gq);
+  const bool queue = use_queue(v, v.n_items, gq, kQueueItems);
   const int grid = queue ? gq : grid_for(L, v.n_items, kWpb, kOccDerivs);
   kDerivsKernels[queue][use_skip(L, v)]<<<grid, kWpb * 32, smem_bytes_derivs(kWpb), L.stream>>>(
       v, L.n_exp, L.n_dev);
@@ -1853,7 +1894,7 @@ cudaError_t launch_pixels_derivs(const Launch& L, const PlanView& v) {
 cudaError_t launch_pixels_grad(const Launch& L, const PlanView& v) {
   if (v.n_items == 0) return cudaSuccess;
   const int gq = grid_for(L, v.n_items, kWpb, kOccGradQ);
-  if (use_queue(v, gq, kQueueItemsRender))
+  if (use_queue(v, v.n_items, gq, kQueueItemsRender))
     grad_kernel<true><<<gq, kWpb * 32, smem_bytes_grad(kWpb), L.stream>>>(v, L.n_exp, L.n_dev);
   else
     grad_kernel<false><<<grid_for(L, v.n_items, kWpb, kOccGrad), kWpb * 32, smem_bytes_grad(kWpb),
@@ -1868,7 +1909,7 @@ cudaError_t launch_pixels_value(const Launch& L, const PlanView& v, bool keep_re
     value_coop_kernel<<<v.n_items, kCoopThreads, 0, L.stream>>>(v, L.n_exp, L.n_dev, mode);
     return cudaGetLastError();
   }
-  return launch_items(L, v, kOccValue, kOccValueQ, kQueueItems, [&](auto q, int grid) {
+  return launch_items(L, v, v.n_items, kOccValue, kOccValueQ, kQueueItems, [&](auto q, int grid) {
     value_kernel<decltype(q)::value>
         <<<grid, kWpb * 32, smem_bytes(kWpb), L.stream>>>(v, L.n_exp, L.n_dev, mode);
   });
@@ -1892,7 +1933,7 @@ cudaError_t launch_commit_render(const Launch& L, const PlanView& v, const int32
 
 cudaError_t launch_render(const Launch& L, const PlanView& v, float* E_out, float* V_out,
                           const celeste_patch* patches) {
-  return launch_items(L, v, kOccRender, kOccRender, kQueueItemsRender, [&](auto q, int grid) {
+  return launch_items(L, v, v.n_items, kOccRender, kOccRender, kQueueItemsRender, [&](auto q, int grid) {
     render_kernel<decltype(q)::value>
         <<<grid, kWpb * 32, smem_bytes(kWpb), L.stream>>>(v, L.n_exp, L.n_dev, E_out, V_out, patches);
   });
@@ -1900,14 +1941,14 @@ cudaError_t launch_render(const Launch& L, const PlanView& v, float* E_out, floa
 
 cudaError_t launch_render_cache(const Launch& L, const PlanView& v, const int32_t* status) {
   if (!v.cache) return cudaSuccess;
-  return launch_items(L, v, kOccRender, kOccRender, kQueueItemsRender, [&](auto q, int grid) {
+  return launch_items(L, v, v.n_items, kOccRender, kOccRender, kQueueItemsRender, [&](auto q, int grid) {
     render_cache_kernel<decltype(q)::value>
         <<<grid, kWpb * 32, smem_bytes(kWpb), L.stream>>>(v, L.n_exp, L.n_dev, status);
   });
 }
 
 cudaError_t launch_accumulate(const Launch& L, const PlanView& v, float* Eimg, float* Vimg) {
-  return launch_items(L, v, kOccRender, kOccRender, kQueueItemsRender, [&](auto q, int grid) {
+  return launch_items(L, v, v.n_items, kOccRender, kOccRender, kQueueItemsRender, [&](auto q, int grid) {
     accumulate_kernel<decltype(q)::value>
         <<<grid, kWpb * 32, smem_bytes(kWpb), L.stream>>>(v, L.n_exp, L.n_dev, Eimg, Vimg);
   });
