@@ -19,6 +19,8 @@ pytestmark = pytest.mark.gpu
     (2, 16, 8, 256, False),    # a quarter, one neighbour: rendered over the overlaps
     (2, 24, 7, 256, False),    # 289 of 576: just above half
     (2, 24, 8, 256, False),    # 256 of 576: just below
+    (86, 33, 24, 32, False),   # 3,010 items over small overlaps: four warps an item
+    (100, 33, 24, 32, False),  # 3,500: a warp an item
     (4, 33, 1, 32, False),     # items of less than a row
     (9, 37, 2, 256, False),    # several items a neighbour, ragged
     (12, 33, 1, 1024, True),   # neighbours in and out of the plan
