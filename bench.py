@@ -42,7 +42,10 @@ UNIT = "visits/s"
 # direct formulation: every component's Hermite polynomials from its own
 # offset and precision.  The kernel shares the offsets of the components of
 # one PSF component and stages pixel-independent constants, and executes
-# EXECUTED_FLOP_PER_VISIT; the roofline reports both fractions.
+# EXECUTED_FLOP_PER_VISIT; the roofline reports both fractions.  Both count
+# every pair of components: in large patches the kernel skips the pairs that
+# vanish exactly (about a fifth of them in blends), so frac_executed is an
+# upper bound of the pipes' own utilisation there.
 FLOP_PER_VISIT = 5320
 EXECUTED_FLOP_PER_VISIT = 4723
 FP32_LANES_PER_SM = 128
