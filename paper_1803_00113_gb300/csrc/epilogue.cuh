@@ -64,12 +64,8 @@ constexpr int kTileChunk = 32;                   // tiles copied to shared memor
 // Barriers among the kPairThreads threads of warps 1..3 (named barrier 1;
 // warp 0 is busy with the KL terms meanwhile) and among warps 1 and 2
 // (named barrier 2).
-static __device__ __forceinline__ void pair_sync() {
-  asm volatile("bar.sync 1, %0;" ::"n"(kPairThreads) : "memory");
-}
-static __device__ __forceinline__ void tile_sync() {
-  asm volatile("bar.sync 2, 64;" ::: "memory");
-}
+static __device__ __forceinline__ void pair_sync() { named_sync(1, kPairThreads); }
+static __device__ __forceinline__ void tile_sync() { named_sync(2, 64); }
 // Asynchronous copy of 16 bytes to shared memory.
 static __device__ __forceinline__ void copy_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
@@ -340,7 +336,7 @@ static __device__ void kl_terms(const real* th, const ModelDev::F32& f, int J, E
     }
   }
   __syncwarp();
-  if (kApart) asm volatile("bar.sync 3, 64;" ::: "memory");
+  if (kApart) named_sync(3, 64);
   // ---- value (lane 0)
   if (lane == 0) {
     real v = fmaf(a, (-S.klt[0] - f.log_prior_a), __fmul_rn(1.f - a, (-S.klt[1] - f.log1m_prior_a)));
@@ -547,7 +543,7 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
       auto apart = [&] {
         if (wid == 2) {
           kl_lone_terms<kMode>(th, f, S, lane);
-          asm volatile("bar.arrive 3, 64;" ::: "memory");
+          named_arrive(3, 64);
         } else if (wid == 3) {
           if (lane < 20) kappa_row(th, lane, S);
         } else if (lane == 0) {

@@ -274,6 +274,20 @@ __device__ __forceinline__ int rotated_tid(int n_sm) {
   return (int)((threadIdx.x + 32u * (blockIdx.x + blockIdx.x / (unsigned)n_sm)) & 127u);
 }
 
+// Named barrier id among the n threads of whole warps that name it: sync waits
+// for the others, arrive does not.  The bar.* forms want all of a warp's
+// threads at once, and after lane-divergent code (here: branches over lanes
+// whose terms differ) nothing else brings them together, so each waits for
+// its warp first; that also orders what the warp's other lanes wrote.
+__device__ __forceinline__ void named_sync(int id, int n) {
+  __syncwarp();
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void named_arrive(int id, int n) {
+  __syncwarp();
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+
 // A slot takes part in a Newton iteration unless its source has stopped.
 __device__ __forceinline__ uint8_t active_of(int32_t st) {
   return (st == CELESTE_ST_CONVERGED || st == CELESTE_ST_FAILED || st == CELESTE_ST_MAXITER) ? 0

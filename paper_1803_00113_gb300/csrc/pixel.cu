@@ -1013,8 +1013,7 @@ __global__ void __launch_bounds__(kCoopThreads, 2) derivs_coop_kernel(PlanView v
     // rounds of an item longer than a block follow each other through the
     // block barrier below.
     auto turn = [&] {
-      __syncwarp();
-      if (wib > 0) asm volatile("bar.sync %0, 64;" ::"r"(wib) : "memory");
+      if (wib > 0) named_sync(wib, 64);
       return q < end;
     };
     if (base + 32 * wib < end) {
@@ -1029,8 +1028,7 @@ __global__ void __launch_bounds__(kCoopThreads, 2) derivs_coop_kernel(PlanView v
     } else {
       turn();
     }
-    __syncwarp();
-    if (wib < kCoopWarps - 1) asm volatile("bar.arrive %0, 64;" ::"r"(wib + 1) : "memory");
+    if (wib < kCoopWarps - 1) named_arrive(wib + 1, 64);
     if (base + kCoopThreads < end) __syncthreads();
   }
   __syncthreads();
