@@ -979,20 +979,24 @@ static __device__ void locate32(TrSmem& S, double Delta, int tid) {
   // lambda_min (scaled) lies in [fa, fb] up to FP32 rounding of the counts
   const float lmin = fa;
   // boundary bracket [la, lb]; the first round of its multisection also
-  // evaluates |p(0)| (thread 127, which holds no probe)
+  // evaluates |p(0)| (thread 127, which holds no probe), stored before the
+  // round's barrier and not again: a thread may read it after later ones
   const float lo = fmaxf(0.f, -lmin);
   float la = lo, lb = lo + gnorm_s / (float)Delta * 1.01f + 1e-6f;
-  auto secular_round = [&]() {
-    const float l = la + (lb - la) * (float)(tid + 1) * kStep;
-    const float n2 = norm2_32s(S.df, S.ef, S.gf, tid < kTrThreads - 1 ? l : 0.f, cps, gps);
-    if (tid == kTrThreads - 1) S.loc[2] = lmin > 0.f ? n2 : 3.4e38f;
-    const int t = first_hit(S, tid < kTrThreads - 1 && n2 <= D2, round++, tid);
+  auto probe = [&]() { return la + (lb - la) * (float)(tid + 1) * kStep; };
+  auto narrow = [&](float n2) {
+    const int t = first_hit(S, n2 <= D2, round++, tid);   // (of threads 0..126)
     const float na = t == 0 ? la : la + (lb - la) * (float)t * kStep;
     const float nb = t == kTrThreads - 1 ? lb : la + (lb - la) * (float)(t + 1) * kStep;
     la = na;
     lb = nb;
   };
-  secular_round();
+  {
+    const float n2 =
+        norm2_32s(S.df, S.ef, S.gf, tid < kTrThreads - 1 ? probe() : 0.f, cps, gps);
+    if (tid == kTrThreads - 1) S.loc[2] = lmin > 0.f ? n2 : 3.4e38f;
+    narrow(n2);
+  }
   const float n0 = S.loc[2];
   // mode 0: try l = 0 first (interior Newton step); mode 1: the boundary
   // root from the bracket; mode 2: the all-FP64 path
@@ -1009,7 +1013,7 @@ static __device__ void locate32(TrSmem& S, double Delta, int tid) {
     if (lmin > 0.f && n0 <= D2 * 1.01f) mode = 0;
     bracket = true;
 #pragma unroll 1
-    for (int r = 1; r < 4; ++r) secular_round();
+    for (int r = 1; r < 4; ++r) narrow(norm2_32s(S.df, S.ef, S.gf, probe(), cps, gps));
     // near the pole (nearly hard case) the FP32 bracket is still a good
     // start; the FP64 iteration below resolves it, and a true hard case
     // (no root above the pole) ends in the all-FP64 path
@@ -1132,6 +1136,7 @@ static __device__ bool tr_solve(TrSmem& S, double Delta, int tid) {
         // hard case, the multiplier within ~1e-10 of -lambda_min): the
         // eigen-based all-FP64 path resolves it.
         if (!fin && bisects >= 3) mode = 2;
+        __syncwarp();                   // every lane has read them
         if (lane == 0) {
           S.lo = lo;
           S.hi = hi;
