@@ -76,6 +76,18 @@ static __device__ __forceinline__ void copy_async16(void* dst, const void* src) 
 
 constexpr int kGeoHess = 55;                     // upper triangle over the 10 w
 
+// The sums of a tile that a pass of this mode has written, kAcc floats apart
+// from tile to tile: all of them, or the value and gradient alone; and where
+// piece e (16 bytes) of a run of tiles lies, in floats from the first.
+template <int kMode>
+constexpr int kTileSums = kMode == 2 ? kAcc : kGradAcc;
+template <int kMode>
+__host__ __device__ constexpr int tile_piece(int e) {
+  constexpr int per = kTileSums<kMode> / 4;
+  return e / per * kAcc + e % per * 4;
+}
+static_assert(kAcc % 4 == 0 && kGradAcc % 4 == 0, "whole pieces");
+
 struct EpiSmem {
   float vs[kPairGroup][4];         // per pair of a group: value sums (s, c of relative, base)
   float W[kPairGroup][kAcc];       // per pair of a group: zero, then the other sums (2..63)
@@ -576,18 +588,19 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
         }
         if (wid < 3) {
           // the tile sums of the group's pairs, whose items are contiguous:
-          // chunks of kTileChunk tiles (256 B each) are copied to shared
-          // memory, one chunk ahead, and warps 1 and 2 add up a pair each at
-          // a time: lane l forms accumulators 2 l and 2 l + 1 by compensated
-          // (Kahan) FP32 summation in tile order, whose error does not grow
-          // with the number of tiles
+          // chunks of kTileChunk tiles (256 B each; 48 B without a Hessian) are
+          // copied to shared memory, one chunk ahead, and warps 1 and 2 add up
+          // a pair each at a time: lane l forms accumulators 2 l and 2 l + 1 by
+          // compensated (Kahan) FP32 summation in tile order, whose error does
+          // not grow with the number of tiles
           const int t0 = __shfl_sync(0xffffffffu, ib, 0);
           const int t1 = __shfl_sync(0xffffffffu, ie, ng - 1);
           auto fetch = [&](int c) {
-            const int n16 = min(kTileChunk, t1 - t0 - c * kTileChunk) * (kAcc / 4);
+            const int n16 = min(kTileChunk, t1 - t0 - c * kTileChunk) * (kTileSums<kMode> / 4);
             const float* src = v.partials + (size_t)(t0 + c * kTileChunk) * kAcc;
             float* dst = &S.tiles[c & 1][0][0];
-            for (int e = u; e < n16; e += 64) copy_async16(dst + 4 * e, src + 4 * e);
+            for (int e = u; e < n16; e += 64)
+              copy_async16(dst + tile_piece<kMode>(e), src + tile_piece<kMode>(e));
             asm volatile("cp.async.commit_group;" ::: "memory");
           };
           const int nc = (t1 - t0 + kTileChunk - 1) / kTileChunk;
@@ -608,7 +621,7 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
             while (g < ng) {
               const int b = __shfl_sync(0xffffffffu, ib, g), e = __shfl_sync(0xffffffffu, ie, g);
               if (b >= c1) break;
-              const int q1 = min(e, c1) - c0;
+              const int q1 = 2 * lane < kTileSums<kMode> ? min(e, c1) - c0 : 0;
 #pragma unroll 4
               for (int q = max(b, c0) - c0; q < q1; ++q) {
                 const float2 y = x[q * (kAcc / 2)];
@@ -630,7 +643,7 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
                 S.vs[g][1] = c.x;
                 S.vs[g][2] = s.y;
                 S.vs[g][3] = c.y;
-              } else {
+              } else if (2 * lane < kTileSums<kMode>) {
                 S.W[g][2 * lane] = s.x - c.x;
                 S.W[g][2 * lane + 1] = s.y - c.y;
               }
