@@ -5,8 +5,9 @@
 
 namespace celeste {
 
+template <int kMode>
 struct EpiBlock {
-  EpiSmem e;
+  EpiShared<kMode> e;
   ModelDev::F32 f;
 };
 
@@ -20,14 +21,14 @@ __global__ void __launch_bounds__(kEpiThreads) epilogue_kernel(PlanView v,
                                                                double* grad_out, double* hess_out,
                                                                int use_trial) {
   extern __shared__ double smd[];
-  EpiBlock& S = *reinterpret_cast<EpiBlock*>(smd);
+  EpiBlock<kMode>& S = *reinterpret_cast<EpiBlock<kMode>*>(smd);
   const int j = blockIdx.x, tid = threadIdx.x;
   if (!v.active[j]) return;
   const bool trial = (use_trial & 1) != 0, pixel_only = kMode == 0 && (use_trial & 2) != 0;
   const double* thd =
       trial ? v.theta_trial + (size_t)j * kTheta : v.theta + (size_t)v.src_ids[j] * kTheta;
   if (tid < kTheta) S.e.th[tid] = (real)thd[tid];
-  stage_model(S.f, model, tid, kEpiThreads);
+  if (!pixel_only) stage_model(S.f, model, tid, kEpiThreads);
   double rel, full;
   epilogue_source<kMode>(v, S.f, model->n_color, S.e, j, tid, pixel_only, rel, full);
   if (tid == 0) {
@@ -36,7 +37,7 @@ __global__ void __launch_bounds__(kEpiThreads) epilogue_kernel(PlanView v,
     // a non-finite value at a trial point is a rejected step, not an error
     if (!isfinite(full) && !trial) set_error(v.err, CELESTE_DERR_NONFINITE);
   }
-  if (kMode >= 1) {
+  if constexpr (kMode >= 1) {
     int bad = 0;
     for (int e = tid; e < kTheta; e += kEpiThreads) {
       grad_out[(size_t)j * kTheta + e] = (double)S.e.gth[e];
@@ -56,7 +57,7 @@ static cudaError_t set_smem_attr() {
   static DeviceOnce once;
   return once.run([] {
     return cudaFuncSetAttribute(epilogue_kernel<kMode>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(EpiBlock));
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(EpiBlock<kMode>));
   });
 }
 
@@ -64,7 +65,7 @@ cudaError_t launch_epilogue(const Launch& L, const PlanView& v, const ModelDev* 
                             double* elbo, double* elbo_rel, double* grad, double* hess) {
   if (v.n == 0) return cudaSuccess;
   if (cudaError_t e = set_smem_attr<2>()) return e;
-  epilogue_kernel<2><<<v.n, kEpiThreads, sizeof(EpiBlock), L.stream>>>(v, model, elbo, elbo_rel, grad,
+  epilogue_kernel<2><<<v.n, kEpiThreads, sizeof(EpiBlock<2>), L.stream>>>(v, model, elbo, elbo_rel, grad,
                                                               hess, 0);
   return cudaGetLastError();
 }
@@ -73,7 +74,7 @@ cudaError_t launch_epilogue_grad(const Launch& L, const PlanView& v, const Model
                                  double* elbo, double* elbo_rel, double* grad) {
   if (v.n == 0) return cudaSuccess;
   if (cudaError_t e = set_smem_attr<1>()) return e;
-  epilogue_kernel<1><<<v.n, kEpiThreads, sizeof(EpiBlock), L.stream>>>(v, model, elbo, elbo_rel, grad,
+  epilogue_kernel<1><<<v.n, kEpiThreads, sizeof(EpiBlock<1>), L.stream>>>(v, model, elbo, elbo_rel, grad,
                                                               nullptr, 0);
   return cudaGetLastError();
 }
@@ -82,7 +83,7 @@ cudaError_t launch_epilogue_value(const Launch& L, const PlanView& v, const Mode
                                   double* elbo, double* elbo_rel, bool use_trial) {
   if (v.n == 0) return cudaSuccess;
   if (cudaError_t e = set_smem_attr<0>()) return e;
-  epilogue_kernel<0><<<v.n, kEpiThreads, sizeof(EpiBlock), L.stream>>>(v, model, elbo, elbo_rel, nullptr,
+  epilogue_kernel<0><<<v.n, kEpiThreads, sizeof(EpiBlock<0>), L.stream>>>(v, model, elbo, elbo_rel, nullptr,
                                                               nullptr, use_trial ? 1 : 0);
   return cudaGetLastError();
 }
@@ -91,7 +92,7 @@ cudaError_t launch_epilogue_loglik(const Launch& L, const PlanView& v, const Mod
                                    double* out) {
   if (v.n == 0) return cudaSuccess;
   if (cudaError_t e = set_smem_attr<0>()) return e;
-  epilogue_kernel<0><<<v.n, kEpiThreads, sizeof(EpiBlock), L.stream>>>(v, model, nullptr, out,
+  epilogue_kernel<0><<<v.n, kEpiThreads, sizeof(EpiBlock<0>), L.stream>>>(v, model, nullptr, out,
                                                                       nullptr, nullptr, 2);
   return cudaGetLastError();
 }
@@ -99,8 +100,7 @@ cudaError_t launch_epilogue_loglik(const Launch& L, const PlanView& v, const Mod
 // KL_s of every slot's source at theta, into kl_out[source id] (for the
 // full-field ELBO, Eq. elbo: the pixel sum minus the sum of the KL_s).
 __global__ void kl_kernel(PlanView v, const ModelDev* __restrict__ model, double* kl_out) {
-  extern __shared__ double smd[];
-  EpiSmem& S = *reinterpret_cast<EpiSmem*>(smd);
+  __shared__ KlSmem S;
   const int j = blockIdx.x;
   const int lane = threadIdx.x;
   const int src = v.src_ids[j];
@@ -113,13 +113,7 @@ __global__ void kl_kernel(PlanView v, const ModelDev* __restrict__ model, double
 
 cudaError_t launch_kl(const Launch& L, const PlanView& v, const ModelDev* model, double* kl_out) {
   if (v.n == 0) return cudaSuccess;
-  static DeviceOnce once;
-  cudaError_t e = once.run([] {
-    return cudaFuncSetAttribute(kl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)sizeof(EpiSmem));
-  });
-  if (e != cudaSuccess) return e;
-  kl_kernel<<<v.n, 32, sizeof(EpiSmem), L.stream>>>(v, model, kl_out);
+  kl_kernel<<<v.n, 32, 0, L.stream>>>(v, model, kl_out);
   return cudaGetLastError();
 }
 

@@ -37,6 +37,8 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 #include "internal.cuh"
 
 namespace celeste {
@@ -88,7 +90,21 @@ __host__ __device__ constexpr int tile_piece(int e) {
 }
 static_assert(kAcc % 4 == 0 && kGradAcc % 4 == 0, "whole pieces");
 
-struct EpiSmem {
+// What a value alone needs of a block's shared memory: 2 KB with the model's
+// constants, which a log-likelihood does without.  (With the derivative
+// passes' buffers, 40 KB, five blocks fit on an SM; 600 sources, a
+// log-likelihood with the constants staged 29.4 us, without 27.5.)
+struct KlSmem {
+  real th[kNuPad];                 // theta of the source (FP32 copy)
+  real kw[kNuPad];                 // colour weights; then grad_nu[a] * kappa_a
+  real klj[2 * kMaxColor];         // log w_j - K_j
+  real kls[8];                     // scalar KL pieces
+  real klt[32];                    // terms of the KL's value and gradient
+  double red[2][kEpiThreads / 32]; // per-warp value sums
+  double vsum[2];                  // the source's value sums (relative, base)
+};
+
+struct EpiSmem : KlSmem {
   float vs[kPairGroup][4];         // per pair of a group: value sums (s, c of relative, base)
   float W[kPairGroup][kAcc];       // per pair of a group: zero, then the other sums (2..63)
   float T[kPairGroup][10 * 10];    // per pair of a group: affine map w <- nu (local)
@@ -96,7 +112,6 @@ struct EpiSmem {
   float img[5 * kPairGroup];       // per pair of a group: calibration and A, FP32
   int band[kPairGroup];
   real pw[2 * kKlSums];            // colour bound: pi-weighted sums per type
-  real th[kNuPad];                 // theta of the source (FP32 copy)
   real gnu[kNuPad];
   real Hnu[kNu * kNu];
   real J[kNu * kTheta];
@@ -106,15 +121,11 @@ struct EpiSmem {
   real DL[20 * kTheta + kTheta];   // d log kappa_a / d theta (padded)
   real D2L[20 * kTheta];           // diagonal second derivatives of log kappa_a
   real kap[kNuPad];                // kappa_a
-  real kw[kNuPad];                 // grad_nu[a] * kappa_a
   real d2S[27];                    // second derivatives of Sigma_s
   real klc[2 * kMaxColor * kKlVals];   // colour-bound pieces per (type, component)
-  real klj[2 * kMaxColor];         // log w_j - K_j
-  real kls[8];                     // scalar KL pieces
-  real klt[32];                    // terms of the KL's value and gradient
-  double red[2][kEpiThreads / 32]; // per-warp value sums
-  double vsum[2];                  // the source's value sums (relative, base)
 };
+template <int kMode>
+using EpiShared = std::conditional_t<kMode == 0, KlSmem, EpiSmem>;
 
 // Rows a of J with J[a][c] != 0 for column c: their number and the k-th one
 // (the flux coordinates of a type feed every band's kE and kM rows).
@@ -213,7 +224,7 @@ static __device__ void sigma_derivs(const real* th, real dS[3][3], real d2S[3][3
 // The terms of KL_s that stand alone, a lane each (lanes 0..8), into S.klt.
 template <int kMode>
 static __device__ __forceinline__ void kl_lone_terms(const real* th, const ModelDev::F32& f,
-                                                     EpiSmem& S, int lane) {
+                                                     KlSmem& S, int lane) {
   if (lane < 6) {
     // softplus of -+theta_0, -+theta_25, -+theta_26
     const int t = lane < 2 ? 0 : (lane < 4 ? 25 : 26);
@@ -245,7 +256,7 @@ static __device__ __forceinline__ void kl_lone_terms(const real* th, const Model
 // and its number of colour components.  kApart: warp 2 forms the lone terms
 // and meets this warp at named barrier 3.
 template <int kMode, bool kApart>
-static __device__ void kl_terms(const real* th, const ModelDev::F32& f, int J, EpiSmem& S,
+static __device__ void kl_terms(const real* th, const ModelDev::F32& f, int J, EpiShared<kMode>& S,
                                 int lane) {
   const real a = sigm(th[0]);
   const real wq = a * (1.f - a);
@@ -276,7 +287,7 @@ static __device__ void kl_terms(const real* th, const ModelDev::F32& f, int J, E
       }
       const real K = 0.5f * (tr + quad - 4.f + f.color_logdet[i][j] - slv);
       S.klj[lane] = f.log_color_w[i][j] - K;
-      if (kMode >= 1) {
+      if constexpr (kMode >= 1) {
         real* o = S.klc + lane * kKlVals;
         real gk[8];
 #pragma unroll
@@ -317,7 +328,7 @@ static __device__ void kl_terms(const real* th, const ModelDev::F32& f, int J, E
     for (int j = 0; j < kMaxColor; ++j) se[i] += S.kw[i * kMaxColor + j];
     Bval[i] = -(S.kls[4 + i] + logf(se[i]));
   }
-  if (kMode >= 1) {
+  if constexpr (kMode >= 1) {
     // pi-weighted sums per type (kKlSums per type): the mean
     // gradient, the precision block and the diagonal ...
     for (int e = lane; e < 2 * kKlVals; e += 32) {
@@ -369,27 +380,28 @@ static __device__ void kl_terms(const real* th, const ModelDev::F32& f, int J, E
     S.kls[0] = v;
   }
   __syncwarp();
-  if (kMode == 0) return;
-  if (lane == 0) {
-    const real la = f.logit_prior_a;
-    const real d2q = wq * (1.f - 2.f * a);
-    S.gth[0] -= wq * (th[0] - la) + wq * (S.kls[3] - S.kls[2]);
-    if (kMode == 2)
-      S.Hth[0] -= wq * ((1.f - 2.f * a) * (th[0] - la) + 1.f) + d2q * (S.kls[3] - S.kls[2]);
-  } else if (lane == 1) {
-    const real lr = th[24], E1 = f.e_radius[0], E2 = f.e_radius[1];
-    S.gth[24] -= 1.f + (lr - E1) / E2;
-    if (kMode == 2) S.Hth[24 * kTheta + 24] -= 1.f / E2;
-  } else if (lane < 4) {
-    const int which = lane - 2;
-    const int t = which ? 26 : 25;
-    const real b1 = (which ? f.e_profile[0] : f.e_axis[0]);
-    const real b2 = (which ? f.e_profile[1] : f.e_axis[1]);
-    const real sg = sigm(th[t]);
-    S.gth[t] -= -(b1 - 1.f) * (1.f - sg) + (b2 - 1.f) * sg;
-    if (kMode == 2) S.Hth[t * kTheta + t] -= (b1 + b2 - 2.f) * sg * (1.f - sg);
+  if constexpr (kMode >= 1) {
+    if (lane == 0) {
+      const real la = f.logit_prior_a;
+      const real d2q = wq * (1.f - 2.f * a);
+      S.gth[0] -= wq * (th[0] - la) + wq * (S.kls[3] - S.kls[2]);
+      if (kMode == 2)
+        S.Hth[0] -= wq * ((1.f - 2.f * a) * (th[0] - la) + 1.f) + d2q * (S.kls[3] - S.kls[2]);
+    } else if (lane == 1) {
+      const real lr = th[24], E1 = f.e_radius[0], E2 = f.e_radius[1];
+      S.gth[24] -= 1.f + (lr - E1) / E2;
+      if (kMode == 2) S.Hth[24 * kTheta + 24] -= 1.f / E2;
+    } else if (lane < 4) {
+      const int which = lane - 2;
+      const int t = which ? 26 : 25;
+      const real b1 = (which ? f.e_profile[0] : f.e_axis[0]);
+      const real b2 = (which ? f.e_profile[1] : f.e_axis[1]);
+      const real sg = sigm(th[t]);
+      S.gth[t] -= -(b1 - 1.f) * (1.f - sg) + (b2 - 1.f) * sg;
+      if (kMode == 2) S.Hth[t * kTheta + t] -= (b1 + b2 - 2.f) * sg * (1.f - sg);
+    }
+    __syncwarp();
   }
-  __syncwarp();
 }
 
 // The rest of the KL's gradient and Hessian, from S.pw and S.klt: the
@@ -459,17 +471,17 @@ static __device__ __forceinline__ void stage_model(ModelDev::F32& dst, const Mod
 template <int kMode>
 static __device__ __forceinline__ void epilogue_source(const PlanView& v,
                                                 const ModelDev::F32& f, int n_color,
-                                                EpiSmem& S, int j, int tid, bool pixel_only,
+                                                EpiShared<kMode>& S, int j, int tid, bool pixel_only,
                                                 double& rel, double& full) {
   const int lane = tid & 31, wid = tid >> 5;
   const real* th = S.th;
   const int p0 = v.slot_pair_ptr[j], p1 = v.slot_pair_ptr[j + 1];
-  if (kMode >= 1) {
+  if constexpr (kMode >= 1) {
     if (tid < kNuPad) S.gnu[tid] = S.gth[tid] = 0.f;
     for (int e = tid; e < kNu * kTheta; e += kEpiThreads) S.J[e] = 0.f;
     for (int e = tid; e < 20 * kTheta; e += kEpiThreads) S.DL[e] = S.D2L[e] = 0.f;
   }
-  if (kMode == 2) {
+  if constexpr (kMode == 2) {
     for (int e = tid; e < kNu * kNu; e += kEpiThreads) S.Hnu[e] = 0.f;
     for (int e = tid; e < kTheta * kTheta; e += kEpiThreads) S.Hth[e] = 0.f;
   }
@@ -477,37 +489,46 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
   if (wid == 0) {
     if (!pixel_only) {
       kl_terms<kMode, (kMode >= 1)>(th, f, n_color, S, lane);
-      if (kMode >= 1) kl_scatter<kMode>(th, S, lane);
+      if constexpr (kMode >= 1) kl_scatter<kMode>(th, S, lane);
     }
   } else {
     const int u = tid - 32;                            // 0 .. kPairThreads - 1
     double vr = 0.0, vb = 0.0;
-    if (kMode == 0) {
+    if constexpr (kMode == 0) {
       // value sums of every pair's items, thread-strided, then one reduction;
-      // eight pairs' first items are loaded together
+      // with three pairs or more of up to an item a thread, eight pairs' items
+      // are loaded together (one or two pairs, or longer ones, lose 0.6-1 us of
+      // 9-22 that way)
       for (int pg = p0; pg < p1; pg += 8) {
-        int ib[8], ie[8];
-        float2 x[8];
+        int ib[8], ie[8], most = 0;
 #pragma unroll
         for (int g = 0; g < 8; ++g) {
           ib[g] = ie[g] = 0;
           if (pg + g < p1) {
-            ib[g] = v.pairs[pg + g].item_begin + u;
+            ib[g] = v.pairs[pg + g].item_begin;
             ie[g] = v.pairs[pg + g].item_end;
           }
+          most = max(most, ie[g] - ib[g]);
         }
-#pragma unroll
-        for (int g = 0; g < 8; ++g)
-          if (ib[g] < ie[g]) x[g] = reinterpret_cast<const float2*>(v.vpartials)[ib[g]];
-#pragma unroll
-        for (int g = 0; g < 8; ++g) {
-          if (ib[g] < ie[g]) {
-            vr += (double)x[g].x;
-            vb += (double)x[g].y;
-            for (int it = ib[g] + kPairThreads; it < ie[g]; it += kPairThreads) {
+        if (p1 - pg < 3 || most > kPairThreads) {
+          for (int pp = pg; pp < min(pg + 8, p1); ++pp) {
+            const int b = v.pairs[pp].item_begin, e = v.pairs[pp].item_end;
+            for (int it = b + u; it < e; it += kPairThreads) {
               vr += (double)v.vpartials[2 * (size_t)it];
               vb += (double)v.vpartials[2 * (size_t)it + 1];
             }
+          }
+          continue;
+        }
+        float2 x[8];
+#pragma unroll
+        for (int g = 0; g < 8; ++g)
+          if (ib[g] + u < ie[g]) x[g] = reinterpret_cast<const float2*>(v.vpartials)[ib[g] + u];
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+          if (ib[g] + u < ie[g]) {
+            vr += (double)x[g].x;
+            vb += (double)x[g].y;
           }
         }
       }
@@ -741,8 +762,8 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
   const double kl = pixel_only ? 0.0 : (double)S.kls[0];
   rel = S.vsum[0] - kl;
   full = S.vsum[1] + S.vsum[0] - kl;
-  if (kMode >= 1) {
-    if (kMode == 2) {
+  if constexpr (kMode >= 1) {
+    if constexpr (kMode == 2) {
       if (tid < 20) S.kw[tid] = S.gnu[tid] * S.kap[tid];
       __syncthreads();
       // X = H_nu J where J's column has support.  Columns 0..20 (ten or
@@ -796,7 +817,7 @@ static __device__ __forceinline__ void epilogue_source(const PlanView& v,
       for (int k = 0; k < nr; ++k, r += dr) gsum = fmaf(S.J[r * kTheta + c], S.gnu[r], gsum);
       S.gth[c] += gsum;
     }
-    if (kMode == 2) {
+    if constexpr (kMode == 2) {
       // Hth += J^T X over d >= c (mirrored), plus the flux-moment
       // second-order term sum_a kw_a (dl dl^T + diag d2l).  Column 0 (twenty
       // rows) has a thread for each d; thread (c, g) of the others takes d =
