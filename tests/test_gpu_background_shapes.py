@@ -1,6 +1,7 @@
 """Backgrounds over overlaps narrower than a chunk's rows (patches wider than a
-chunk, chunks inside a row or across two): the same bits as the gather from a
-render cache."""
+chunk, chunks inside a row or across two), with items shared by two or four
+warps or by none, and of plans without neighbours (the sky alone): the same
+bits as the gather from a render cache."""
 import numpy as np
 import pytest
 import torch
@@ -37,6 +38,12 @@ def _scene(n, w, h, sx, sy):
     (2, 33, 65, 0, 48, 32),        # items of less than a row
     (2, 33, 65, 0, 48, 100),
     (9, 101, 40, 80, 0, 256),      # overlaps of a fifth of a row
+    (60, 90, 70, 70, 0, 64),       # more items than are shared
+    (1, 1, 1, 0, 0, 256),          # no neighbours from here on
+    (1, 31, 33, 0, 0, 32),
+    (3, 31, 33, 31, 0, 256),
+    (1, 333, 7, 0, 0, 1024),
+    (150, 40, 40, 40, 0, 64),      # 3,750 items
 ])
 def test_background_equals_the_gather(n, w, h, sx, sy, ppi):
     if not torch.cuda.is_available():
@@ -56,3 +63,17 @@ def test_background_equals_the_gather(n, w, h, sx, sy, ppi):
     ctx.synchronize()
     for a, b in zip(*got):
         assert np.array_equal(a, b)
+
+
+def test_sky_alone_reports_a_sky_of_zero():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1803_00113_gb300 import celeste as cel
+    p = _scene(1, 20, 20, 0, 0)
+    p.sky = np.zeros_like(p.sky)
+    ctx = cel.Context(p.model)
+    cel.background(cel.Plan(ctx, cel.DeviceProblem(p), [0]))
+    with pytest.raises(cel.CelesteError):
+        ctx.synchronize()

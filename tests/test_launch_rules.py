@@ -1,5 +1,6 @@
-"""Host-side index arithmetic of the pixel launches, compiled as it is: overlaps
-enumerated pixel by pixel against a mask."""
+"""Host-side rules and index arithmetic of the pixel launches, compiled as they
+are: overlaps enumerated pixel by pixel against a mask, and the
+shares of a background's item."""
 import ctypes
 import itertools
 import os
@@ -12,6 +13,7 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
                     "paper_1803_00113_gb300", "csrc")
 SOURCE = """
+#include "launch_rules.h"
 #include "overlap.h"
 using namespace celeste;
 extern "C" {
@@ -19,6 +21,7 @@ void overlap(int c0, int c1, int w, int nx, int ny, int nw, int nh, int* out) {
   const Overlap o = chunk_overlap(c0, c1, w, nx, ny, nw, nh);
   out[0] = o.x; out[1] = o.y; out[2] = o.w; out[3] = o.begin; out[4] = o.end;
 }
+int shares(long long px, int items, int sm) { return background_shares(px, items, sm); }
 }
 """
 
@@ -32,7 +35,9 @@ def rules(tmp_path_factory):
     (d / "rules.cpp").write_text(SOURCE)
     subprocess.run([cxx, "-std=c++17", "-O2", "-shared", "-fPIC", f"-I{CSRC}", str(d / "rules.cpp"),
                     "-o", str(d / "rules.so")], check=True)
-    return ctypes.CDLL(str(d / "rules.so"))
+    lib = ctypes.CDLL(str(d / "rules.so"))
+    lib.shares.argtypes = [ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
+    return lib
 
 
 @pytest.mark.parametrize("w,h", [(1, 7), (5, 4), (16, 16), (17, 9), (300, 3), (37, 20), (64, 5)])
@@ -54,3 +59,15 @@ def test_overlap_of_a_chunk(rules, w, h):
                     q = np.arange(b, max(b, e))
                     got = (oy + q // max(ow, 1)) * w + ox + q % max(ow, 1)
                     assert np.array_equal(got, c0 + np.flatnonzero(mask[c0:c1])), (c0, c1, nx, ny, nw, nh)
+
+
+def test_shares_are_a_pass_or_more(rules):
+    sm = 152
+    for items in (1, 37, 3040, 3041, 50000):
+        for mean in (1, 32, 64, 127, 128, 255, 256, 4096):
+            n = rules.shares(mean * items, items, sm)
+            assert n in (1, 2, 4) and (n == 1 or mean >= 64 * n)
+            assert n == 1 or items <= 20 * sm
+            if items <= 20 * sm and mean >= 256:
+                assert n == 4
+    assert rules.shares(0, 0, sm) == 1
