@@ -20,4 +20,27 @@ inline int background_shares(int64_t n_pixels, int n_items, int sm_count) {
   return mean >= 256 ? 4 : (mean >= 128 ? 2 : 1);
 }
 
+// A block of eight warps per item instead of a warp: where its blocks are
+// resident together (two per SM in the derivative pass, five in the value
+// pass), or nearly so with items of six passes of a warp and more (two
+// rounds; part of a class's sources have often stopped), and, in the
+// derivative pass, an item has more than one pass.  Beyond, the persistent
+// kernels fill the GPU and are faster.  One 41 x 41 source, a Newton
+// iteration: derivatives 26.5 -> 14.2 us, values 14.0 -> 8.7.  Calls on n
+// sources of one item, a warp against a block an item: derivatives of 304
+// items of 100 pixels 1.10, of 608 items of 25 pixels 0.83; values of 760
+// items of 64 pixels 1.00, of 912 0.93, of 810 items of 1,024 pixels 1.30;
+// 600 field sources, a class of 1,100 items: 249 us of derivatives in a pass
+// with eight items per SM, 236 with four.
+inline bool block_per_item_derivs(int64_t n_pixels, int n_items, int sm_count) {
+  if (n_items <= 0) return false;
+  const int64_t mean = n_pixels / n_items;
+  return mean > 32 && n_items <= (mean >= 192 ? 4 : 2) * sm_count;
+}
+inline bool block_per_item_values(int64_t n_pixels, int n_items, int sm_count) {
+  if (n_items <= 0) return false;
+  const int64_t mean = n_pixels / n_items;
+  return n_items <= (mean >= 192 ? 8 : 5) * sm_count;
+}
+
 }  // namespace celeste

@@ -1909,16 +1909,9 @@ cudaError_t launch_background(const Launch& L, const PlanView& v) {
   });
 }
 
-// A block per item up to four (derivatives) or eight (values) items per SM:
-// two and four rounds of resident blocks.  One 41 x 41 source, a Newton
-// iteration: derivatives 26.5 -> 14.2 us, values 14.0 -> 8.7.  Beyond, the
-// persistent kernels fill the GPU and are faster (600 field sources, a class
-// of 1,100 items: 249 us of derivatives in a pass with eight items per SM,
-// 236 with four).
-constexpr int kCoopDerivs = 4, kCoopValues = 8;
 cudaError_t launch_pixels_derivs(const Launch& L, const PlanView& v) {
   if (v.n_items == 0) return cudaSuccess;
-  if (v.n_items <= kCoopDerivs * L.sm_count) {
+  if (block_per_item_derivs(v.n_bg, v.n_items, L.sm_count)) {
     derivs_coop_kernel<<<v.n_items, kCoopThreads, 0, L.stream>>>(v, L.n_exp, L.n_dev);
     return cudaGetLastError();
   }
@@ -1945,7 +1938,7 @@ cudaError_t launch_pixels_grad(const Launch& L, const PlanView& v) {
 cudaError_t launch_pixels_value(const Launch& L, const PlanView& v, bool keep_render) {
   if (v.n_items == 0) return cudaSuccess;
   const int mode = !keep_render || !v.cache ? 0 : (v.cache_half ? 2 : 1);
-  if (v.n_items <= kCoopValues * L.sm_count) {
+  if (block_per_item_values(v.n_bg, v.n_items, L.sm_count)) {
     value_coop_kernel<<<v.n_items, kCoopThreads, 0, L.stream>>>(v, L.n_exp, L.n_dev, mode);
     return cudaGetLastError();
   }

@@ -1,6 +1,6 @@
 """Host-side rules and index arithmetic of the pixel launches, compiled as they
-are: overlaps enumerated pixel by pixel against a mask, and the
-shares of a background's item."""
+are: overlaps enumerated pixel by pixel against a mask, the shares of a
+background's item, and when a block takes an item."""
 import ctypes
 import itertools
 import os
@@ -22,6 +22,8 @@ void overlap(int c0, int c1, int w, int nx, int ny, int nw, int nh, int* out) {
   out[0] = o.x; out[1] = o.y; out[2] = o.w; out[3] = o.begin; out[4] = o.end;
 }
 int shares(long long px, int items, int sm) { return background_shares(px, items, sm); }
+int block_derivs(long long px, int items, int sm) { return block_per_item_derivs(px, items, sm); }
+int block_values(long long px, int items, int sm) { return block_per_item_values(px, items, sm); }
 }
 """
 
@@ -36,7 +38,8 @@ def rules(tmp_path_factory):
     subprocess.run([cxx, "-std=c++17", "-O2", "-shared", "-fPIC", f"-I{CSRC}", str(d / "rules.cpp"),
                     "-o", str(d / "rules.so")], check=True)
     lib = ctypes.CDLL(str(d / "rules.so"))
-    lib.shares.argtypes = [ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
+    for f in (lib.shares, lib.block_derivs, lib.block_values):
+        f.argtypes = [ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
     return lib
 
 
@@ -71,3 +74,14 @@ def test_shares_are_a_pass_or_more(rules):
             if items <= 20 * sm and mean >= 256:
                 assert n == 4
     assert rules.shares(0, 0, sm) == 1
+
+
+def test_short_items_take_a_block_only_where_they_are_resident(rules):
+    sm = 152
+    for items, mean, derivs, values in [(1, 1, 0, 1), (1, 32, 0, 1), (1, 33, 1, 1), (304, 64, 1, 1),
+                                        (305, 64, 0, 1), (608, 191, 0, 1), (608, 192, 1, 1),
+                                        (609, 256, 0, 1), (760, 25, 0, 1), (761, 25, 0, 0),
+                                        (761, 192, 0, 1), (1216, 1024, 0, 1), (1217, 1024, 0, 0)]:
+        assert rules.block_derivs(mean * items, items, sm) == derivs, (items, mean)
+        assert rules.block_values(mean * items, items, sm) == values, (items, mean)
+    assert not rules.block_derivs(0, 0, sm) and not rules.block_values(0, 0, sm)
