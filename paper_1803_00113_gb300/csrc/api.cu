@@ -123,6 +123,7 @@ cudaError_t derivs_launch(celeste_ctx* c, celeste_plan* p, const Launch& L) {
 // cached moments, so only the own pairs need records, and it joins their
 // launch.
 int run_start(celeste_ctx* c, celeste_plan* p, bool background) {
+  if (background) nbr_room(c, p);
   Launch L = make_launch(c, p);
   const PlanView& v = p->v;
   ++c->launches;
@@ -160,7 +161,11 @@ void* MemPool::get(bool host, size_t bytes) {
     }
   }
   void* ptr = nullptr;
-  const cudaError_t e = host ? cudaMallocHost(&ptr, bytes) : cudaMalloc(&ptr, bytes);
+  cudaError_t e = host ? cudaMallocHost(&ptr, bytes) : cudaMalloc(&ptr, bytes);
+  if (!host && e != cudaSuccess && trim()) {
+    cudaGetLastError();
+    e = cudaMalloc(&ptr, bytes);
+  }
   if (e != cudaSuccess) return nullptr;
   std::lock_guard<std::mutex> lk(mu_);
   size_[host][ptr] = bytes;
@@ -172,6 +177,18 @@ void MemPool::put(bool host, void* ptr) {
   std::lock_guard<std::mutex> lk(mu_);
   auto it = size_[host].find(ptr);
   if (it != size_[host].end()) free_[host].emplace(it->second, ptr);
+}
+
+bool MemPool::trim() {
+  std::lock_guard<std::mutex> lk(mu_);
+  auto& fr = free_[0];
+  const bool any = !fr.empty();
+  for (auto& kv : fr) {
+    size_[0].erase(kv.second);
+    cudaFree(kv.second);
+  }
+  fr.clear();
+  return any;
 }
 
 // Frees the cached blocks.  Blocks still held by plans or fits stay theirs:
@@ -197,6 +214,37 @@ uint64_t g_ctx_serial = 0;
 
 void* ctx_alloc(celeste_ctx* c, bool host, size_t bytes) {
   return c->pool.get(host, bytes);
+}
+
+cudaError_t device_malloc(celeste_ctx* c, void** ptr, size_t bytes) {
+  cudaError_t e = cudaMalloc(ptr, bytes);
+  if (e != cudaSuccess && c->pool.trim()) {
+    cudaGetLastError();
+    e = cudaMalloc(ptr, bytes);
+  }
+  return e;
+}
+
+void* nbr_alloc(celeste_ctx* c, int64_t area) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;   // (this thread's)
+  if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
+  const size_t bytes = (size_t)area * sizeof(float2);
+  size_t room = 0, total = 0;
+  void* ptr = nullptr;
+  if (cudaMemGetInfo(&room, &total) == cudaSuccess && bytes <= room / 4)
+    ptr = ctx_alloc(c, false, bytes);
+  if (!ptr) cudaGetLastError();
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return ptr;
+}
+
+void nbr_room(celeste_ctx* c, celeste_plan* p) {
+  if (p->nbr_area == 0) return;
+  if (void* ptr = nbr_alloc(c, p->nbr_area)) {
+    p->allocs.push_back(ptr);
+    p->v.nbr_render = static_cast<float2*>(ptr);
+  }
+  p->nbr_area = 0;
 }
 
 void ctx_release(celeste_ctx* c, uint64_t serial, bool host,
@@ -425,6 +473,13 @@ int celeste_profile_read(celeste_ctx* c, int reset, double* total_ms, int64_t* l
 
 int celeste_plan_create(celeste_ctx* c, const celeste_problem* pr, const int32_t* ids, int32_t n,
                         const celeste_tuning* tuning, celeste_plan** out) {
+  return plan_create(c, pr, ids, n, tuning, true, out);
+}
+
+}  // extern "C"
+
+int celeste::plan_create(celeste_ctx* c, const celeste_problem* pr, const int32_t* ids, int32_t n,
+                         const celeste_tuning* tuning, bool backgrounds, celeste_plan** out) {
   if (!c || !pr || !out || n < 0 || (n > 0 && !ids)) return CELESTE_EINVAL;
   *out = nullptr;
   if (!pr->h_patch_ptr || !pr->h_patches || !pr->h_images || !pr->h_nbr_ptr ||
@@ -551,7 +606,8 @@ int celeste_plan_create(celeste_ctx* c, const celeste_problem* pr, const int32_t
   // patch and gathered, rather than rendered over every overlap, where the
   // overlaps cover at least half of the neighbour pairs, or a quarter and some
   // own pair has six neighbours (a chunk's chain of neighbours is then cut
-  // short), and the moments take at most 1 GB.  An overlap is cut into chunks
+  // short), and the moments take at most 1 GB (allocated when the first
+  // background is formed).  An overlap is cut into chunks
   // of 256 own pixels with a record staged for each, so a pixel of it costs
   // about three times one of a whole patch: backgrounds at ratios of 2.8 (300
   // blended sources) 750 -> 276 us, 1.4 (a crowded field) 126 -> 66, 0.76
@@ -561,7 +617,7 @@ int celeste_plan_create(celeste_ctx* c, const celeste_problem* pr, const int32_t
   std::vector<Item> nbr_items;
   size_t max_nbr = 0;
   for (int pp = 0; pp < n_own; ++pp) max_nbr = std::max(max_nbr, per_pair[pp].size());
-  if (!pr->render_cache && nbr_area > 0 && nbr_area <= kMaxNbrRender &&
+  if (backgrounds && !pr->render_cache && nbr_area > 0 && nbr_area <= kMaxNbrRender &&
       (2 * overlap >= nbr_area || (4 * overlap >= nbr_area && max_nbr >= 6))) {
     std::vector<std::vector<int32_t>> users(pairs.size() - n_own);   // slots, ascending
     for (int pp = 0; pp < n_own; ++pp) {
@@ -631,10 +687,10 @@ int celeste_plan_create(celeste_ctx* c, const celeste_problem* pr, const int32_t
   if (!nbr_items.empty()) {
     int no_room = CELESTE_OK;   // (then every overlap is rendered)
     d_nbr_items = dev_alloc<Item>(p, nbr_items.size(), &no_room);
-    v.nbr_render = dev_alloc<float2>(p, (size_t)nbr_area, &no_room);
-    if (no_room != CELESTE_OK) {
+    if (no_room == CELESTE_OK) {
+      p->nbr_area = nbr_area;
+    } else {
       cudaGetLastError();
-      v.nbr_render = nullptr;
       nbr_items.clear();
     }
   }
@@ -667,6 +723,8 @@ int celeste_plan_create(celeste_ctx* c, const celeste_problem* pr, const int32_t
   *out = p;
   return CELESTE_OK;
 }
+
+extern "C" {
 
 int celeste_plan_destroy(celeste_plan* p) {
   if (!p) return CELESTE_EINVAL;
@@ -751,6 +809,7 @@ int celeste_newton_step(celeste_ctx* c, const celeste_plan* pc, double* delta, i
   Launch L = make_launch(c, p);
   PlanView& v = p->v;
   const bool cached = v.cache != nullptr;
+  if (!cached) nbr_room(c, p);
   // active set and records; with a render cache the background comes from
   // cached moments, so the own records are all it needs and it joins the
   // same launch

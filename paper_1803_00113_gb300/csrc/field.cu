@@ -63,7 +63,7 @@ int celeste_field_create(celeste_ctx* c, const celeste_problem* pr, const celest
     for (int s = 0; s < S; ++s)
       if (color[s] == col) cls.push_back(s);
     celeste_plan* p = nullptr;
-    rc = celeste_plan_create(c, pr, cls.data(), (int)cls.size(), tuning, &p);
+    rc = plan_create(c, pr, cls.data(), (int)cls.size(), tuning, false, &p);
     if (rc == CELESTE_OK) F->plans.push_back(p);
   }
   // partial sums: about eight blocks per SM over all images
@@ -71,7 +71,7 @@ int celeste_field_create(celeste_ctx* c, const celeste_problem* pr, const celest
   auto alloc = [&](size_t bytes) -> void* {
     void* ptr = nullptr;
     if (rc != CELESTE_OK) return nullptr;
-    if (cudaMalloc(&ptr, bytes ? bytes : 1) != cudaSuccess) {
+    if (device_malloc(c, &ptr, bytes ? bytes : 1) != cudaSuccess) {
       rc = CELESTE_ENOMEM;
       return nullptr;
     }

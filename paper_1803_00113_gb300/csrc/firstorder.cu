@@ -201,7 +201,7 @@ int celeste_lbfgs_create(celeste_ctx* c, const celeste_plan* pc, int32_t m, cele
   auto alloc = [&](size_t bytes) -> void* {
     void* ptr = nullptr;
     if (rc != CELESTE_OK) return nullptr;
-    if (cudaMalloc(&ptr, bytes) != cudaSuccess) {
+    if (device_malloc(c, &ptr, bytes) != cudaSuccess) {
       rc = CELESTE_ENOMEM;
       return nullptr;
     }
@@ -253,6 +253,7 @@ int celeste_lbfgs_step(celeste_ctx* c, celeste_lbfgs* B, int32_t* status, const 
   celeste_plan* p = B->plan;
   PlanView& v = p->v;
   if (v.n == 0) return CELESTE_OK;
+  nbr_room(c, p);
   const Launch L = make_launch(c, p);
   const int nb = (v.n + 127) / 128;
   // value and gradient where a step was accepted (or at the start)

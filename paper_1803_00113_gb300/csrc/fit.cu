@@ -194,6 +194,18 @@ int fit_create_segments(celeste_ctx* c, const celeste_problem* pr, const int32_t
     if (rcs[col] != CELESTE_OK && rc == CELESTE_OK) rc = rcs[col];
     if (plans[col]) F->plans.push_back(plans[col]);
   }
+  // the classes run one after another: one buffer holds each one's neighbour
+  // renders in its turn
+  int64_t nbr_area = 0;
+  for (celeste_plan* p : F->plans) nbr_area = std::max(nbr_area, p->nbr_area);
+  if (rc == CELESTE_OK && nbr_area > 0) {
+    void* ptr = nbr_alloc(c, nbr_area);
+    if (ptr) F->allocs.push_back(ptr);
+    for (celeste_plan* p : F->plans) {
+      if (p->nbr_area > 0) p->v.nbr_render = static_cast<float2*>(ptr);
+      p->nbr_area = 0;
+    }
+  }
   if (rc == CELESTE_OK && pr->render_cache) {
     // sources outside the region that border it: rendered into the cache
     // once per run, since backgrounds are gathered from there
@@ -208,7 +220,7 @@ int fit_create_segments(celeste_ctx* c, const celeste_problem* pr, const int32_t
         }
       }
     if (!outside.empty())
-      rc = celeste_plan_create(c, pr, outside.data(), (int)outside.size(), tuning, &F->outside);
+      rc = plan_create(c, pr, outside.data(), (int)outside.size(), tuning, false, &F->outside);
   }
   auto alloc = [&](size_t bytes) -> void* {
     if (rc != CELESTE_OK) return nullptr;

@@ -22,12 +22,14 @@ namespace celeste {
 // between passes) would otherwise pay a cudaMalloc/cudaFree pair per buffer,
 // and cudaFree waits for the device.  A freed block returns to its context
 // once the context's stream has finished with it, and a later request of at
-// least half its size takes it back.  Blocks go back to CUDA when the
-// context is destroyed.
+// least half its size takes it back.  Free blocks go back to CUDA when an
+// allocation fails that needs their room (device_malloc below included), and
+// when the context is destroyed.
 class MemPool {
  public:
   void* get(bool host, size_t bytes);
   void put(bool host, void* ptr);
+  bool trim();                       // frees the cached device blocks; false: none
   void release_all();
 
  private:
@@ -62,6 +64,8 @@ struct celeste_plan {
   const celeste_patch* d_patches = nullptr;
   double* rel_trial = nullptr;
   std::vector<void*> allocs;
+  int64_t nbr_area = 0;              // float2 that v.nbr_render would take; 0: not wanted
+                                     // (or there, or could not be had)
   int64_t visits = 0;
   celeste_tuning tuning{};
 };
@@ -93,10 +97,25 @@ namespace celeste {
 
 // Memory of a plan or fit: from its context's pool while the context lives.
 void* ctx_alloc(celeste_ctx* c, bool host, size_t bytes);
+// cudaMalloc for an object of the context (freed with cudaFree).
+cudaError_t device_malloc(celeste_ctx* c, void** ptr, size_t bytes);
 // Returns blocks taken with ctx_alloc: to the pool of the context with the
 // given serial if it still exists (after its stream has finished with
 // them), else to CUDA.
 void ctx_release(celeste_ctx* c, uint64_t serial, bool host, const std::vector<void*>& blocks);
+
+// celeste_plan_create; backgrounds: whether the plan will form any (without, it
+// prepares no neighbour renders).
+int plan_create(celeste_ctx* c, const celeste_problem* pr, const int32_t* ids, int32_t n,
+                const celeste_tuning* tuning, bool backgrounds, celeste_plan** out);
+// The scratch of a plan's neighbour renders (v.nbr_render, float2[nbr_area]), by
+// the first call that forms its backgrounds, so that plans made for other calls
+// do not hold it.  Optional: where it would take more than a quarter of the
+// device's free memory, the plan renders over the overlaps instead, then and
+// afterwards (the same values).  Callable while the stream is being captured.
+void nbr_room(celeste_ctx* c, celeste_plan* p);
+// The block itself (context pool), or null.
+void* nbr_alloc(celeste_ctx* c, int64_t area);
 
 // Launch configuration of a plan's kernels on the context's stream.
 Launch make_launch(const celeste_ctx* c, const celeste_plan* p);
