@@ -22,10 +22,11 @@ inline int background_shares(int64_t n_pixels, int n_items, int sm_count) {
 
 // A block of eight warps per item instead of a warp: where its blocks are
 // resident together (two per SM in the derivative pass, five in the value
-// pass), or nearly so with items of six passes of a warp and more (two
-// rounds; part of a class's sources have often stopped), and, in the
-// derivative pass, an item has more than one pass.  Beyond, the persistent
-// kernels fill the GPU and are faster.  One 41 x 41 source, a Newton
+// pass), and, in the derivative pass, an item has more than one pass; longer
+// items also in two rounds (from three passes in derivatives, six in values),
+// since part of a class's sources have often stopped: fits of 56 sources lose
+// up to 1 % without.  Beyond, the persistent kernels fill the GPU and are
+// faster.  One 41 x 41 source, a Newton
 // iteration: derivatives 26.5 -> 14.2 us, values 14.0 -> 8.7.  Calls on n
 // sources of one item, a warp against a block an item: derivatives of 304
 // items of 100 pixels 1.10, of 608 items of 25 pixels 0.83; values of 760
@@ -35,7 +36,7 @@ inline int background_shares(int64_t n_pixels, int n_items, int sm_count) {
 inline bool block_per_item_derivs(int64_t n_pixels, int n_items, int sm_count) {
   if (n_items <= 0) return false;
   const int64_t mean = n_pixels / n_items;
-  return mean > 32 && n_items <= (mean >= 192 ? 4 : 2) * sm_count;
+  return mean > 32 && n_items <= (mean >= 96 ? 4 : 2) * sm_count;
 }
 inline bool block_per_item_values(int64_t n_pixels, int n_items, int sm_count) {
   if (n_items <= 0) return false;

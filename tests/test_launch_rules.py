@@ -79,8 +79,8 @@ def test_shares_are_a_pass_or_more(rules):
 def test_short_items_take_a_block_only_where_they_are_resident(rules):
     sm = 152
     for items, mean, derivs, values in [(1, 1, 0, 1), (1, 32, 0, 1), (1, 33, 1, 1), (304, 64, 1, 1),
-                                        (305, 64, 0, 1), (608, 191, 0, 1), (608, 192, 1, 1),
-                                        (609, 256, 0, 1), (760, 25, 0, 1), (761, 25, 0, 0),
+                                        (305, 95, 0, 1), (608, 96, 1, 1), (609, 256, 0, 1),
+                                        (761, 191, 0, 0), (760, 25, 0, 1), (761, 25, 0, 0),
                                         (761, 192, 0, 1), (1216, 1024, 0, 1), (1217, 1024, 0, 0)]:
         assert rules.block_derivs(mean * items, items, sm) == derivs, (items, mean)
         assert rules.block_values(mean * items, items, sm) == values, (items, mean)
