@@ -604,21 +604,19 @@ int celeste::plan_create(celeste_ctx* c, const celeste_problem* pr, const int32_
 
   // Without a render cache each neighbour pair is rendered once over its
   // patch and gathered, rather than rendered over every overlap, where the
-  // overlaps cover at least half of the neighbour pairs, or a quarter and some
-  // own pair has six neighbours (a chunk's chain of neighbours is then cut
-  // short), and the moments take at most 1 GB (allocated when the first
-  // background is formed).  An overlap is cut into chunks
-  // of 256 own pixels with a record staged for each, so a pixel of it costs
-  // about three times one of a whole patch: backgrounds at ratios of 2.8 (300
-  // blended sources) 750 -> 276 us, 1.4 (a crowded field) 126 -> 66, 0.76
-  // 86 -> 61, 0.32 91 -> 92; three sources at 0.26: 16 -> 19, the second launch.
-  // Eleven classes of 100 blended sources, up to ten neighbours: 546 -> 402 with
-  // the second part of the rule.
+  // overlaps cover at least half of the neighbour pairs and the moments take
+  // at most 1 GB (allocated when the first background is formed).  An overlap
+  // is cut into chunks of 256 own pixels with a record staged for each, so a
+  // pixel of it costs about twice one of a whole patch, and the gather is a
+  // launch more.  Backgrounds over overlaps against once, at ratios of 2.8
+  // (300 blended sources) 638 against 279 us, 1.8 and 1.35 (crowded fields)
+  // 166 / 84 and 123 / 66, 0.76 85 / 60, 0.35 to 0.55 (eleven classes of 333
+  // blended sources) 765 / 873, of 100 433 / 398, 0.31 (600 field sources)
+  // 72 / 88.  Launches of a few hundred items lose the extra launch up to a
+  // ratio of one (100 patches of 41 x 41 at 0.74: 14 / 21).
   std::vector<Item> nbr_items;
-  size_t max_nbr = 0;
-  for (int pp = 0; pp < n_own; ++pp) max_nbr = std::max(max_nbr, per_pair[pp].size());
   if (backgrounds && !pr->render_cache && nbr_area > 0 && nbr_area <= kMaxNbrRender &&
-      (2 * overlap >= nbr_area || (4 * overlap >= nbr_area && max_nbr >= 6))) {
+      2 * overlap >= nbr_area) {
     std::vector<std::vector<int32_t>> users(pairs.size() - n_own);   // slots, ascending
     for (int pp = 0; pp < n_own; ++pp) {
       for (const int32_t q : per_pair[pp]) {
