@@ -63,10 +63,9 @@ struct TrSmem {
   double lam, lo, hi;              // multiplier and its bracket (unscaled)
   double lmin_lo;                  // lower bound of lambda_min (unscaled, FP32 accuracy)
   double lam_b;                    // boundary start when an interior try fails (0: none)
-  int positive;                    // FP32 finds B positive definite
   int tried0;                      // l = 0 has been evaluated
   int bisects;                     // bisection steps of the FP64 iteration
-  float betaf[32], dfr[32], efr[32], gfr[32];
+  float dfr[32], efr[32], gfr[32];
   float loc[4];                    // locate32: scale, |g|^2 (scaled), |p(0)|^2
   unsigned hmask[2][4];            // locate32: probe ballots of the four warps
   int mode;                        // 0 interior candidate, 1 boundary, 2 full FP64 path
@@ -1022,7 +1021,6 @@ static __device__ void locate32(TrSmem& S, double Delta, int tid) {
     S.mode = mode;
     const double sc = (double)scale;
     S.lmin_lo = (double)scale * (double)fa;
-    S.positive = lmin > 0.f ? 1 : 0;
     // the FP32 root estimate starts the FP64 iteration (0: no estimate)
     S.lam = bracket ? sc * 0.5 * ((double)la + (double)lb) : 0.0;
     S.lam_b = S.lam;
