@@ -225,10 +225,10 @@ int celeste_profile_kernels(celeste_ctx* ctx, int reset, double* ms, int64_t* la
  * should not overlap (one colour class of the overlap graph, Sec. 4.4).
  * tuning may be NULL.  The plan keeps pointers into *problem's arrays, not
  * the struct itself; it stays valid while those arrays do.  Of a crowded
- * problem without a render cache, the first call that forms the plan's
- * backgrounds may take up to 1 GB more for its neighbours' renders, never
- * more than a quarter of the device's free memory (without, the same values
- * are formed more slowly). */
+ * problem without a render cache, a plan takes up to 1 GB more for its
+ * neighbours' renders, never more than a quarter of the device's free memory
+ * (without, the same values are formed more slowly): what exceeds a 1,024th
+ * of the device's memory with the first call that forms its backgrounds. */
 int celeste_plan_create(celeste_ctx* ctx, const celeste_problem* problem,
                         const int32_t* h_src_ids, int32_t n, const celeste_tuning* tuning,
                         celeste_plan** out);

@@ -473,13 +473,13 @@ int celeste_profile_read(celeste_ctx* c, int reset, double* total_ms, int64_t* l
 
 int celeste_plan_create(celeste_ctx* c, const celeste_problem* pr, const int32_t* ids, int32_t n,
                         const celeste_tuning* tuning, celeste_plan** out) {
-  return plan_create(c, pr, ids, n, tuning, true, out);
+  return plan_create(c, pr, ids, n, tuning, NbrScratch::kPlan, out);
 }
 
 }  // extern "C"
 
 int celeste::plan_create(celeste_ctx* c, const celeste_problem* pr, const int32_t* ids, int32_t n,
-                         const celeste_tuning* tuning, bool backgrounds, celeste_plan** out) {
+                         const celeste_tuning* tuning, NbrScratch nbr, celeste_plan** out) {
   if (!c || !pr || !out || n < 0 || (n > 0 && !ids)) return CELESTE_EINVAL;
   *out = nullptr;
   if (!pr->h_patch_ptr || !pr->h_patches || !pr->h_images || !pr->h_nbr_ptr ||
@@ -605,7 +605,7 @@ int celeste::plan_create(celeste_ctx* c, const celeste_problem* pr, const int32_
   // Without a render cache each neighbour pair is rendered once over its
   // patch and gathered, rather than rendered over every overlap, where the
   // overlaps cover at least half of the neighbour pairs and the moments take
-  // at most 1 GB (allocated when the first background is formed).  An overlap
+  // at most 1 GB.  An overlap
   // is cut into chunks of 256 own pixels with a record staged for each, so a
   // pixel of it costs about twice one of a whole patch, and the gather is a
   // launch more.  Backgrounds over overlaps against once, at ratios of 2.8
@@ -615,7 +615,7 @@ int celeste::plan_create(celeste_ctx* c, const celeste_problem* pr, const int32_
   // 72 / 88.  Launches of a few hundred items lose the extra launch up to a
   // ratio of one (100 patches of 41 x 41 at 0.74: 14 / 21).
   std::vector<Item> nbr_items;
-  if (backgrounds && !pr->render_cache && nbr_area > 0 && nbr_area <= kMaxNbrRender &&
+  if (nbr != NbrScratch::kNone && !pr->render_cache && nbr_area > 0 && nbr_area <= kMaxNbrRender &&
       2 * overlap >= nbr_area) {
     std::vector<std::vector<int32_t>> users(pairs.size() - n_own);   // slots, ascending
     for (int pp = 0; pp < n_own; ++pp) {
@@ -718,6 +718,10 @@ int celeste::plan_create(celeste_ctx* c, const celeste_problem* pr, const int32_
   v.slot_items = d_slot_items;
   v.items = d_items;
   v.nbr_items = d_nbr_items;
+  size_t room = 0, total = 0;
+  if (nbr == NbrScratch::kPlan && p->nbr_area > 0 && cudaMemGetInfo(&room, &total) == cudaSuccess &&
+      (size_t)p->nbr_area * sizeof(float2) <= total / 1024)
+    nbr_room(c, p);
   *out = p;
   return CELESTE_OK;
 }

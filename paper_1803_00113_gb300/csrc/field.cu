@@ -63,7 +63,7 @@ int celeste_field_create(celeste_ctx* c, const celeste_problem* pr, const celest
     for (int s = 0; s < S; ++s)
       if (color[s] == col) cls.push_back(s);
     celeste_plan* p = nullptr;
-    rc = plan_create(c, pr, cls.data(), (int)cls.size(), tuning, false, &p);
+    rc = plan_create(c, pr, cls.data(), (int)cls.size(), tuning, NbrScratch::kNone, &p);
     if (rc == CELESTE_OK) F->plans.push_back(p);
   }
   // partial sums: about eight blocks per SM over all images

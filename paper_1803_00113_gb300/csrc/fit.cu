@@ -174,8 +174,8 @@ int fit_create_segments(celeste_ctx* c, const celeste_problem* pr, const int32_t
   cudaGetDevice(&device);
   auto plan_class = [&](int col) {
     cudaSetDevice(device);
-    rcs[col] = celeste_plan_create(c, pr, cls[col].data(), (int)cls[col].size(), tuning,
-                                   &plans[col]);
+    rcs[col] = plan_create(c, pr, cls[col].data(), (int)cls[col].size(), tuning,
+                           NbrScratch::kCaller, &plans[col]);
   };
   const int n_threads =
       std::min<int>(n_colors, std::max(1u, std::min(16u, std::thread::hardware_concurrency())));
@@ -220,7 +220,7 @@ int fit_create_segments(celeste_ctx* c, const celeste_problem* pr, const int32_t
         }
       }
     if (!outside.empty())
-      rc = plan_create(c, pr, outside.data(), (int)outside.size(), tuning, false, &F->outside);
+      rc = plan_create(c, pr, outside.data(), (int)outside.size(), tuning, NbrScratch::kNone, &F->outside);
   }
   auto alloc = [&](size_t bytes) -> void* {
     if (rc != CELESTE_OK) return nullptr;

@@ -104,15 +104,19 @@ cudaError_t device_malloc(celeste_ctx* c, void** ptr, size_t bytes);
 // them), else to CUDA.
 void ctx_release(celeste_ctx* c, uint64_t serial, bool host, const std::vector<void*>& blocks);
 
-// celeste_plan_create; backgrounds: whether the plan will form any (without, it
-// prepares no neighbour renders).
+// celeste_plan_create, and what becomes of the scratch of its neighbour renders
+// (v.nbr_render, float2[nbr_area]): none for a plan that forms no backgrounds;
+// left to the caller; or by itself, when the plan is made up to a 1,024th of
+// the device's memory and otherwise when it first forms backgrounds, so that a
+// plan made for other calls does not hold it.
+enum class NbrScratch { kNone, kCaller, kPlan };
 int plan_create(celeste_ctx* c, const celeste_problem* pr, const int32_t* ids, int32_t n,
-                const celeste_tuning* tuning, bool backgrounds, celeste_plan** out);
-// The scratch of a plan's neighbour renders (v.nbr_render, float2[nbr_area]), by
-// the first call that forms its backgrounds, so that plans made for other calls
-// do not hold it.  Optional: where it would take more than a quarter of the
-// device's free memory, the plan renders over the overlaps instead, then and
-// afterwards (the same values).  Callable while the stream is being captured.
+                const celeste_tuning* tuning, NbrScratch nbr, celeste_plan** out);
+// Before a call that forms the plan's backgrounds: that scratch, if it is still
+// to come (an allocation, 50-120 us).  Optional: where it would take more than
+// a quarter of the device's free memory, the plan renders over the overlaps
+// instead, then and afterwards (the same values).  Callable while the stream is
+// being captured.
 void nbr_room(celeste_ctx* c, celeste_plan* p);
 // The block itself (context pool), or null.
 void* nbr_alloc(celeste_ctx* c, int64_t area);

@@ -1,7 +1,8 @@
 """The buffer of a plan's neighbour renders (8 bytes a pixel of every neighbour
 patch) is there only where backgrounds are formed: not in a whole-field ELBO's
-plans, not before a plan's first background, and once for all classes of a
-fit.  Taken while a stream is being captured it gives the same values."""
+plans, beyond a 1,024th of the device's memory not before a plan's first
+background, and once for all classes of a fit.  Taken while a stream is being
+captured it gives the same values."""
 import numpy as np
 import pytest
 import torch
@@ -50,23 +51,44 @@ def test_field_elbo_takes_none(crowded):
     assert taken < PLANS + BUFFER
 
 
-def test_plan_takes_it_with_its_first_background(crowded):
-    cel, dp = crowded
+@pytest.fixture(scope="module")
+def large(crowded):
+    """Nine neighbours of 2,100 x 2,100 pixels: 318 MB."""
+    cel, _ = crowded
+    total = torch.cuda.mem_get_info()[1]
+    side = 2100
+    while 8 * 9 * side * side <= total // 1024:
+        side += 100
+    return cel, cel.DeviceProblem(_scene(10, side, 0)), 8 * 9 * side * side
+
+
+def test_plan_takes_much_of_it_with_its_first_background(large):
+    cel, dp, buffer = large
     ctx = cel.Context(dp.host.model)
     E = torch.zeros(2, dp.n_pool, dtype=torch.float32, device=ctx.device)
 
-    def render():
-        plan = cel.Plan(ctx, dp, [0])
-        cel._check(cel.lib().celeste_render(ctx.handle, plan.handle, cel._ptr(E[0]), cel._ptr(E[1])), "r")
+    def call(f, plan):
+        cel._check(f(ctx.handle, plan.handle, cel._ptr(E[0]), cel._ptr(E[1])), "call")
         return plan
 
-    taken, plan = _taken(render)
+    # the plan's own: 8 bytes a pixel of one patch, a ninth
+    taken, plan = _taken(lambda: call(cel.lib().celeste_render, cel.Plan(ctx, dp, [0])))
+    assert taken < buffer // 2
+    taken, _ = _taken(lambda: call(cel.lib().celeste_background, plan))
+    assert buffer // 2 < taken < 2 * buffer
+    assert _taken(lambda: call(cel.lib().celeste_background, plan))[0] == 0
+    ctx.synchronize()
+
+
+def test_plan_takes_little_of_it_at_once(crowded):
+    cel, dp = crowded
+    ctx = cel.Context(dp.host.model)
+    taken, plan = _taken(lambda: cel.Plan(ctx, dp, [0]))
+    assert taken >= BUFFER // 2
+    E = torch.zeros(2, dp.n_pool, dtype=torch.float32, device=ctx.device)
+    taken, _ = _taken(lambda: cel._check(cel.lib().celeste_background(
+        ctx.handle, plan.handle, cel._ptr(E[0]), cel._ptr(E[1])), "b"))
     assert taken < BUFFER // 2
-    bg = lambda: cel._check(cel.lib().celeste_background(ctx.handle, plan.handle, cel._ptr(E[0]),
-                                                         cel._ptr(E[1])), "b")
-    taken, _ = _taken(bg)
-    assert BUFFER // 2 < taken < 2 * BUFFER
-    assert _taken(bg)[0] == 0
     ctx.synchronize()
 
 
@@ -78,8 +100,8 @@ def test_classes_of_a_fit_share_one(crowded):
     assert BUFFER // 2 < taken < PLANS + 2 * BUFFER
 
 
-def test_first_background_under_capture(crowded):
-    cel, dp = crowded
+def test_first_background_under_capture(large):
+    cel, dp, _ = large
     ref = [t.cpu().numpy() for t in cel.background(cel.Plan(cel.Context(dp.host.model), dp, [3, 4]))]
     side = torch.cuda.Stream()
     ctx = cel.Context(dp.host.model, stream=side)
