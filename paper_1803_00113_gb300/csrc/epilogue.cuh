@@ -90,10 +90,8 @@ __host__ __device__ constexpr int tile_piece(int e) {
 }
 static_assert(kAcc % 4 == 0 && kGradAcc % 4 == 0, "whole pieces");
 
-// What a value alone needs of a block's shared memory: 2 KB with the model's
-// constants, which a log-likelihood does without.  (With the derivative
-// passes' buffers, 40 KB, five blocks fit on an SM; 600 sources, a
-// log-likelihood with the constants staged 29.4 us, without 27.5.)
+// What a value alone needs of a block's shared memory: half a KB.  (With the
+// derivative passes' buffers, 45 KB, five blocks fit on an SM.)
 struct KlSmem {
   real th[kNuPad];                 // theta of the source (FP32 copy)
   real kw[kNuPad];                 // colour weights; then grad_nu[a] * kappa_a
@@ -461,7 +459,7 @@ static __device__ __forceinline__ void stage_model(ModelDev::F32& dst, const Mod
 }
 
 // Slot j of the plan, by the whole block (tid 0..127; S.th holds theta and
-// f the model's FP32 constants, both in shared memory).  kMode: 0 value,
+// f the model's FP32 constants, in shared memory for kMode >= 1).  kMode: 0 value,
 // 1 value + gradient, 2 value + gradient + Hessian.  Warp 0 evaluates the KL
 // terms; warps 1 and 2 add up the tile sums, a pair each at a time, while
 // warp 3 forms the Jacobian and the images' maps; then the maps are applied

@@ -1,7 +1,7 @@
 """The value epilogue adds an item a thread: three pairs or more of up to 96 items
 each are loaded eight pairs together, fewer or longer ones a pair at a time.
-Either side of those lines, against the oracle; and a block of it holds a few
-kilobytes of shared memory, not the derivative passes' buffers."""
+Either side of those lines, against the oracle; and a block of it holds less than a
+kilobyte of shared memory, not the derivative passes' buffers."""
 import os
 import subprocess
 
@@ -73,8 +73,7 @@ def test_block_of_the_value_epilogue_is_small(tmp_path):
         pytest.skip("no nvcc")
     src = tmp_path / "size.cu"
     src.write_text('#include "epilogue.cuh"\nusing namespace celeste;\n'
-                   'static_assert(sizeof(EpiShared<0>) <= 1024 && '
-                   'sizeof(EpiShared<0>) + sizeof(ModelDev::F32) <= 4096, "");\n')
+                   'static_assert(sizeof(EpiShared<0>) <= 1024, "");\n')
     r = subprocess.run([nvcc, *build_lib.ARCH, "-std=c++17", f"-I{build_lib.INCLUDE}",
                         f"-I{build_lib.CSRC}", "-c", str(src), "-o", str(tmp_path / "size.o")],
                        capture_output=True, text=True)
