@@ -32,7 +32,7 @@
 // without branches (a divergent 18-way choice of map entries alone took 4k
 // cycles a pair), and every small dense product is spread over all threads.
 // One source with one 41 x 41 patch per band: 25k cycles (53k before) for
-// value, gradient and Hessian; with two 61 x 61 patches per band: 31k (84k).
+// value, gradient and Hessian; with two 61 x 61 patches per band: 28k (84k).
 #pragma once
 
 #include <math.h>

@@ -589,7 +589,7 @@ static __device__ __forceinline__ void ldl_entries(short2 (&rc)[kLdlRounds], int
 // reciprocal each, ~5 FP64 instructions of ~65 cycles): warp 0 does nothing
 // else, one column ahead, while warps 1..3 spread the trailing triangle
 // evenly over their threads, with the column and its multiples (each
-// formed once, by the lane of its row) passed by shuffles.  17.5k cycles, 34.8k
+// formed once, by the lane of its row) passed by shuffles.  17.1k cycles, 34.8k
 // with one entry's product and FMA after the other and FP64 comparisons of
 // the pivot.  Returns false
 // (the same on every thread) when a pivot is not positive.  On success
